@@ -52,6 +52,13 @@ struct dsm_lattice {
   int step_form;   // DSM_STEP_AUTO or DSM_STEP_TWO_PASS
   int zrun;        // planes per block of the single-pass step (0: automatic)
   int zrun_auto;
+  // step on moments (dsm_mom.cuh): mok, the parameters allow it; mom, the
+  // current state is held as moments (buffer mc); mcp, Cb[0] holds the C of its
+  // next step; mstat, the frozen solid's data is made; mfit, the canonical
+  // state is the result of a step with every relaxation time 1, so moments
+  // represent it; mstepped, mom and stepped since set_fluid
+  bool mok, mom, mcp, mstat, mfit, mstepped;
+  int mc, mzrun;
   // observables ring (dsm_set_observables_ring): caller-owned device records,
   // one appended by dsm_step after each step that is a multiple of ring_every
   double *ring = nullptr;
@@ -282,6 +289,163 @@ cudaError_t z_unpack(dsm_lattice *h) {
   return cudaSuccess;
 }
 
+// ---- step on moments ----------------------------------------------------------
+// It applies to FP32 and FP64 lattices with every relaxation time 1, equal
+// densities and periodic faces, whatever their size, in the automatic storage
+// form of g; dsm_set_step_form chooses one pass or two.
+bool m_eligible(const dsm_params *p) {
+  return (p->precision == DSM_F32 || p->precision == DSM_F64) && p->tau2 == 1.0 &&
+         p->tau3 == 1.0 && p->tau_g == 1.0 && p->rho2 == p->rho3 && !has_walls(p);
+}
+bool m_active(const dsm_lattice *h) {
+  return h->mok && h->eq;
+}
+
+// The moments use buffers the g_eq form leaves idle: buffer b in g[b]; the
+// solid's pairs and link bits behind them, its link fractions in f[0].  The
+// canonical copy of a state held as moments goes to buffer 1.
+MomRaw m_raw(const dsm_lattice *h, int src) {
+  MomRaw r;
+  memset(&r, 0, sizeof(r));
+  r.nx = h->prm.nx;
+  r.ny = h->prm.ny;
+  r.nz = h->prm.nz;
+  r.N = h->N;
+  r.pitch = h->pitch;
+  const size_t plane = (size_t)h->pitch * h->tab.real_bytes;
+  const int nm = mom_reals(h->kind);
+  for (int o = 0; o < 2; o++) {
+    char *b = (char *)h->g[o ? src ^ 1 : src];
+    void **d = o ? r.out : r.in;
+    d[0] = b;
+    d[1] = b + 4 * plane;
+    d[2] = b + (nm - 1) * plane;
+  }
+  r.sol = (char *)h->g[0] + nm * plane;
+  r.lk = (char *)h->g[1] + nm * plane;
+  r.qpl = h->f[0];
+  r.near = h->mask;
+  r.count = (int *)(h->obs + 6);
+  if (h->kind == DSM_D3Q19) {
+    r.list = (char *)r.lk + plane;
+    r.wall = (char *)r.sol + 2 * plane;
+  }
+  r.c1 = h->C1;
+  r.err = h->err;
+  r.k[0] = h->sp.kappa2;
+  r.ak[0] = h->sp.a2 * h->sp.kappa2;
+  r.kl = h->sp.kappa3;
+  r.akl = h->sp.a2 * h->sp.kappa3;
+  r.rho = h->sp.rho3;
+  for (int a = 0; a < 3; a++) r.body[a] = h->sp.body[a];
+  r.alpha_s = h->sp.alpha_s;
+  return r;
+}
+
+// canonical planes of buffer b
+MomPlanes m_planes(const dsm_lattice *h, int b) {
+  const size_t plane = (size_t)h->pitch * h->tab.real_bytes;
+  return {h->f[b], h->M, (char *)h->M + plane, h->Cb[b]};
+}
+
+cudaError_t m_statics(dsm_lattice *h) {
+  if (h->mstat) return cudaSuccess;
+  const cudaError_t e = h->tab.mom_solid(m_raw(h, 0), h->stream);
+  if (e == cudaSuccess) h->mstat = true;
+  return e;
+}
+
+// A state held as moments -> canonical form (buffer 1, g as g_eq).
+cudaError_t m_leave(dsm_lattice *h) {
+  if (!h->mom) return cudaSuccess;
+  const cudaError_t e = h->tab.mom_expand(m_raw(h, h->mc), m_planes(h, 1), 1, h->stream);
+  if (e != cudaSuccess) return e;
+  h->cur = 1;
+  h->g_implicit = true;
+  h->mom = h->mcp = h->mstat = false;
+  h->mfit = true;
+  return cudaSuccess;
+}
+
+// A new state arrives by other means.
+void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mstat = h->mfit = false; }
+
+// C of the next step of a state held as moments, into Cb[0].
+cudaError_t m_c(dsm_lattice *h) {
+  if (h->mcp) return cudaSuccess;
+  const cudaError_t e = h->tab.mom_c(m_raw(h, h->mc), h->Cb[0], h->stream);
+  if (e == cudaSuccess) h->mcp = true;
+  return e;
+}
+
+// Canonical state (mfit) -> moments, buffer 0.
+cudaError_t m_enter(dsm_lattice *h) {
+  MomRaw r = m_raw(h, 1);  // out = buffer 0
+  cudaError_t e = h->tab.mom_enter(r, m_planes(h, h->cur), h->stream);
+  if (e == cudaSuccess) e = m_statics(h);
+  if (e != cudaSuccess) return e;
+  h->mc = 0;
+  h->mom = true;
+  h->mstepped = true;
+  h->mcp = false;
+  return cudaSuccess;
+}
+
+// Planes per block of the 3D step: runs of zr planes give tiles * ceil(nz / zr)
+// blocks in waves of the resident ones; a run costs about three planes more
+// than it advances (two of halo on each side, partly summed, and the first
+// copies).  101^3: 36.7 us with the 9 planes this gives, 42.4 / 37.5 / 43.2
+// with 6 / 13 / 17; 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96.
+int m_zrun(dsm_lattice *h) {
+  if (h->zrun > 0) return h->zrun;
+  if (h->mzrun) return h->mzrun;
+  h->mzrun = 1;
+  if (h->kind != DSM_D3Q19) return 1;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int per_sm = h->tab.mom_resident(), nz = h->prm.nz;
+  const long long resident = (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
+  const long long tiles = (long long)z_tiles_x(h->prm.nx) * z_tiles_y(h->prm.ny);
+  double best = 1e300;
+  for (int zr = 1; zr <= nz; zr++) {
+    const long long blocks = tiles * ((nz + zr - 1) / zr);
+    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0);
+    if (cost < best - 1e-9) {
+      best = cost;
+      h->mzrun = zr;
+    }
+  }
+  return h->mzrun;
+}
+
+// The second pass of a step of a state held as moments (C in Cb[0]).
+cudaError_t m_collide(dsm_lattice *h) {
+  cudaError_t e = m_statics(h);
+  if (e == cudaSuccess)
+    e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_STEP, 0, nullptr, nullptr, h->stream);
+  if (e != cudaSuccess) return e;
+  h->mc ^= 1;
+  h->mcp = false;
+  h->mstepped = true;
+  return cudaSuccess;
+}
+
+// One step of a state held as moments, in one pass or two.
+cudaError_t m_step(dsm_lattice *h) {
+  cudaError_t e = m_statics(h);
+  if (h->step_form == DSM_STEP_TWO_PASS) {
+    if (e == cudaSuccess) e = m_c(h);
+    return e == cudaSuccess ? m_collide(h) : e;
+  }
+  if (e == cudaSuccess) e = h->tab.mom_step(m_raw(h, h->mc), m_zrun(h), h->stream);
+  if (e != cudaSuccess) return e;
+  h->mc ^= 1;
+  h->mcp = false;
+  h->mstepped = true;
+  return cudaSuccess;
+}
+
 // Read and clear nothing: report the latched device error word.
 dsm_status read_err(dsm_lattice *h, int *word) {
   int w = 0;
@@ -327,7 +491,17 @@ namespace {
 // without synchronising: the moments and observables passes over the
 // canonical state, then the deterministic final reduction.
 cudaError_t obs_launch(dsm_lattice *h) {
-  cudaError_t e = z_unpack(h);
+  cudaError_t e;
+  if (h->mom) {
+    e = m_statics(h);
+    if (e == cudaSuccess) e = m_c(h);
+    if (e == cudaSuccess)
+      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_OBS, 0, nullptr, h->partials, h->stream);
+    if (e != cudaSuccess) return e;
+    obs_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, h->obs_blocks, h->obs);
+    return cudaGetLastError();
+  }
+  e = z_unpack(h);
   if (e != cudaSuccess) return e;
   LBRaw a = raw_of(h, h->cur);
   e = h->tab.moments(a, h->stream);
@@ -465,6 +639,7 @@ dsm_status dsm_create(const dsm_params *p, void *d_workspace, size_t bytes, void
   h->sp = step_params(p, h->kappa);
   h->g_form = DSM_G_AUTO;
   h->eq = p->tau_g == 1.0 && !has_walls(p);
+  h->mok = m_eligible(p) && t.mom_step;
   // no solid yet: C1 = 0 everywhere; clear the error word and the mask
   cudaError_t e = cudaMemsetAsync(h->C1, 0, pitch * t.real_bytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->mask, 0, pitch, h->stream);
@@ -488,6 +663,7 @@ dsm_status dsm_set_solid(dsm_lattice *h, const void *d_field, int kind) {
   h->has_solid = true;
   h->has_fluid = false;
   h->zpacked = false;
+  m_drop(h);
   return DSM_OK;
 }
 
@@ -505,6 +681,7 @@ dsm_status dsm_relax_solid(dsm_lattice *h, const unsigned char *d_mask, int step
   h->g_implicit = false;
   h->has_fluid = false;
   h->zpacked = false;
+  m_drop(h);
   LBRaw r = raw_of(h, 1);  // out = buffer 0
   r.eq = 0;
   if ((e = h->tab.init(r, h->C1, 1, h->stream)) != cudaSuccess) return DSM_E_CUDA;
@@ -544,8 +721,19 @@ dsm_status dsm_solid_region(dsm_lattice *h, unsigned char *d_mask) {
 dsm_status dsm_set_fluid(dsm_lattice *h, const void *d_c2) {
   if (!h || !d_c2) return DSM_E_INVAL;
   h->cur = 0;
-  LBRaw r = raw_of(h, 1);  // writes buffer 0
-  cudaError_t e = h->tab.init(r, d_c2, 2, h->stream);
+  cudaError_t e;
+  if (m_active(h)) {  // the rest state as moments
+    if (!h->mom) h->mstat = false;  // (its buffers held another form)
+    e = m_statics(h);
+    if (e == cudaSuccess) e = h->tab.mom_init(m_raw(h, 1), d_c2, h->stream);  // writes buffer 0
+    h->mc = 0;
+    h->mom = true;
+    h->mcp = h->mfit = h->mstepped = false;
+  } else {
+    m_drop(h);
+    LBRaw r = raw_of(h, 1);  // writes buffer 0
+    e = h->tab.init(r, d_c2, 2, h->stream);
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, h->stream);
   if (e != cudaSuccess) return DSM_E_CUDA;
   h->step = 0;
@@ -561,11 +749,16 @@ dsm_status dsm_step(dsm_lattice *h, long long nsteps) {
   TraceRange trace_range("dsm_step");
   if (!h || nsteps < 0) return DSM_E_INVAL;
   if (!h->has_fluid || h->latched) return DSM_E_STATE;
-  const bool single = z_active(h);
+  const bool mom = m_active(h), single = !mom && z_active(h);
   if (!single && z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  if (!mom && m_leave(h) != cudaSuccess) return DSM_E_CUDA;
   for (long long t = 0; t < nsteps; t++) {
     cudaError_t e;
-    if (single && h->g_implicit) {
+    if (mom && (h->mom || (h->mfit && h->g_implicit))) {
+      if (!h->mom && m_enter(h) != cudaSuccess) return DSM_E_CUDA;
+      e = m_step(h);
+      if (e != cudaSuccess) return DSM_E_CUDA;
+    } else if (single && h->g_implicit) {
       // one pass per step over the padded g_eq state
       if (!h->zpacked && (e = z_pack(h)) != cudaSuccess) return DSM_E_CUDA;
       LBRaw a = raw_of(h, h->cur);
@@ -575,16 +768,19 @@ dsm_status dsm_step(dsm_lattice *h, long long nsteps) {
       if (e != cudaSuccess) return DSM_E_CUDA;
       h->zc ^= 1;
     } else {
-      // moments pass, then the fused pass (also the first step after
-      // dsm_set_fluid, whose g are populations)
+      // moments pass, then the fused pass (also the first step of a state given
+      // as populations)
       LBRaw a = raw_of(h, h->cur);
       e = h->tab.moments(a, h->stream);
       if (e == cudaSuccess) e = h->tab.node(a, 2, MODE_STEP, h->stream);
       if (e != cudaSuccess) return DSM_E_CUDA;
+      h->mfit = h->mok && h->eq;
     }
-    h->cur ^= 1;
+    if (!h->mom) {
+      h->cur ^= 1;
+      h->g_implicit = h->eq;
+    }
     h->step++;
-    h->g_implicit = h->eq;
     if (h->ring && h->step % h->ring_every == 0) {
       // observables record into the ring: device work only, no synchronisation
       if ((e = obs_launch(h)) != cudaSuccess) return DSM_E_CUDA;
@@ -645,7 +841,7 @@ dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun) {
   if (!h) return DSM_E_INVAL;
   const bool single = z_active(h);
   if (single_pass) *single_pass = single ? 1 : 0;
-  if (zrun) *zrun = single ? (h->zrun > 0 ? h->zrun : z_auto_run(h)) : 0;
+  if (zrun) *zrun = single ? (h->zrun > 0 ? h->zrun : m_active(h) ? m_zrun(h) : z_auto_run(h)) : 0;
   return DSM_OK;
 }
 
@@ -654,6 +850,13 @@ dsm_status dsm_step_moments(dsm_lattice *h) {
   if (!h) return DSM_E_INVAL;
   if (!h->has_fluid || h->latched) return DSM_E_STATE;
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  if (m_active(h) && !h->mom && h->mfit && h->g_implicit && m_enter(h) != cudaSuccess)
+    return DSM_E_CUDA;
+  if (h->mom) {
+    if (m_c(h) != cudaSuccess) return DSM_E_CUDA;
+    h->moments_ready = true;
+    return DSM_OK;
+  }
   LBRaw a = raw_of(h, h->cur);
   if (h->tab.moments(a, h->stream) != cudaSuccess) return DSM_E_CUDA;
   h->moments_ready = true;
@@ -665,11 +868,18 @@ dsm_status dsm_step_collide(dsm_lattice *h) {
   if (!h) return DSM_E_INVAL;
   if (!h->has_fluid || h->latched || !h->moments_ready) return DSM_E_STATE;
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  if (h->mom) {
+    if (m_c(h) != cudaSuccess || m_collide(h) != cudaSuccess) return DSM_E_CUDA;
+    h->step++;
+    h->moments_ready = false;
+    return DSM_OK;
+  }
   LBRaw a = raw_of(h, h->cur);
   if (h->tab.node(a, 2, MODE_STEP, h->stream) != cudaSuccess) return DSM_E_CUDA;
   h->cur ^= 1;
   h->step++;
   h->g_implicit = h->eq;
+  h->mfit = h->mok && h->eq;
   h->moments_ready = false;
   return DSM_OK;
 }
@@ -714,6 +924,18 @@ dsm_status dsm_get_field(dsm_lattice *h, int field, void *d_dst) {
     return cuda_status(e);
   }
   if (!h->has_fluid) return DSM_E_STATE;
+  if (h->mom) {
+    if (field == DSM_FIELD_C2 && !h->mcp)
+      return cuda_status(h->tab.mom_c(m_raw(h, h->mc), d_dst, h->stream));
+    if (field == DSM_FIELD_C2)
+      return cuda_status(cudaMemcpyAsync(d_dst, h->Cb[0], h->N * h->tab.real_bytes,
+                                         cudaMemcpyDeviceToDevice, h->stream));
+    e = m_statics(h);
+    if (e == cudaSuccess) e = m_c(h);
+    if (e == cudaSuccess)
+      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_FIELDS, field, d_dst, nullptr, h->stream);
+    return cuda_status(e);
+  }
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
   LBRaw a = raw_of(h, h->cur);
   a.out = d_dst;
@@ -726,6 +948,9 @@ dsm_status dsm_get_field(dsm_lattice *h, int field, void *d_dst) {
 dsm_status dsm_get_populations(dsm_lattice *h, void *d_f, void *d_g) {
   if (!h || !d_f || !d_g) return DSM_E_INVAL;
   if (!h->has_fluid) return DSM_E_STATE;
+  if (h->mom)
+    return cuda_status(h->tab.mom_expand(m_raw(h, h->mc), {d_f, nullptr, nullptr, d_g}, 2,
+                                         h->stream));
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
   LBRaw a = raw_of(h, h->cur);
   return cuda_status(h->tab.get_pops(a, d_f, d_g, h->stream));
@@ -733,6 +958,7 @@ dsm_status dsm_get_populations(dsm_lattice *h, void *d_f, void *d_g) {
 
 dsm_status dsm_set_populations(dsm_lattice *h, const void *d_f, const void *d_g) {
   if (!h || !d_f || !d_g) return DSM_E_INVAL;
+  m_drop(h);
   LBRaw a = raw_of(h, h->cur ^ 1);  // out = current buffer
   cudaError_t e = h->tab.set_pops(a, d_f, d_g, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, h->stream);
@@ -749,12 +975,14 @@ dsm_status dsm_set_g_storage(dsm_lattice *h, int form) {
   if (!h || (form != DSM_G_AUTO && form != DSM_G_POPULATIONS)) return DSM_E_INVAL;
   const bool eq = form == DSM_G_AUTO && h->prm.tau_g == 1.0 && !has_walls(&h->prm);
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  if (!eq && m_leave(h) != cudaSuccess) return DSM_E_CUDA;
   if (h->g_implicit && !eq) {
     // write the current g_eq out as populations of the current buffer
     LBRaw a = raw_of(h, h->cur ^ 1);  // g_out = current buffer
     a.Cprev = h->Cb[h->cur];
     if (h->tab.materialize(a, h->stream) != cudaSuccess) return DSM_E_CUDA;
     h->g_implicit = false;
+    h->mfit = false;
     h->moments_ready = false;
   }
   h->g_form = form;
@@ -765,19 +993,22 @@ dsm_status dsm_set_g_storage(dsm_lattice *h, int form) {
 dsm_status dsm_get_g_storage(dsm_lattice *h, int *form, int *implicit_now) {
   if (!h) return DSM_E_INVAL;
   if (form) *form = h->g_form;
-  if (implicit_now) *implicit_now = h->g_implicit ? 1 : 0;
+  if (implicit_now) *implicit_now = (h->mom ? h->mstepped : h->g_implicit) ? 1 : 0;
   return DSM_OK;
 }
 
 // Raw state (checkpoint): a 256-byte header, then the current buffer's f, g,
 // 16-bit g_0, C of the last collision and the g_eq planes, each region
-// 256-byte aligned.  Restoring it continues the run bitwise.
+// 256-byte aligned; a state held as moments (implicit = 2) has them in the
+// place of f, and the density they belong to in the header.  Restoring it
+// continues the run bitwise.
 namespace {
 constexpr unsigned kStateMagic = 0x53534d44u;  // "DSMS"
 struct StateHeader {
   unsigned magic, version;
   int lattice, precision, nx, ny, nz, implicit;
   long long step, pitch;
+  double rho;
 };
 struct StateLayout {
   size_t f, g, g0, C, M, total;
@@ -822,7 +1053,8 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
   hd.nx = h->prm.nx;
   hd.ny = h->prm.ny;
   hd.nz = h->prm.nz;
-  hd.implicit = h->g_implicit ? 1 : 0;
+  hd.implicit = h->mom ? 2 : h->g_implicit ? 1 : 0;
+  hd.rho = h->sp.rho3;
   hd.step = h->step;
   hd.pitch = h->pitch;
   char *d = (char *)d_dst;
@@ -830,6 +1062,13 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
   const size_t real = h->pitch * h->tab.real_bytes;
   cudaStream_t st = h->stream;
   cudaError_t e = cudaMemcpyAsync(d, &hd, sizeof(hd), cudaMemcpyHostToDevice, st);
+  if (h->mom) {
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(d + L.f, h->g[h->mc], mom_reals(h->kind) * real,
+                          cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return cuda_status(e);
+  }
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + L.f, h->f[h->cur], pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + L.g, h->g[h->cur], pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && h->tab.k16)
@@ -852,12 +1091,38 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
   if (e != cudaSuccess) return DSM_E_CUDA;
   if (hd.magic != kStateMagic || hd.version != 1 || hd.lattice != h->kind ||
       hd.precision != h->prm.precision || hd.nx != h->prm.nx || hd.ny != h->prm.ny ||
-      hd.nz != h->prm.nz || hd.pitch != h->pitch || (hd.implicit != 0 && hd.implicit != 1) ||
-      hd.step < 0)
+      hd.nz != h->prm.nz || hd.pitch != h->pitch || hd.implicit < 0 || hd.implicit > 2 ||
+      (hd.implicit == 2 && (h->tab.k16 || !(hd.rho > 0.0))) || hd.step < 0)
     return DSM_E_INVAL;
   const char *d = (const char *)d_src;
   const size_t pop = (size_t)h->q * h->pitch * h->tab.store_bytes;
   const size_t real = h->pitch * h->tab.real_bytes;
+  m_drop(h);
+  h->cur = 0;
+  if (hd.implicit == 2) {
+    e = cudaMemcpyAsync(h->g[0], d + L.f, mom_reals(h->kind) * real, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, st);
+    h->mc = 0;
+    h->mom = h->mstepped = true;
+    if (e == cudaSuccess && (!m_active(h) || hd.rho != h->sp.rho3)) {
+      // a handle that holds its state otherwise: expanded with the density the
+      // moments belong to
+      MomRaw r = m_raw(h, 0);
+      r.rho = hd.rho;
+      e = h->tab.mom_expand(r, m_planes(h, 1), 1, st);
+      h->cur = 1;
+      h->mom = false;
+    }
+    if (e != cudaSuccess) return DSM_E_CUDA;
+    h->step = hd.step;
+    h->g_implicit = true;
+    h->zpacked = false;
+    h->has_fluid = true;
+    h->latched = false;
+    h->moments_ready = false;
+    if (!h->mom && !h->eq) return dsm_set_g_storage(h, h->g_form);
+    return DSM_OK;
+  }
   e = cudaMemcpyAsync(h->f[0], d + L.f, pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->g[0], d + L.g, pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && h->tab.k16)
@@ -866,7 +1131,6 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->M, d + L.M, 4 * real, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, st);
   if (e != cudaSuccess) return DSM_E_CUDA;
-  h->cur = 0;
   h->step = hd.step;
   h->g_implicit = hd.implicit != 0;
   h->zpacked = false;
@@ -1033,12 +1297,22 @@ static dsm_status batch_items(dsm_lattice *const *hs, int n, const long long *ns
   return DSM_OK;
 }
 
+// Scratch of a batched call: of the population form's launch over all handles,
+// and of the launch on moments over those that can take it.
+static size_t batch_need(dsm_lattice *const *hs, int n, const std::vector<BatchRaw> &items) {
+  int m = 0;
+  for (int i = 0; i < n; i++) m += hs[i]->mok;
+  size_t b = (size_t)round_up((long long)hs[0]->tab.batch_bytes(items.data(), n), 256);
+  if (m) b += hs[0]->tab.mom_batch_bytes(m);
+  return b;
+}
+
 dsm_status dsm_batch_scratch_bytes(dsm_lattice *const *hs, int n, size_t *bytes) {
   if (!bytes) return DSM_E_INVAL;
   std::vector<BatchRaw> items;
   dsm_status s = batch_items(hs, n, nullptr, items);
   if (s != DSM_OK) return s;
-  *bytes = hs[0]->tab.batch_bytes(items.data(), n);
+  *bytes = batch_need(hs, n, items);
   return DSM_OK;
 }
 
@@ -1051,19 +1325,71 @@ dsm_status dsm_batch_step(dsm_lattice *const *hs, int n, const long long *nsteps
   if (s != DSM_OK) return s;
   for (int i = 0; i < n; i++)
     if (!hs[i]->has_fluid || hs[i]->latched) return DSM_E_STATE;
-  for (int i = 0; i < n; i++)
-    if (z_unpack(hs[i]) != cudaSuccess) return DSM_E_CUDA;
-  if (scratch_bytes < hs[0]->tab.batch_bytes(items.data(), n) || ((uintptr_t)d_scratch & 255u))
+  if (scratch_bytes < batch_need(hs, n, items) || ((uintptr_t)d_scratch & 255u))
     return DSM_E_WORKSPACE;
-  cudaError_t e = hs[0]->tab.batch(items.data(), n, d_scratch, scratch_bytes,
-                                   hs[0]->sp.rho_contrast != 0, hs[0]->eq, g_wait_limit,
-                                   hs[0]->stream);
-  if (e != cudaSuccess) return DSM_E_CUDA;
+  const LBTable &tab = hs[0]->tab;
+  cudaStream_t st = hs[0]->stream;
+  // lattices stepped on moments, and the others: a launch of each kind
+  std::vector<MomBatchRaw> mi;
+  std::vector<BatchRaw> pi;
+  std::vector<long long> left(nsteps, nsteps + n);
   for (int i = 0; i < n; i++) {
-    hs[i]->cur ^= (int)(nsteps[i] & 1);
-    hs[i]->step += nsteps[i];
-    hs[i]->moments_ready = false;
-    if (nsteps[i] > 0) hs[i]->g_implicit = hs[i]->eq;
+    dsm_lattice *h = hs[i];
+    if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+    if (!m_active(h)) {
+      if (m_leave(h) != cudaSuccess) return DSM_E_CUDA;
+      BatchRaw b = items[i];  // (leaving may have moved the current buffer)
+      b.r[0] = raw_of(h, 0);
+      b.r[1] = raw_of(h, 1);
+      b.cur0 = h->cur;
+      pi.push_back(b);
+      continue;
+    }
+    if (left[i] > 0 && !h->mom && !(h->mfit && h->g_implicit)) {
+      // a state given as populations: its first step as dsm_step takes it
+      LBRaw a = raw_of(h, h->cur);
+      if (tab.moments(a, st) != cudaSuccess || tab.node(a, 2, MODE_STEP, st) != cudaSuccess)
+        return DSM_E_CUDA;
+      h->cur ^= 1;
+      h->step++;
+      h->g_implicit = h->mfit = true;
+      h->moments_ready = false;
+      left[i]--;
+    }
+    if (left[i] == 0) continue;
+    if (!h->mom && m_enter(h) != cudaSuccess) return DSM_E_CUDA;
+    if (m_statics(h) != cudaSuccess) return DSM_E_CUDA;
+    MomBatchRaw b;
+    b.r[0] = m_raw(h, 0);
+    b.r[1] = m_raw(h, 1);
+    b.nsteps = left[i];
+    b.cur0 = h->mc;
+    mi.push_back(b);
+  }
+  size_t used = 0;
+  if (!pi.empty()) {
+    used = (size_t)round_up((long long)tab.batch_bytes(pi.data(), (int)pi.size()), 256);
+    if (tab.batch(pi.data(), (int)pi.size(), d_scratch, scratch_bytes, hs[0]->sp.rho_contrast != 0,
+                  hs[0]->eq, g_wait_limit, st) != cudaSuccess)
+      return DSM_E_CUDA;
+  }
+  if (!mi.empty() && tab.mom_batch(mi.data(), (int)mi.size(), (char *)d_scratch + used,
+                                   scratch_bytes - used, g_wait_limit, st) != cudaSuccess)
+    return DSM_E_CUDA;
+  for (int i = 0; i < n; i++) {
+    dsm_lattice *h = hs[i];
+    h->moments_ready = false;
+    h->step += left[i];
+    if (left[i] == 0) continue;
+    if (m_active(h)) {
+      h->mc ^= (int)(left[i] & 1);
+      h->mcp = false;
+      h->mstepped = true;
+    } else {
+      h->cur ^= (int)(left[i] & 1);
+      h->g_implicit = h->eq;
+      h->mfit = h->mok && h->eq;
+    }
   }
   return DSM_OK;
 }

@@ -251,6 +251,30 @@ struct ZMaps {
   CUtensorMap Q, U, C1;
 };
 
+// The step on moments (dsm_mom.cuh), type-erased: buffers q1, q2, w, pe of the
+// state it reads and writes, the frozen solid's data, and the constants.
+struct MomRaw {
+  int nx, ny, nz;
+  long long N, pitch;
+  void *in[4], *out[4];
+  void *sol, *lk, *qpl, *near, *list, *wall;
+  int *count;
+  const void *c1;
+  int *err;
+  double k[3], ak[3], kl, akl, rho, body[3], alpha_s;
+};
+// canonical planes of a state: f, A, u, C (pitch apart), or populations f and
+// g (N apart, in C)
+struct MomPlanes {
+  void *f, *A, *U, *C;
+};
+// one lattice of a batched launch on moments: r[p] reads buffer p
+struct MomBatchRaw {
+  MomRaw r[2];
+  long long nsteps;
+  int cur0;
+};
+
 struct LBTable {
   cudaError_t (*moments)(const LBRaw &, cudaStream_t);
   cudaError_t (*node)(const LBRaw &, int stage, int mode, cudaStream_t);
@@ -270,6 +294,22 @@ struct LBTable {
   cudaError_t (*zpack)(const LBRaw &r, void *Qz0, void *Qz1, void *Uz0, void *Uz1, void *C1z,
                        cudaStream_t);
   cudaError_t (*zunpack)(const LBRaw &r, const void *Qz, const void *Uz, void *Cout, cudaStream_t);
+  // step on moments (FP32 and FP64; null for 16-bit storage): one step with
+  // zrun planes per block (3D), its resident blocks per SM, the two passes (C
+  // of the step, then the rest: step, field or observables), and the
+  // conversions around it
+  cudaError_t (*mom_step)(const MomRaw &r, int zrun, cudaStream_t);
+  int (*mom_resident)();
+  cudaError_t (*mom_c)(const MomRaw &r, void *c, cudaStream_t);
+  cudaError_t (*mom_node)(const MomRaw &r, const void *c, int mode, int field, void *fields,
+                          double *partials, cudaStream_t);
+  cudaError_t (*mom_solid)(const MomRaw &r, cudaStream_t);
+  cudaError_t (*mom_init)(const MomRaw &r, const void *c, cudaStream_t);
+  cudaError_t (*mom_enter)(const MomRaw &r, const MomPlanes &p, cudaStream_t);
+  cudaError_t (*mom_expand)(const MomRaw &r, const MomPlanes &p, int what, cudaStream_t);
+  cudaError_t (*mom_batch)(const MomBatchRaw *items, int n, void *scratch, size_t bytes,
+                           unsigned long long spins, cudaStream_t);
+  size_t (*mom_batch_bytes)(int n);
   int q, real_bytes, store_bytes;
   bool k16;
 };

@@ -20,6 +20,8 @@
 // trajectory, up to rounding; 4 + 1 reals per node move instead of 2Q.
 #pragma once
 
+#include <string.h>
+
 #include <vector>
 
 #include "dsm_common.cuh"
@@ -30,6 +32,31 @@ namespace dsm {
 
 enum { MODE_STEP = 0, MODE_FIELDS = 1, MODE_OBS = 2 };
 constexpr int OBS_K = 5;  // sum C, sum C1, kinetic, max |u|, nonfinite
+
+// The observables of one block in FP64: sums of the first three values, maxima
+// of the others.
+__device__ __forceinline__ void block_reduce_obs(const double (&vals)[OBS_K], double *out) {
+  __shared__ double sh[OBS_K][32];
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int lane = tid & 31, warp = tid >> 5;
+  const int nw = (blockDim.x * blockDim.y * blockDim.z + 31) >> 5;
+#pragma unroll
+  for (int k = 0; k < OBS_K; k++) {
+    double v = vals[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double w2 = __shfl_down_sync(0xffffffffu, v, o);
+      v = (k == 3 || k == 4) ? fmax(v, w2) : v + w2;
+    }
+    if (lane == 0) sh[k][warp] = v;
+  }
+  __syncthreads();
+  if (tid < OBS_K) {
+    double v = sh[tid][0];
+    for (int w2 = 1; w2 < nw; w2++) v = (tid == 3 || tid == 4) ? fmax(v, sh[tid][w2]) : v + sh[tid][w2];
+    out[tid] = v;
+  }
+}
 
 template <class T>
 __device__ __forceinline__ T bwell(T c) {
@@ -785,26 +812,7 @@ __device__ __forceinline__ void node_body(const LBArgs<T, S> &a, int x, int y, i
       vals[2] = valid ? 0.5 * double(rho) * double(uu) : 0.0;
       vals[3] = valid ? sqrt(double(uu)) : 0.0;
       vals[4] = (valid && bad) ? 1.0 : 0.0;
-      __shared__ double sh[OBS_K][32];
-      const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-      const int lane = tid & 31, warp = tid >> 5;
-      const int nw = (blockDim.x * blockDim.y * blockDim.z + 31) >> 5;
-#pragma unroll
-      for (int k = 0; k < OBS_K; k++) {
-        double v = vals[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double w2 = __shfl_down_sync(0xffffffffu, v, o);
-          v = (k == 3 || k == 4) ? fmax(v, w2) : v + w2;
-        }
-        if (lane == 0) sh[k][warp] = v;
-      }
-      __syncthreads();
-      if (tid < OBS_K) {
-        double v = sh[tid][0];
-        for (int w2 = 1; w2 < nw; w2++) v = (tid == 3 || tid == 4) ? fmax(v, sh[tid][w2]) : v + sh[tid][w2];
-        a.partials[b * OBS_K + tid] = v;
-      }
+      block_reduce_obs(vals, a.partials + b * OBS_K);
     }
     return;
   }
@@ -1204,6 +1212,12 @@ inline dim3 lb_grid(int kind, int nx, int ny, int nz) {
   return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y, (nz + b.z - 1) / b.z);
 }
 
+}  // namespace dsm
+
+#include "dsm_mom.cuh"
+
+namespace dsm {
+
 template <class T, class S>
 LBArgs<T, S> typed(const LBRaw &r) {
   LBArgs<T, S> a;
@@ -1500,6 +1514,8 @@ struct LBOps {
     t.get_pops = &get_pops;
     t.set_pops = &set_pops;
     t.materialize = &materialize;
+    t.mom_step = nullptr;
+    if constexpr (!Store<S>::k16) MomOps<K, T>::table(t);
     t.q = Lat<K>::Q;
     t.real_bytes = sizeof(T);
     t.store_bytes = sizeof(S);
