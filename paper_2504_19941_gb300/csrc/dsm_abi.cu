@@ -373,7 +373,7 @@ void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mstat = h->mfit = false; }
 // C of the next step of a state held as moments, into Cb[0].
 cudaError_t m_c(dsm_lattice *h) {
   if (h->mcp) return cudaSuccess;
-  const cudaError_t e = h->tab.mom_c(m_raw(h, h->mc), h->Cb[0], h->stream);
+  const cudaError_t e = h->tab.mom_c(m_raw(h, h->mc), h->Cb[0], 0, h->stream);
   if (e == cudaSuccess) h->mcp = true;
   return e;
 }
@@ -391,11 +391,6 @@ cudaError_t m_enter(dsm_lattice *h) {
   return cudaSuccess;
 }
 
-// Planes per block of the 3D step: runs of zr planes give tiles * ceil(nz / zr)
-// blocks in waves of the resident ones; a run costs about three planes more
-// than it advances (two of halo on each side, partly summed, and the first
-// copies).  101^3: 36.7 us with the 9 planes this gives, 42.4 / 37.5 / 43.2
-// with 6 / 13 / 17; 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96.
 int m_zrun(dsm_lattice *h) {
   if (h->zrun > 0) return h->zrun;
   if (h->mzrun) return h->mzrun;
@@ -404,26 +399,35 @@ int m_zrun(dsm_lattice *h) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per_sm = h->tab.mom_resident(), nz = h->prm.nz;
-  const long long resident = (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
-  const long long tiles = (long long)z_tiles_x(h->prm.nx) * z_tiles_y(h->prm.ny);
-  double best = 1e300;
-  for (int zr = 1; zr <= nz; zr++) {
-    const long long blocks = tiles * ((nz + zr - 1) / zr);
-    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0);
-    if (cost < best - 1e-9) {
-      best = cost;
-      h->mzrun = zr;
-    }
-  }
+  const int per_sm = h->tab.mom_resident();
+  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz,
+                      (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1));
   return h->mzrun;
+}
+
+// Whether dsm_relax_solid runs on moments: D2Q9 in FP32 or FP64, each axis
+// periodic, or a mirror on both sides (a wall's bounce-back has no image node).
+bool m_relax_of(const dsm_lattice *h, MomRelax *m) {
+  if (h->kind != DSM_D2Q9 || !h->tab.mom_relax) return false;
+  const int n[2] = {h->prm.nx, h->prm.ny};
+  for (int a = 0; a < 2; a++) {
+    const int lo = h->prm.face[2 * a], hi = h->prm.face[2 * a + 1];
+    if (lo == DSM_FACE_WALL || hi == DSM_FACE_WALL) return false;
+    m->mirror[a] = lo == DSM_FACE_MIRROR;
+    if (m->mirror[a] && n[a] < 2) return false;
+  }
+  m->mask = h->mask;
+  m->beta2 = 2.0 * h->sp.beta;
+  m->omega2 = 2.0 * h->sp.omega;
+  return true;
 }
 
 // The second pass of a step of a state held as moments (C in Cb[0]).
 cudaError_t m_collide(dsm_lattice *h) {
   cudaError_t e = m_statics(h);
   if (e == cudaSuccess)
-    e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_STEP, 0, nullptr, nullptr, h->stream);
+    e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], 0, MODE_STEP, 0, 0, nullptr, nullptr,
+                        h->stream);
   if (e != cudaSuccess) return e;
   h->mc ^= 1;
   h->mcp = false;
@@ -496,7 +500,8 @@ cudaError_t obs_launch(dsm_lattice *h) {
     e = m_statics(h);
     if (e == cudaSuccess) e = m_c(h);
     if (e == cudaSuccess)
-      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_OBS, 0, nullptr, h->partials, h->stream);
+      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], 0, MODE_OBS, 0, 0, nullptr, h->partials,
+                          h->stream);
     if (e != cudaSuccess) return e;
     obs_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, h->obs_blocks, h->obs);
     return cudaGetLastError();
@@ -682,6 +687,25 @@ dsm_status dsm_relax_solid(dsm_lattice *h, const unsigned char *d_mask, int step
   h->has_fluid = false;
   h->zpacked = false;
   m_drop(h);
+  MomRelax mr;
+  if (m_relax_of(h, &mr)) {
+    // every relaxation time is 1 here, so moments carry the state (dsm_mom.cuh)
+    MomRaw a[2] = {m_raw(h, 0), m_raw(h, 1)};
+    for (MomRaw &r : a) {
+      r.k[0] = h->sp.kappa1 + h->sp.kappa3;
+      r.ak[0] = h->sp.a2 * r.k[0];
+      r.rho = 1.0;
+    }
+    e = h->tab.mom_relax(a[1], mr, 0, h->C1, h->stream);
+    for (int t = 0; t < steps && e == cudaSuccess; t++)
+      e = h->tab.mom_relax(a[t & 1], mr, 1, nullptr, h->stream);
+    if (e == cudaSuccess) e = h->tab.mom_relax(a[steps & 1], mr, 2, h->C1, h->stream);
+    h->sp.beta = h->prm.beta;
+    h->sp.omega = h->prm.omega;
+    if (e != cudaSuccess) return DSM_E_CUDA;
+    h->has_solid = true;
+    return DSM_OK;
+  }
   LBRaw r = raw_of(h, 1);  // out = buffer 0
   r.eq = 0;
   if ((e = h->tab.init(r, h->C1, 1, h->stream)) != cudaSuccess) return DSM_E_CUDA;
@@ -725,7 +749,7 @@ dsm_status dsm_set_fluid(dsm_lattice *h, const void *d_c2) {
   if (m_active(h)) {  // the rest state as moments
     if (!h->mom) h->mstat = false;  // (its buffers held another form)
     e = m_statics(h);
-    if (e == cudaSuccess) e = h->tab.mom_init(m_raw(h, 1), d_c2, h->stream);  // writes buffer 0
+    if (e == cudaSuccess) e = h->tab.mom_init(m_raw(h, 1), d_c2, 0, h->stream);  // writes buffer 0
     h->mc = 0;
     h->mom = true;
     h->mcp = h->mfit = h->mstepped = false;
@@ -926,14 +950,15 @@ dsm_status dsm_get_field(dsm_lattice *h, int field, void *d_dst) {
   if (!h->has_fluid) return DSM_E_STATE;
   if (h->mom) {
     if (field == DSM_FIELD_C2 && !h->mcp)
-      return cuda_status(h->tab.mom_c(m_raw(h, h->mc), d_dst, h->stream));
+      return cuda_status(h->tab.mom_c(m_raw(h, h->mc), d_dst, 0, h->stream));
     if (field == DSM_FIELD_C2)
       return cuda_status(cudaMemcpyAsync(d_dst, h->Cb[0], h->N * h->tab.real_bytes,
                                          cudaMemcpyDeviceToDevice, h->stream));
     e = m_statics(h);
     if (e == cudaSuccess) e = m_c(h);
     if (e == cudaSuccess)
-      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], MODE_FIELDS, field, d_dst, nullptr, h->stream);
+      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], 0, MODE_FIELDS, field, 0, d_dst, nullptr,
+                          h->stream);
     return cuda_status(e);
   }
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;

@@ -268,6 +268,12 @@ struct MomRaw {
 struct MomPlanes {
   void *f, *A, *U, *C;
 };
+// the solid's relaxation on moments (2D): its region, penalties, mirror axes
+struct MomRelax {
+  const unsigned char *mask;
+  double beta2, omega2;
+  int mirror[2];
+};
 // one lattice of a batched launch on moments: r[p] reads buffer p
 struct MomBatchRaw {
   MomRaw r[2];
@@ -300,11 +306,12 @@ struct LBTable {
   // conversions around it
   cudaError_t (*mom_step)(const MomRaw &r, int zrun, cudaStream_t);
   int (*mom_resident)();
-  cudaError_t (*mom_c)(const MomRaw &r, void *c, cudaStream_t);
-  cudaError_t (*mom_node)(const MomRaw &r, const void *c, int mode, int field, void *fields,
-                          double *partials, cudaStream_t);
+  cudaError_t (*mom_c)(const MomRaw &r, void *c, long long cstride, cudaStream_t);
+  cudaError_t (*mom_node)(const MomRaw &r, const void *c, long long cstride, int mode, int field,
+                          int index, void *fields, double *partials, cudaStream_t);
+  cudaError_t (*mom_relax)(const MomRaw &r, const MomRelax &m, int what, void *c, cudaStream_t);
   cudaError_t (*mom_solid)(const MomRaw &r, cudaStream_t);
-  cudaError_t (*mom_init)(const MomRaw &r, const void *c, cudaStream_t);
+  cudaError_t (*mom_init)(const MomRaw &r, const void *c, long long cstride, cudaStream_t);
   cudaError_t (*mom_enter)(const MomRaw &r, const MomPlanes &p, cudaStream_t);
   cudaError_t (*mom_expand)(const MomRaw &r, const MomPlanes &p, int what, cudaStream_t);
   cudaError_t (*mom_batch)(const MomBatchRaw *items, int n, void *scratch, size_t bytes,

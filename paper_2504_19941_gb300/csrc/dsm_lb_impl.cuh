@@ -1515,6 +1515,7 @@ struct LBOps {
     t.set_pops = &set_pops;
     t.materialize = &materialize;
     t.mom_step = nullptr;
+    t.mom_relax = nullptr;
     if constexpr (!Store<S>::k16) MomOps<K, T>::table(t);
     t.q = Lat<K>::Q;
     t.real_bytes = sizeof(T);

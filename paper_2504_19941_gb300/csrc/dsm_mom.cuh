@@ -1359,6 +1359,62 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// Stage 1: the state at rest of C1 (cf) into a.out, and the C1 the next step
+// would see.  Beyond a mirror the neighbour is the edge node, its velocity
+// reversed along the normal.
+template <class T>
+__global__ void __launch_bounds__(256)
+    mom_relax_init_kernel(const __grid_constant__ MomArgs<T> a, const __grid_constant__ Mom1<T> m1,
+                          const T *cf) {
+  using L = Lat<0>;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= a.nx || y >= a.ny) return;
+  const int face[6] = {m1.mirror[0], m1.mirror[0], m1.mirror[1], m1.mirror[1], 0, 0};
+  Hood h;
+  h.init_faces(x, y, 0, a.nx, a.ny, 1, face);
+  h.guard(a.err);
+  const int n = h.g(h.ox[1] + h.oy[1]);
+  const T C = cf[n];
+  T lap = T(0);
+#pragma unroll
+  for (int i = 1; i < L::Q; i++) lap += T(L::w(i)) * (cf[h.plus<L>(i)] - C);
+  T mu = a.k[0] * mom_well(C) - a.ak[0] * (T(6) * lap);
+  if (m1.mask[n] != 0 ? C < T(0.5) : C > T(0.5)) mu += m1.beta2 * (C - T(0.5));
+  if (C < T(0)) mu += m1.omega2 * C;
+  if (C > T(1)) mu -= m1.omega2 * (T(1) - C);
+  mom_store<0, T>(a.out, n, mu, T(0), T(0), T(0), T(0), C, T(0), T(0), T(0));
+}
+template <class T>
+__global__ void __launch_bounds__(256)
+    mom_relax_c_kernel(const __grid_constant__ MomArgs<T> a, const __grid_constant__ Mom1<T> m1,
+                       T *out) {
+  using L = Lat<0>;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= a.nx || y >= a.ny) return;
+  const int face[6] = {m1.mirror[0], m1.mirror[0], m1.mirror[1], m1.mirror[1], 0, 0};
+  Hood h;
+  h.init_faces(x, y, 0, a.nx, a.ny, 1, face);
+  h.guard(a.err);
+  const int n = h.g(h.ox[1] + h.oy[1]);
+  const Quad<T> q = reinterpret_cast<const Quad<T> *>(a.in.q1)[n];
+  const T uu = fm(q.v[3], q.v[3], ml(q.v[2], q.v[2]));
+  T sa = T(0), sd = T(0);
+#pragma unroll
+  for (int i = 1; i < L::Q; i++) {
+    const Quad<T> p = reinterpret_cast<const Quad<T> *>(a.in.q1)[h.minus<L>(i)];
+    const bool rx = m1.mirror[0] && x - L::cx(i) != (x - L::cx(i) + a.nx) % a.nx;
+    const bool ry = m1.mirror[1] && y - L::cy(i) != (y - L::cy(i) + a.ny) % a.ny;
+    const T u[3] = {rx ? -p.v[2] : p.v[2], ry ? -p.v[3] : p.v[3], T(0)};
+    const T g = fm(p.v[1], mom_b(mom_dot<L>(i, u)), p.v[0]);
+    if (L::w(i) == L::w(1)) sa = ad(sa, g);
+    else sd = ad(sd, g);
+  }
+  const T o = fm(ml(T(1.5), q.v[1]), uu, ml(T(1.0 - L::w(0)), q.v[0]));
+  out[n] = ad(q.v[1], fm(T(L::w(1)), sa, fm(T(L::w(L::Q - 1)), sd, -o)));
+}
+
 // canonical state planes: f (Q), u (D), and A and C of each free fluid
 template <class T>
 struct MomCanon {
@@ -1588,16 +1644,40 @@ struct Mom3 {
   }
 };
 
+// Planes per block of the 3D step: runs of zr planes give tiles * ceil(nz / zr)
+// blocks in waves of the resident ones; a run costs about three planes more
+// than it advances (two of halo on each side, partly summed, and the first
+// copies).  101^3: 36.7 us with the 9 planes this gives, 42.4 / 37.5 / 43.2
+// with 6 / 13 / 17; 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96
+// (without the wall pass).
+inline int mom_zrun(int nx, int ny, int nz, long long resident) {
+  const long long tiles = (long long)((nx + M3_X - 1) / M3_X) * ((ny + 7) / 8);
+  double best = 1e300;
+  int run = 1;
+  for (int zr = 1; zr <= nz; zr++) {
+    const long long blocks = tiles * ((nz + zr - 1) / zr);
+    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0);
+    if (cost < best - 1e-9) {
+      best = cost;
+      run = zr;
+    }
+  }
+  return run;
+}
+
 inline int mom_blocks(long long n) {
   const long long b = (n + 255) / 256;
   return (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
 }
 
-template <int K, class T>
+template <int K, class T, int NF = 1>
 struct MomOps {
+  // 3D: 32 x 8 tiles, two nodes per thread; blocks per SM by what the sums of
+  // NF fluids leave of the registers (128, 168, 255 per thread)
+  using Step3 = Mom3<T, NF, 8, 2, (NF == 1 ? 4 : NF == 2 ? 3 : 2)>;
   static cudaError_t step(const MomRaw &r, int zrun, cudaStream_t st) {
     if constexpr (K == 1) {
-      return Mom3<T, 1, 8, 2, 4>::step(r, zrun, st);
+      return Step3::step(r, zrun, st);
     } else {
       Mom1<T> m1 = {};
       // small lattices: 64-thread tiles, so that the work spreads over the SMs
@@ -1614,7 +1694,7 @@ struct MomOps {
     }
   }
   static int resident() {
-    if constexpr (K == 1) return Mom3<T, 1, 8, 2, 4>::resident();
+    if constexpr (K == 1) return Step3::resident();
     else return 0;
   }
   static cudaError_t solid(const MomRaw &r, cudaStream_t st) {
@@ -1626,37 +1706,71 @@ struct MomOps {
         mom_typed<T>(r));
     return cudaGetLastError();
   }
-  static cudaError_t init(const MomRaw &r, const void *c, cudaStream_t st) {
-    mom_init_kernel<K, T, 1><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0,
-                               st>>>(mom_typed<T>(r), (const T *)c, 0);
+  // (c, cn, out: planes cstride apart, one per free fluid)
+  static cudaError_t init(const MomRaw &r, const void *c, long long cstride, cudaStream_t st) {
+    mom_init_kernel<K, T, NF><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0,
+                               st>>>(mom_typed<T>(r), (const T *)c, cstride);
     return cudaGetLastError();
   }
   static cudaError_t enter(const MomRaw &r, const MomPlanes &p, cudaStream_t st) {
-    mom_enter_kernel<K, T, 1><<<mom_blocks(r.N), 256, 0, st>>>(
+    mom_enter_kernel<K, T, NF><<<mom_blocks(r.N), 256, 0, st>>>(
         mom_typed<T>(r), MomCanon<T>{(T *)p.f, (T *)p.A, (T *)p.U, (T *)p.C});
     return cudaGetLastError();
   }
-  static cudaError_t c_pass(const MomRaw &r, void *out, cudaStream_t st) {
-    mom_c_kernel<K, T, 1><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0, st>>>(
-        mom_typed<T>(r), (T *)out, 0);
+  static cudaError_t c_pass(const MomRaw &r, void *out, long long cstride, cudaStream_t st) {
+    mom_c_kernel<K, T, NF><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0, st>>>(
+        mom_typed<T>(r), (T *)out, cstride);
     return cudaGetLastError();
   }
-  static cudaError_t node(const MomRaw &r, const void *cn, int mode, int field, void *fields,
-                          double *partials, cudaStream_t st) {
+  static cudaError_t node(const MomRaw &r, const void *cn, long long cstride, int mode, int field,
+                          int index, void *fields, double *partials, cudaStream_t st) {
     const dim3 g = lb_grid(K, r.nx, r.ny, r.nz), b = lb_block(K, r.nx, r.ny, r.nz);
     const MomArgs<T> a = mom_typed<T>(r);
     const T *c = (const T *)cn;
     T *o = (T *)fields;
-    if (mode == MODE_STEP) mom_node_kernel<K, T, 1, MODE_STEP><<<g, b, 0, st>>>(a, c, 0, o, field, 0, partials);
+    if (mode == MODE_STEP)
+      mom_node_kernel<K, T, NF, MODE_STEP><<<g, b, 0, st>>>(a, c, cstride, o, field, index, partials);
     else if (mode == MODE_FIELDS)
-      mom_node_kernel<K, T, 1, MODE_FIELDS><<<g, b, 0, st>>>(a, c, 0, o, field, 0, partials);
-    else mom_node_kernel<K, T, 1, MODE_OBS><<<g, b, 0, st>>>(a, c, 0, o, field, 0, partials);
+      mom_node_kernel<K, T, NF, MODE_FIELDS><<<g, b, 0, st>>>(a, c, cstride, o, field, index, partials);
+    else if constexpr (NF == 1)
+      mom_node_kernel<K, T, NF, MODE_OBS><<<g, b, 0, st>>>(a, c, cstride, o, field, index, partials);
     return cudaGetLastError();
   }
   static cudaError_t expand(const MomRaw &r, const MomPlanes &p, int what, cudaStream_t st) {
-    mom_expand_kernel<K, T, 1><<<mom_blocks(r.N), 256, 0, st>>>(
+    mom_expand_kernel<K, T, NF><<<mom_blocks(r.N), 256, 0, st>>>(
         mom_typed<T>(r), MomCanon<T>{(T *)p.f, (T *)p.A, (T *)p.U, (T *)p.C}, what);
     return cudaGetLastError();
+  }
+  static Mom1<T> relax_typed(const MomRelax &m) {
+    Mom1<T> m1;
+    m1.mask = m.mask;
+    m1.beta2 = T(m.beta2);
+    m1.omega2 = T(m.omega2);
+    m1.mirror[0] = m.mirror[0];
+    m1.mirror[1] = m.mirror[1];
+    return m1;
+  }
+  // stage 1 (2D): what 0, the state at rest of c; 1, one step; 2, C into c
+  static cudaError_t relax(const MomRaw &r, const MomRelax &m, int what, void *c, cudaStream_t st) {
+    if constexpr (K != 0) {
+      return cudaErrorNotSupported;
+    } else {
+      const dim3 g = lb_grid(K, r.nx, r.ny, 1), b = lb_block(K, r.nx, r.ny, 1);
+      const MomArgs<T> a = mom_typed<T>(r);
+      const Mom1<T> m1 = relax_typed(m);
+      if (what == 0) {
+        mom_relax_init_kernel<T><<<g, b, 0, st>>>(a, m1, (const T *)c);
+      } else if (what == 2) {
+        mom_relax_c_kernel<T><<<g, b, 0, st>>>(a, m1, (T *)c);
+      } else if ((long long)r.nx * r.ny < 2ll * 152 * 256) {
+        mom_step2_kernel<T, 16, 4, 1><<<dim3((r.nx + 15) / 16, (r.ny + 3) / 4), dim3(16, 4),
+                                        M2Smem<T, 16, 4>::total, st>>>(a, m1);
+      } else {
+        mom_step2_kernel<T, 32, 8, 1><<<dim3((r.nx + 31) / 32, (r.ny + 7) / 8), dim3(32, 8),
+                                        M2Smem<T, 32, 8>::total, st>>>(a, m1);
+      }
+      return cudaGetLastError();
+    }
   }
   static constexpr size_t batch_smem() {
     return K == 1 ? (size_t)M3Smem<T, 1, 8>::total : (size_t)M2Smem<T, 32, 8>::total;
@@ -1743,6 +1857,7 @@ struct MomOps {
     return cudaSuccess;
   }
   static void table(LBTable &t) {
+    t.mom_relax = &relax;
     t.mom_step = &step;
     t.mom_resident = &resident;
     t.mom_solid = &solid;

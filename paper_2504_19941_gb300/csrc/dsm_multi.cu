@@ -678,12 +678,21 @@ struct dsm_mlattice {
   int zc, nxp, nyp, step_form, zrun, zrun_auto;
   char *Qz[2], *Uz[2], *Pz[2], *C1z;
   CUtensorMap maps[2][4];
+  // step on moments (dsm_mom.cuh): mok, every relaxation time 1, equal
+  // densities, and a lattice the single-pass step takes.  The state is then
+  // always held as moments, buffer mc: quads (A_2, C_2, u_x, u_y) in Qz, u_z in
+  // Uz, pairs in Pz, quads (dP, G) in mq2; mcp, C[0] holds the C of its next step
+  bool mok, mstat, mcp;
+  int mc, mzrun;
+  char *mq2[2], *msol, *mlk, *mnear, *mlist, *mwall;
+  int *mcount;
 };
 
 namespace {
 
 struct MLLayout {
-  size_t f[2], g[2], C[2], C1, M, err, Qz[2], Uz[2], Pz[2], C1z, total;
+  size_t f[2], g[2], C[2], C1, M, err, Qz[2], Uz[2], Pz[2], C1z, mq2[2], msol, mlk, mnear, mlist,
+      mwall, total;
 };
 
 // g held as g_eq: tau_g = 1 and every face periodic
@@ -720,6 +729,15 @@ MLLayout ml_layout(int q, int nf, int real_bytes, long long pitch, bool eq,
     L.Pz[b] = take(2 * (size_t)(nf - 1) * P * real_bytes);
   }
   L.C1z = take(P * real_bytes);
+  // and of the step on moments, per node: quads (dP, G) twice, the solid's
+  // pairs, link bits, a byte, a list entry, and the wall sums
+  const size_t n = z ? (size_t)pitch : 0;
+  for (int b = 0; b < 2; b++) L.mq2[b] = take(4 * n * real_bytes);
+  L.msol = take(2 * n * real_bytes);
+  L.mlk = take(4 * n);
+  L.mnear = take(n);
+  L.mlist = take(4 * n + 256);
+  L.mwall = take(4 * n * real_bytes);
   L.total = o;
   return L;
 }
@@ -1017,8 +1035,114 @@ cudaError_t mlz_unpack(dsm_mlattice *h) {
   return e;
 }
 
+// ---- step on moments ----------------------------------------------------------
+MomRaw mlm_raw(const dsm_mlattice *h, int src) {
+  MomRaw r;
+  memset(&r, 0, sizeof(r));
+  r.nx = h->prm.nx;
+  r.ny = h->prm.ny;
+  r.nz = h->prm.nz;
+  r.N = h->N;
+  r.pitch = h->pitch;
+  for (int o = 0; o < 2; o++) {
+    const int b = o ? src ^ 1 : src;
+    void **d = o ? r.out : r.in;
+    d[0] = h->Qz[b];
+    d[1] = h->mq2[b];
+    d[2] = h->Uz[b];
+    d[3] = h->Pz[b];
+  }
+  r.sol = h->msol;
+  r.lk = h->mlk;
+  r.qpl = h->f[0];
+  r.near = h->mnear;
+  r.list = h->mlist;
+  r.wall = h->mwall;
+  r.count = h->mcount;
+  r.c1 = h->C1;
+  r.err = h->err;
+  const double a2 = h->prm.alpha * h->prm.alpha;
+  for (int f = 0; f < h->nf; f++) {
+    r.k[f] = h->kappa[1 + f];
+    r.ak[f] = a2 * h->kappa[1 + f];
+  }
+  r.kl = h->kappa[h->nf + 1];
+  r.akl = a2 * r.kl;
+  r.rho = h->rho[h->nf];
+  for (int a = 0; a < 3; a++) r.body[a] = h->prm.body_force[a];
+  r.alpha_s = h->prm.alpha_s > 0.0 ? h->prm.alpha_s : h->prm.alpha;
+  return r;
+}
+// dispatch over the free fluids
+template <class T, class Fn>
+cudaError_t mlm_dispatch(const dsm_mlattice *h, Fn fn) {
+  switch (h->nf) {
+    case 1: return fn(MomOps<1, T, 1>());
+    case 2: return fn(MomOps<1, T, 2>());
+    case 3: return fn(MomOps<1, T, 3>());
+    default: return cudaErrorInvalidValue;
+  }
+}
+template <class T>
+cudaError_t mlm_init(dsm_mlattice *h) {
+  h->mc = 0;
+  h->mcp = false;
+  return mlm_dispatch<T>(h, [&](auto k) {
+    cudaError_t e = cudaSuccess;
+    if (!h->mstat) e = k.solid(mlm_raw(h, 0), h->stream);
+    if (e != cudaSuccess) return e;
+    h->mstat = true;
+    return k.init(mlm_raw(h, 1), h->C[0], h->pitch, h->stream);
+  });
+}
+template <class T>
+cudaError_t mlm_c(dsm_mlattice *h) {  // C of the next step, into C[0]
+  if (h->mcp) return cudaSuccess;
+  const cudaError_t e = mlm_dispatch<T>(
+      h, [&](auto k) { return k.c_pass(mlm_raw(h, h->mc), h->C[0], h->pitch, h->stream); });
+  if (e == cudaSuccess) h->mcp = true;
+  return e;
+}
+// planes per block: as the two-fluid step (m_zrun, dsm_abi.cu)
+template <class T>
+int mlm_zrun(dsm_mlattice *h) {
+  if (h->zrun > 0) return h->zrun;
+  if (h->mzrun) return h->mzrun;
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  mlm_dispatch<T>(h, [&](auto k) {
+    per_sm = k.resident();
+    return cudaSuccess;
+  });
+  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz,
+                      (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1));
+  return h->mzrun;
+}
+template <class T>
+cudaError_t mlm_step(dsm_mlattice *h) {
+  cudaError_t e;
+  if (h->step_form == DSM_STEP_TWO_PASS) {
+    e = mlm_c<T>(h);
+    if (e == cudaSuccess)
+      e = mlm_dispatch<T>(h, [&](auto k) {
+        return k.node(mlm_raw(h, h->mc), h->C[0], h->pitch, MODE_STEP, 0, 0, nullptr, nullptr,
+                      h->stream);
+      });
+  } else {
+    const int zrun = mlm_zrun<T>(h);
+    e = mlm_dispatch<T>(h, [&](auto k) { return k.step(mlm_raw(h, h->mc), zrun, h->stream); });
+  }
+  if (e == cudaSuccess) {
+    h->mc ^= 1;
+    h->mcp = false;
+  }
+  return e;
+}
+
 template <class T>
 cudaError_t ml_step(dsm_mlattice *h) {
+  if (h->mok) return mlm_step<T>(h);
   if (mlz_active(h)) {
     if (!h->zpacked) {
       if (!mlz_maps(h)) return cudaErrorInvalidValue;
@@ -1050,6 +1174,14 @@ cudaError_t ml_step(dsm_mlattice *h) {
 
 template <class T>
 cudaError_t ml_fields(dsm_mlattice *h, int field, int index, void *dst) {
+  if (h->mok) {
+    const cudaError_t e = mlm_c<T>(h);
+    if (e != cudaSuccess) return e;
+    return mlm_dispatch<T>(h, [&](auto k) {
+      return k.node(mlm_raw(h, h->mc), h->C[0], h->pitch, MODE_FIELDS, field, index, dst, nullptr,
+                    h->stream);
+    });
+  }
   const cudaError_t eu = mlz_unpack<T>(h);
   if (eu != cudaSuccess) return eu;
   MLArgs<T> a = ml_args<T>(h, h->cur);
@@ -1127,6 +1259,15 @@ dsm_status dsm_ml_create(const dsm_params *p, int nfluid, const double *kappa, c
     h->Pz[b] = w + L.Pz[b];
   }
   h->C1z = h->zok ? w + L.C1z : nullptr;
+  h->mok = h->zok;
+  for (int f = 0; f < nfluid; f++) h->mok = h->mok && tau[f] == 1.0 && rho[f] == rho[0];
+  for (int b = 0; b < 2; b++) h->mq2[b] = w + L.mq2[b];
+  h->msol = w + L.msol;
+  h->mlk = w + L.mlk;
+  h->mnear = w + L.mnear;
+  h->mcount = (int *)(w + L.mlist);
+  h->mlist = w + L.mlist + 256;
+  h->mwall = w + L.mwall;
   // no solid until one is set: C1 = 0; no error latched
   if (cudaMemsetAsync(h->C1, 0, (size_t)pitch * rb, h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) != cudaSuccess) {
@@ -1159,6 +1300,7 @@ dsm_status dsm_ml_set_solid(dsm_mlattice *h, const void *d_field, int kind) {
   h->has_solid = true;
   h->has_fluid = false;
   h->zpacked = false;
+  h->mstat = false;
   return DSM_OK;
 }
 
@@ -1177,7 +1319,8 @@ dsm_status dsm_ml_set_fluids(dsm_mlattice *h, const void *d_c) {
   h->zpacked = false;
   if (cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) != cudaSuccess) return DSM_E_CUDA;
   cudaError_t e;
-  if (h->real_bytes == 8) e = ml_dispatch<double, InitL>(h, ml_args<double>(h, 1));
+  if (h->mok) e = h->real_bytes == 8 ? mlm_init<double>(h) : mlm_init<float>(h);
+  else if (h->real_bytes == 8) e = ml_dispatch<double, InitL>(h, ml_args<double>(h, 1));
   else e = ml_dispatch<float, InitL>(h, ml_args<float>(h, 1));
   if (e != cudaSuccess) return DSM_E_CUDA;
   h->has_fluid = true;
@@ -1208,6 +1351,13 @@ dsm_status dsm_ml_get_field(dsm_mlattice *h, int field, int index, void *d_dst) 
 dsm_status dsm_ml_get_populations(dsm_mlattice *h, void *d_f, void *d_g) {
   if (!h || (!d_f && !d_g)) return DSM_E_INVAL;
   if (!h->has_fluid) return DSM_E_STATE;
+  if (h->mok) {
+    auto get = [&](auto k) {
+      return k.expand(mlm_raw(h, h->mc), {d_f, nullptr, nullptr, d_g}, 2, h->stream);
+    };
+    return ml_status(h->real_bytes == 8 ? mlm_dispatch<double>(h, get)
+                                        : mlm_dispatch<float>(h, get));
+  }
   const size_t row = (size_t)h->N * h->real_bytes, pb = (size_t)h->pitch * h->real_bytes;
   for (int i = 0; d_f && i < h->q; i++)
     if (cudaMemcpyAsync((char *)d_f + i * row, h->f[h->cur] + i * pb, row,
@@ -1253,7 +1403,9 @@ dsm_status dsm_ml_step_info(dsm_mlattice *h, int *single_pass, int *zrun) {
   if (single_pass) *single_pass = single ? 1 : 0;
   if (zrun) {
     *zrun = 0;
-    if (single) *zrun = h->zrun > 0 ? h->zrun
+    if (single && h->mok)
+      *zrun = h->real_bytes == 8 ? mlm_zrun<double>(h) : mlm_zrun<float>(h);
+    else if (single) *zrun = h->zrun > 0 ? h->zrun
                                     : (h->real_bytes == 8 ? mlz_auto_run<double>(h)
                                                           : mlz_auto_run<float>(h));
   }
