@@ -22,6 +22,7 @@ struct FEArgs {
   const float *c1, *c2;
   const unsigned char *mask;
   float *grad;
+  const float *dir;  // direction of the slope (null: none)
   double *partials;
 };
 
@@ -61,13 +62,27 @@ dsm_status fem_args_of(const dsm_params *p, int nfluid, const double *kappa, con
 cudaError_t fe_multi_launch(int kind, FEMArgs a, const FEMCons &cons, double *energy,
                             double *terms, void *scratch, cudaStream_t st);
 
+// What one energy evaluation leaves besides the gradient: E and its terms
+// (null: not wanted), and the constraint's derivative dE/dV (dEcs).  With dir,
+// also the slope of the gradient along dir.
+// counter (zero before and after): the evaluation's last block sums the
+// partials; null: a second launch does.
+struct FEFin {
+  double dP, kcs, V0;
+  double *energy, *terms, *dEcs, *slope;
+  unsigned *counter;
+};
+constexpr int FE_KS = FE_K + 1;  // partials of an evaluation with a slope
+
 long long fe_blocks(int kind, int nx, int ny, int nz);
 size_t fe_scratch_bytes(int kind, int nx, int ny, int nz);
-// defer: when given, the constraint's constant is not added to the gradient;
-// *defer receives its device address (null when there is none).
 cudaError_t fe_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
-                      double *terms, void *scratch, cudaStream_t st,
-                      const double **defer = nullptr);
+                      double *terms, void *scratch, cudaStream_t st);
+// Energy, complete gradient and its slope along a.dir.  scratch:
+// fe_slope_scratch_bytes() bytes, its first 256 zero before and after.
+size_t fe_slope_scratch_bytes();
+cudaError_t fe_slope_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
+                            double *slope, void *scratch, cudaStream_t st);
 
 constexpr int LINCOMB_MAX = 64;  // most vectors one dsm_vec_lincomb combines
 struct LinCoef {
@@ -77,27 +92,21 @@ struct LinCoef {
 
 size_t vec_scratch_bytes(long long n);
 size_t vec_dots_scratch_bytes(long long n, int nv);
+// elements a grid-stride vector pass of n elements has in flight per step
+int vec_blocks(long long n);
 cudaError_t vec_dots(long long n, int nv, const float *V, long long stride, const float *x,
                      double *out, void *scratch, cudaStream_t st);
-// A trial point's gradient and slope: g += c[0] if c is given, out[0] = g.d,
-// one launch (scratch: vec_scratch_bytes(n), whose counter word starts and
-// ends at zero).
+// g += c[0] if c is given, out[0] = g.d, one launch (counter: zero before and
+// after; partials: VEC_BLOCKS doubles).
 cudaError_t vec_trial_slope(long long n, const double *c, float *g, const float *d, double *out,
-                            void *scratch, cudaStream_t st);
-// the counter word of a vec_scratch_bytes scratch (behind the block partials)
-inline unsigned *vec_scratch_counter(void *scratch) {
-  return (unsigned *)((char *)scratch + VEC_BLOCKS * sizeof(double));
-}
-// out[0] = a.a, out[1] = b.b, out[2] = c.c in one pass (scratch:
-// vec_dots_scratch_bytes(n, 3))
-cudaError_t vec_sumsq3(long long n, const float *a, const float *b, const float *c, double *out,
-                       void *scratch, cudaStream_t st);
+                            double *partials, unsigned *counter, cudaStream_t st);
 cudaError_t vec_lincomb(long long n, int nv, const float *V, long long stride, const double *coef,
                         const float *x, double cx, float *y, cudaStream_t st);
 cudaError_t vec_dot(long long n, const float *x, const float *y, double *out, const double *scale,
                     void *scratch, cudaStream_t st);
 cudaError_t vec_axpy_dev(long long n, double sign, const double *a, const double *b,
                          const float *x, float *y, cudaStream_t st);
+cudaError_t vec_scale_dev(long long n, const double *a, const float *x, float *y, cudaStream_t st);
 cudaError_t vec_axpby(long long n, double a, const float *x, double b, float *y, cudaStream_t st);
 cudaError_t lbfgs_direction(long long n, int m, const int *order, const float *S, const float *Y,
                             const double *rho, const double *gamma, const float *g, float *r,

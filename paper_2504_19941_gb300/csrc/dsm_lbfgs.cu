@@ -15,8 +15,12 @@
 //
 // The pair bookkeeping (the s.y and y.y matrices, S^T g, Y^T g, gamma, the
 // ring of stored pairs) and the compact-form solve live on the device, in one
-// small state block updated by one-thread kernels; the host drives only the
-// line search, whose decisions need the trial's energy and slope.  Each trial
+// small state block; the host drives only the line search, whose decisions need
+// the trial's energy and slope.  An iteration whose first trial is accepted is
+// three or four launches: the direction and the first trial point
+// (lb_dir_kernel), the trial's energy, gradient and slope (fe_slope_launch: two
+// with a volume constraint), and, once the host has taken it, the new pair with every dot product of the update, whose last block
+// folds them into the state and solves for the next direction (lb_pair_kernel).  Each trial
 // reads one block of six doubles (slope, energy, the direction's initial
 // slope, |g|^2 of the current point, the pairs in use, the next pair's slot),
 // so an iteration whose first trial is accepted reads the host once.
@@ -24,9 +28,11 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "dsm_em.cuh"
+#include "dsm_reduce.cuh"
 #include "dsm_trace.cuh"
 
 using namespace dsm;
@@ -106,67 +112,72 @@ __global__ void lb_init_kernel(LbState *s) {
 // when there are none or the compact direction does not descend (the pairs
 // are then dropped): coef, cx, and rb[2] .. rb[5].  The pairs' k x k matrices
 // are staged into shared memory by the lanes and solved there by the warp.
-__global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, const double *dots, int m,
-                                                     double sy1) {
-  __shared__ double sy[LB_MAX_M * LB_MAX_M], yy[LB_MAX_M * LB_MAX_M];
-  __shared__ double A[LB_MAX_M], B[LB_MAX_M], w[LB_MAX_M];
-  __shared__ double cs[LB_MAX_M], cy[LB_MAX_M];
-  __shared__ int ord[LB_MAX_M];
-  __shared__ int ok_s;
-  const int l = threadIdx.x;
+struct LbStepShared {
+  double sy[LB_MAX_M * LB_MAX_M], yy[LB_MAX_M * LB_MAX_M], w[LB_MAX_M];
+};
+// (called by one warp; every global access of a kind is in flight at once: a
+// lane holds pair l's slot and products)
+__device__ void lb_step(LbState *s, const double *dots, int m, double sy1, LbStepShared &h) {
+  double *sy = h.sy, *yy = h.yy, *w = h.w;
+  const int l = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  int k = s->k, nxt = s->nxt;
+  int slot = l < k ? s->order[l] : -1;  // of pair l, oldest first
+  double gg = s->rb[3], gamma = s->gamma;
+  double Al = 0.0, Bl = 0.0;
   if (dots) {
-    const int nxt = s->nxt;
     const double yy1 = dots[2 * m], ss = dots[2 * m + 2];
+    gg = dots[2 * m + 1];
     const bool accept = sy1 > 1e-12 * sqrt(ss * yy1);
-    for (int i = l; i < m; i += 32) {
-      const double agn = dots[i], bgn = dots[m + i];
+    if (l < m) {  // lane l: slot l
+      const double agn = dots[l], bgn = dots[m + l], ag = s->Ag[l], bg = s->Bg[l];
       if (accept) {
-        if (i == nxt) {
-          s->SY[i * m + nxt] = sy1;
-          s->YY[i * m + nxt] = yy1;
-        } else {
-          const double yy_i = bgn - s->Bg[i];  // y_i . y_new
-          s->SY[i * m + nxt] = agn - s->Ag[i];  // s_i . y_new
-          s->YY[i * m + nxt] = yy_i;
-          s->YY[nxt * m + i] = yy_i;
-        }
+        const double yy_l = l == nxt ? yy1 : bgn - bg;   // y_l . y_new
+        s->SY[l * m + nxt] = l == nxt ? sy1 : agn - ag;  // s_l . y_new
+        s->YY[l * m + nxt] = yy_l;
+        s->YY[nxt * m + l] = yy_l;
       }
-      s->Ag[i] = agn;
-      s->Bg[i] = bgn;
+      s->Ag[l] = agn;
+      s->Bg[l] = bgn;
     }
+    // drop the pair that slot nxt held, append the new one
+    const unsigned kept = __ballot_sync(full, l < k && slot != nxt);
+    const int src = __fns(kept, 0, l + 1);  // lane of the l-th kept pair (-1: none)
+    const int moved = __shfl_sync(full, slot, src & 31);
+    k = __popc(kept);
+    slot = l < k ? moved : -1;
+    if (accept) {
+      if (l == k) slot = nxt;
+      k++;
+      gamma = sy1 / yy1;
+      nxt = nxt + 1 == m ? 0 : nxt + 1;
+    }
+    if (l < k) s->order[l] = slot;
     if (l == 0) {
-      int k = 0;
-      for (int i = 0; i < s->k; i++)
-        if (s->order[i] != nxt) s->order[k++] = s->order[i];
-      if (accept) {
-        s->gamma = sy1 / yy1;
-        s->order[k++] = nxt;
-        s->nxt = (nxt + 1) % m;
-      }
-      s->k = k;
-      s->rb[3] = dots[2 * m + 1];
+      s->gamma = gamma;
+      s->nxt = nxt;
+      s->rb[3] = gg;
     }
-    __syncthreads();
+    __syncwarp();
+    const int ls = slot < 0 ? 0 : slot;
+    Al = dots[ls];
+    Bl = dots[m + ls];
+  } else if (l < k) {
+    Al = s->Ag[slot];
+    Bl = s->Bg[slot];
   }
-  const int k = s->k;
-  const double gg = s->rb[3], gamma = s->gamma;
-  for (int i = l; i < k; i += 32) {
-    ord[i] = s->order[i];
-  }
-  __syncthreads();
-  for (int i = l; i < k; i += 32) {
-    for (int j = 0; j < k; j++) {
-      sy[i * k + j] = s->SY[ord[i] * m + ord[j]];
-      yy[i * k + j] = s->YY[ord[i] * m + ord[j]];
+  for (int e0 = 0; e0 < k * k; e0 += 32) {  // the stored pairs' products, oldest first
+    const int e = e0 + l, i = e / (k > 0 ? k : 1), j = e - i * k;
+    const int si = __shfl_sync(full, slot, i & 31), sj = __shfl_sync(full, slot, j & 31);
+    if (e < k * k) {
+      sy[e] = s->SY[si * m + sj];
+      yy[e] = s->YY[si * m + sj];
     }
-    A[i] = s->Ag[ord[i]];
-    B[i] = s->Bg[ord[i]];
   }
-  __syncthreads();
+  __syncwarp();
   // the compact-form solve across the warp (lane l owns pair l): the
   // triangular substitutions column by column with the diagonal's
   // reciprocals, the middle product row by row, dg0 by a warp reduction
-  const unsigned full = 0xffffffffu;
   bool ok = k > 0;
   double cx = -gamma, dg0 = 0.0, wl = 0.0, ul = 0.0;
   if (ok) {
@@ -174,7 +185,7 @@ __global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, const double *d
     ok = __all_sync(full, dl != 0.0);
     if (ok) {
       const double inv = 1.0 / dl;
-      double r = l < k ? A[l] : 0.0;  // R w = a, R upper triangular
+      double r = l < k ? Al : 0.0;  // R w = a, R upper triangular
       for (int i = k - 1; i >= 0; i--) {
         const double wi = __shfl_sync(full, r, i) * __shfl_sync(full, inv, i);
         if (l == i) wl = wi;
@@ -184,7 +195,7 @@ __global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, const double *d
       __syncwarp();
       double zl = 0.0;  // (D + gamma YY) w - gamma b
       if (l < k) {
-        zl = sy[l * k + l] * wl - gamma * B[l];
+        zl = sy[l * k + l] * wl - gamma * Bl;
         for (int j = 0; j < k; j++) zl += gamma * yy[l * k + j] * w[j];
       }
       for (int j = 0; j < k; j++) {  // R^T u = z, R^T lower triangular
@@ -192,7 +203,7 @@ __global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, const double *d
         if (l == j) ul = uj;
         if (l > j) zl -= sy[j * k + l] * uj;
       }
-      double part = l < k ? -ul * A[l] + gamma * wl * B[l] : 0.0;
+      double part = l < k ? -ul * Al + gamma * wl * Bl : 0.0;
       for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(full, part, o);
       dg0 = cx * gg + part;
       ok = dg0 < 0.0;
@@ -202,63 +213,237 @@ __global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, const double *d
     cx = -1.0 / fmax(sqrt(gg), 1e-300);
     dg0 = cx * gg;
   }
-  if (l < k) {
-    cs[l] = -ul;
-    cy[l] = gamma * wl;
-  }
   if (l == 0) {
-    ok_s = ok;
     s->k = ok ? k : 0;
     s->cx = cx;
     s->rb[2] = dg0;
     s->rb[4] = ok ? (double)k : 0.0;
-    s->rb[5] = (double)s->nxt;
+    s->rb[5] = (double)nxt;
   }
-  __syncthreads();
   for (int i = l; i < 2 * m; i += 32) s->coef[i] = 0.0;
-  __syncthreads();
-  if (ok_s)
-    for (int i = l; i < k; i += 32) {
-      s->coef[ord[i]] = cs[i];
-      s->coef[m + ord[i]] = cy[i];
-    }
+  __syncwarp();
+  if (ok && l < k) {
+    s->coef[slot] = -ul;
+    s->coef[m + slot] = gamma * wl;
+  }
+}
+
+__global__ void __launch_bounds__(32) lb_step_kernel(LbState *s, int m) {
+  __shared__ LbStepShared h;
+  lb_step(s, nullptr, m, 0.0, h);
+}
+
+// W elements of a vector (W = 4: 16 bytes aligned)
+template <int W>
+struct Pack {
+  float v[W];
+};
+template <int W>
+__device__ __forceinline__ Pack<W> ld(const float *p) {
+  Pack<W> r;
+  if constexpr (W == 4) {
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    r.v[0] = q.x;
+    r.v[1] = q.y;
+    r.v[2] = q.z;
+    r.v[3] = q.w;
+  } else {
+    r.v[0] = *p;
+  }
+  return r;
+}
+template <int W>
+__device__ __forceinline__ void stv(float *p, const Pack<W> &a) {
+  if constexpr (W == 4) *reinterpret_cast<float4 *>(p) = make_float4(a.v[0], a.v[1], a.v[2], a.v[3]);
+  else *p = a.v[0];
 }
 
 // d = cx g + sum_j coef_j V_j over the 2m stored vectors, coefficients from
-// the device state (a vector with a zero coefficient is not read)
-__global__ void __launch_bounds__(256) lb_lincomb_kernel(long long n, int nv, const float *V,
-                                                         long long stride, const LbState *s,
-                                                         const float *g, float *d) {
-  __shared__ float c[2 * LB_MAX_M];
+// the device state (a vector with a zero coefficient is not read), and the first
+// trial point xt = x + d.  W elements of a vector per load, five vectors' loads
+// in flight; from the far end of the vectors to their start, because the pass
+// over the same vectors before it (lb_pair_kernel) runs forward and what it read
+// last is still in L2 (20 vectors of 128^3 are 168 MB, L2 129).  128^3: 24.5 us,
+// where the combination and the trial point took 35.0 + 6.6 us.
+template <int W>
+__global__ void __launch_bounds__(256) lb_dir_kernel(long long n, int nv, const float *V,
+                                                     const LbState *s, const float *g, float *d,
+                                                     const float *x, float *xt) {
+  __shared__ float c[2 * LB_MAX_M + 5];
+  __shared__ int v[2 * LB_MAX_M + 5];
+  __shared__ int used;
   __shared__ float cx;
-  if (threadIdx.x < nv) c[threadIdx.x] = (float)s->coef[threadIdx.x];
-  if (threadIdx.x == 0) cx = (float)s->cx;
+  if (threadIdx.x == 0) {
+    int k = 0;
+    for (int j = 0; j < nv; j++)
+      if ((float)s->coef[j] != 0.0f) {
+        c[k] = (float)s->coef[j];
+        v[k++] = j;
+      }
+    used = k;
+    cx = (float)s->cx;
+  }
   __syncthreads();
-  // four elements a grid apart per iteration: four loads per stream in flight
-  const long long G = (long long)gridDim.x * blockDim.x;
-  long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  for (; k + 3 * G < n; k += 4 * G) {
-    float acc[4];
+  const int nu = used;
+  const long long G = (long long)gridDim.x * blockDim.x, N = n / W;
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= N) return;
+  for (long long i = t + (N - 1 - t) / G * G; i >= 0; i -= G) {
+    const long long k = W * i;
+    Pack<W> acc = ld<W>(g + k);
+    Pack<W> xx = ld<W>(x + k);
 #pragma unroll
-    for (int u = 0; u < 4; u++) acc[u] = cx * g[k + u * G];
-    for (int j = 0; j < nv; j++) {
-      if (c[j] == 0.0f) continue;
-      const float *vj = V + j * stride + k;
-      float vv[4];
+    for (int u = 0; u < W; u++) acc.v[u] = cx * acc.v[u];
+    int j = 0;
+    for (; j + 5 <= nu; j += 5) {
+      Pack<W> vv[5];
 #pragma unroll
-      for (int u = 0; u < 4; u++) vv[u] = vj[u * G];
+      for (int e = 0; e < 5; e++) vv[e] = ld<W>(V + v[j + e] * n + k);
 #pragma unroll
-      for (int u = 0; u < 4; u++) acc[u] += c[j] * vv[u];
+      for (int e = 0; e < 5; e++)
+#pragma unroll
+        for (int u = 0; u < W; u++) acc.v[u] += c[j + e] * vv[e].v[u];
+    }
+    for (; j < nu; j++) {
+      const Pack<W> vv = ld<W>(V + v[j] * n + k);
+#pragma unroll
+      for (int u = 0; u < W; u++) acc.v[u] += c[j] * vv.v[u];
+    }
+    stv<W>(d + k, acc);
+#pragma unroll
+    for (int u = 0; u < W; u++) xx.v[u] += acc.v[u];
+    stv<W>(xt + k, xx);
+  }
+}
+
+// The accepted step's update in one pass over the vectors: the pair (s = step d,
+// y = gt - g into slot nxt), every stored vector against the new gradient gt
+// (v < hi is s_v, else y_{v-hi}; slots hi.. have never held a pair), and y.y,
+// gt.gt, s.s, all as carried-error sums.  gt is read once for all of them, W
+// elements of a vector per load, five vectors' loads in flight.  The grid's last
+// block sums the partials into dots and, on the update's last launch, folds them
+// into the state and solves for the next direction (lb_step).  128^3, m = 10:
+// 50.6 us, where seven launches (the pair in two, 20 dot products one vector per
+// block row at 59 us, three squares, two sums, the solve) took 91.  Bound by
+// latency (16 warps per SM at 118 registers); two block rows of ten vectors took
+// 70.9, staging in shared memory by asynchronous copies 56.
+constexpr int LB_NV = 20, LB_NK = LB_NV + 3, LB_BLOCKS = 152 * 2, LB_NT = 256;
+struct LbPair {
+  long long n;
+  int m, hi, v0, cnt, nxt, last;
+  float step;
+  double sy;
+  const float *d, *g, *gt;
+  float *V;
+  double *partials, *dots;
+  unsigned *counter;
+  LbState *s;
+};
+__device__ __forceinline__ void lb_acc(FF &s, float a, float b) {
+  const FF p = two_prod(a, b);
+  const FF t = two_sum(s.hi, p.hi);
+  s.hi = t.hi;
+  s.lo += t.lo + p.lo;
+}
+template <bool PAIR, int W>
+__global__ void __launch_bounds__(LB_NT, 2) lb_pair_kernel(const __grid_constant__ LbPair a) {
+  __shared__ FF sh[LB_NT / 32][32];
+  __shared__ LbStepShared hs;
+  __shared__ bool last;
+  FF acc[32];
+#pragma unroll
+  for (int j = 0; j < 32; j++) acc[j] = FF{0.0f, 0.0f};
+  const long long G = (long long)gridDim.x * LB_NT;
+  auto vec = [&](int j) {  // vector v0 + j
+    const int v = a.v0 + j;
+    return (long long)(v < a.hi ? v : a.m + v - a.hi) * a.n;
+  };
+  for (long long i = blockIdx.x * (long long)LB_NT + threadIdx.x; i < a.n / W; i += G) {
+    const long long k = W * i;
+    const Pack<W> gg = ld<W>(a.gt + k);
+    if (PAIR) {
+      Pack<W> ss = ld<W>(a.d + k), yy = ld<W>(a.g + k);
+#pragma unroll
+      for (int u = 0; u < W; u++) {
+        ss.v[u] = a.step * ss.v[u];
+        yy.v[u] = gg.v[u] - yy.v[u];
+        lb_acc(acc[LB_NV], yy.v[u], yy.v[u]);
+        lb_acc(acc[LB_NV + 1], gg.v[u], gg.v[u]);
+        lb_acc(acc[LB_NV + 2], ss.v[u], ss.v[u]);
+      }
+      stv<W>(a.V + a.nxt * a.n + k, ss);  // (read again below by this thread)
+      stv<W>(a.V + (a.m + a.nxt) * a.n + k, yy);
     }
 #pragma unroll
-    for (int u = 0; u < 4; u++) d[k + u * G] = acc[u];
+    for (int j0 = 0; j0 < LB_NV; j0 += 5) {
+      if (j0 + 5 <= a.cnt) {
+        Pack<W> vv[5];
+#pragma unroll
+        for (int e = 0; e < 5; e++) vv[e] = ld<W>(a.V + vec(j0 + e) + k);
+#pragma unroll
+        for (int e = 0; e < 5; e++)
+#pragma unroll
+          for (int u = 0; u < W; u++) lb_acc(acc[j0 + e], vv[e].v[u], gg.v[u]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 5; e++)
+          if (j0 + e < a.cnt) {
+            const Pack<W> vv = ld<W>(a.V + vec(j0 + e) + k);
+#pragma unroll
+            for (int u = 0; u < W; u++) lb_acc(acc[j0 + e], vv.v[u], gg.v[u]);
+          }
+      }
+    }
   }
-  for (; k < n; k += G) {
-    float acc = cx * g[k];
-    for (int j = 0; j < nv; j++)
-      if (c[j] != 0.0f) acc += c[j] * V[j * stride + k];
-    d[k] = acc;
+  // 32 sums across the warp by halving: lane l ends with sum l (31 pair sums
+  // instead of 5 x 23)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int e = 0; e < o; e++) {
+      const FF keep = up ? acc[e + o] : acc[e], send = up ? acc[e] : acc[e + o];
+      const FF got = {__shfl_xor_sync(0xffffffffu, send.hi, o),
+                      __shfl_xor_sync(0xffffffffu, send.lo, o)};
+      acc[e] = ff_add(keep, got);
+    }
   }
+  sh[warp][lane] = acc[0];
+  __syncthreads();
+  if (threadIdx.x < LB_NK) {
+    FF r = sh[0][threadIdx.x];
+    for (int w = 1; w < LB_NT / 32; w++) r = ff_add(r, sh[w][threadIdx.x]);
+    a.partials[(long long)threadIdx.x * gridDim.x + blockIdx.x] = (double)r.hi + (double)r.lo;
+  }
+  // the block that counts itself last finishes; no block waits for another
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int j = warp; j < LB_NK; j += LB_NT / 32) {  // a warp per sum
+    const volatile double *p = a.partials + (long long)j * gridDim.x;
+    double t = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += p[b];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+      const int v = a.v0 + j;
+      if (j < a.cnt) a.dots[v < a.hi ? v : a.m + v - a.hi] = t;
+      else if (PAIR && j >= LB_NV) a.dots[2 * a.m + j - LB_NV] = t;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *a.counter = 0u;
+  if (a.last && warp == 0) lb_step(a.s, a.dots, a.m, a.sy, hs);
+}
+template <bool PAIR, int W>
+cudaError_t lb_pair_launch(const LbPair &a, int grid, cudaStream_t st) {
+  lb_pair_kernel<PAIR, W><<<grid, LB_NT, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 // drop the stored pairs (after a line search that found no step)
@@ -299,7 +484,8 @@ struct Minimiser {
   float *xb[2], *gb[2], *d, *hist;
   double *E[2], *dots, *vout;  // vout: the state's read-back block
   LbState *state;
-  void *fe_scr, *vec_scr, *dots_scr;
+  void *fe_scr, *vec_scr, *dots_scr, *slope_scr;
+  int hi = 0;  // slots that have held a pair
 
   cudaError_t evaluate(const float *x, double *e_out, float *g_out) {
     if (multi) {
@@ -320,12 +506,11 @@ struct Minimiser {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e;
   }
-  // trial point xt = x + a d: energy and directional derivative, read back
-  // with the rest of the state's block (rb: 6 doubles).  Two fluids: the
-  // energy goes straight into the block, and the constraint's constant is
-  // added to the gradient in the same pass that takes the slope.
-  cudaError_t trial(double a, const float *x, float *xt, double *Et, float *gt, double *rb) {
-    cudaError_t e = vec_lincomb(n, 1, d, n, &a, x, 1.0, xt, st);
+  // energy and slope at the trial point xt = x + a d (made: xt is there
+  // already), read back with the rest of the state's block (rb: 6 doubles).
+  cudaError_t trial(double a, const float *x, float *xt, double *Et, float *gt, double *rb,
+                    bool made) {
+    cudaError_t e = made ? cudaSuccess : vec_lincomb(n, 1, d, n, &a, x, 1.0, xt, st);
     if (multi) {
       if (e == cudaSuccess) e = evaluate(xt, Et, gt);
       if (e == cudaSuccess) e = vec_dot(n, gt, d, vout, nullptr, vec_scr, st);
@@ -336,12 +521,42 @@ struct Minimiser {
       b.c1 = active == 2 ? fixed : xt;
       b.c2 = active == 2 ? xt : fixed;
       b.grad = gt;
-      const double *cst = nullptr;
-      if (e == cudaSuccess) e = fe_launch(kind, b, dP, kcs, V0, vout + 1, nullptr, fe_scr, st, &cst);
-      if (e == cudaSuccess) e = vec_trial_slope(n, cst, gt, d, vout, vec_scr, st);
+      b.dir = d;
+      if (e == cudaSuccess) e = fe_slope_launch(kind, b, dP, kcs, V0, vout + 1, vout, slope_scr, st);
     }
     if (e == cudaSuccess) e = read(rb, vout, 6);
     return e;
+  }
+  // the accepted step: the new pair in slot nxt, every dot product of the
+  // update, and the state's next direction
+  cudaError_t update(int nxt, double step, double sy, const float *g, const float *gt) {
+    LbPair a;
+    a.n = n;
+    a.m = m;
+    a.nxt = nxt;
+    a.step = (float)step;
+    a.sy = sy;
+    a.d = d;
+    a.g = g;
+    a.gt = gt;
+    a.V = hist;
+    a.counter = (unsigned *)dots_scr;
+    a.partials = (double *)((char *)dots_scr + 256);
+    a.dots = dots;
+    a.s = state;
+    a.hi = hi = std::max(hi, nxt + 1);
+    const int w = n % 4 == 0 ? 4 : 1;  // (every vector starts n reals after another)
+    const int grid = (int)std::min<long long>((n / w + LB_NT - 1) / LB_NT, LB_BLOCKS);
+    for (int v = 0; v < 2 * hi; v += LB_NV) {
+      a.v0 = v;
+      a.cnt = std::min(LB_NV, 2 * hi - v);
+      a.last = v + LB_NV >= 2 * hi;
+      const cudaError_t e =
+          v == 0 ? (w == 4 ? lb_pair_launch<true, 4>(a, grid, st) : lb_pair_launch<true, 1>(a, grid, st))
+                 : (w == 4 ? lb_pair_launch<false, 4>(a, grid, st) : lb_pair_launch<false, 1>(a, grid, st));
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
   }
 };
 
@@ -366,18 +581,24 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
   M.fe_scr = w + off[8];
   M.vec_scr = w + off[9];
   M.dots_scr = w + off[10];
+  M.slope_scr = w + off[11];
   const long long n = M.n;
   cudaStream_t st = M.st;
-  const int lgrid = (int)std::min<long long>((n + 255) / 256, 152 * 16);
+  // 16-byte loads: every vector of the workspace starts a multiple of n reals
+  // after an aligned address; the caller's x may start anywhere
+  const bool wide = n % 4 == 0 && ((uintptr_t)d_x & 15u) == 0;
+  const int lgrid = (int)std::min<long long>((n / (wide ? 4 : 1) + 255) / 256, 152 * 8);
 #define CK(expr)                                    \
   do {                                              \
     if ((expr) != cudaSuccess) return DSM_E_CUDA;   \
   } while (0)
 
   // stored pairs start at zero, so unused slots add nothing to a combination;
-  // the fused slope pass's block counter starts at zero
+  // the block counters start at zero
   CK(cudaMemsetAsync(M.hist, 0, (size_t)2 * m * n * sizeof(float), st));
-  CK(cudaMemsetAsync(vec_scratch_counter(M.vec_scr), 0, sizeof(unsigned), st));
+  CK(cudaMemsetAsync(M.dots, 0, (size_t)(2 * m + 3) * sizeof(double), st));
+  CK(cudaMemsetAsync(M.dots_scr, 0, 256, st));
+  CK(cudaMemsetAsync(M.slope_scr, 0, 256, st));
   lb_init_kernel<<<1, 1, 0, st>>>(M.state);
   CK(cudaGetLastError());
   int cur = 0;  // x = xb[cur], g = gb[cur], E = E[cur]
@@ -390,24 +611,23 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
   long long it = 0, evals = 1;
   int converged = 0;
   bool fresh = false;  // gg is that of the current point (read after its last update)
-  const double *pending = nullptr;  // the accepted step's dots, not yet folded into the state
-  double pending_sy = 0.0;          // and its pair's s.y
+  bool solved = false;  // the state holds the current point's direction (lb_pair_kernel)
   while (it < max_iter) {
-    // the pair update and the direction on the device, then the first trial
-    // (a = 1), whose read also brings |g|^2 of the current point and the
-    // direction's slope
-    lb_step_kernel<<<1, 32, 0, st>>>(M.state, pending, m, pending_sy);
+    // the direction and the first trial (a = 1), whose read also brings |g|^2
+    // of the current point and the direction's slope
+    if (!solved) lb_step_kernel<<<1, 32, 0, st>>>(M.state, m);
     CK(cudaGetLastError());
-    pending = nullptr;
+    solved = false;
     const float *x = M.xb[cur];
     float *xt = M.xb[cur ^ 1];
     const float *g = M.gb[cur];
     float *gt = M.gb[cur ^ 1];
     double *Et = M.E[cur ^ 1];
-    lb_lincomb_kernel<<<lgrid, 256, 0, st>>>(n, 2 * m, M.hist, n, M.state, g, M.d);
+    if (wide) lb_dir_kernel<4><<<lgrid, 256, 0, st>>>(n, 2 * m, M.hist, M.state, g, M.d, x, xt);
+    else lb_dir_kernel<1><<<lgrid, 256, 0, st>>>(n, 2 * m, M.hist, M.state, g, M.d, x, xt);
     CK(cudaGetLastError());
     double a = 1.0;
-    CK(M.trial(a, x, xt, Et, gt, rb));
+    CK(M.trial(a, x, xt, Et, gt, rb, true));
     double df = rb[0], f = rb[1];
     const double dg0 = rb[2];
     gg = rb[3];
@@ -461,7 +681,7 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
       d_prev = df;
       if (trials >= max_trials) break;
       a *= 2.0;
-      CK(M.trial(a, x, xt, Et, gt, rb));
+      CK(M.trial(a, x, xt, Et, gt, rb, false));
       df = rb[0];
       f = rb[1];
       trials++;
@@ -470,7 +690,7 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
     if (!done && !bracketed) step = a_prev;  // never bracketed: the last descending point
     while (!done && bracketed && trials < max_trials) {
       a = cubic_step(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2]);
-      CK(M.trial(a, x, xt, Et, gt, rb));
+      CK(M.trial(a, x, xt, Et, gt, rb, false));
       df = rb[0];
       f = rb[1];
       trials++;
@@ -500,24 +720,17 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
       break;
     }
     if (last != step) {  // the accepted point is not the last one evaluated
-      CK(M.trial(step, x, xt, Et, gt, rb));
+      CK(M.trial(step, x, xt, Et, gt, rb, false));
       df = rb[0];
       f = rb[1];
       evals++;
     }
     // new pair s = step d, y = g_new - g into slot nxt; every stored s, y
-    // against g_new in one batched pass (the new pair's included), then y.y,
-    // g_new.g_new and s.s; s.y = step (g_new.d - g.d) from the slopes.  The
-    // device folds them into its state (no host read).
-    float *s_new = M.hist + (size_t)nxt * n;
-    float *y_new = M.hist + (size_t)(m + nxt) * n;
-    const double minus1 = -1.0;
-    CK(vec_axpby(n, step, M.d, 0.0, s_new, st));
-    CK(vec_lincomb(n, 1, g, n, &minus1, gt, 1.0, y_new, st));
-    CK(vec_dots(n, 2 * m, M.hist, n, gt, M.dots, M.dots_scr, st));
-    CK(vec_sumsq3(n, y_new, gt, s_new, M.dots + 2 * m, M.dots_scr, st));
-    pending = M.dots;  // folded in by the next iteration's lb_step_kernel
-    pending_sy = step * (df - dg0);
+    // against g_new (the new pair's included), y.y, g_new.g_new and s.s;
+    // s.y = step (g_new.d - g.d) from the slopes.  The device folds them into
+    // its state and solves for the next direction (no host read).
+    CK(M.update(nxt, step, step * (df - dg0), g, gt));
+    solved = true;
     fresh = false;
     cur ^= 1;
     f_val = f;
@@ -574,7 +787,8 @@ static size_t lbfgs_layout_n(long long n, int m, size_t fe_bytes, size_t off[12]
   off[7] = take(sizeof(LbState));                 // the pair bookkeeping on the device
   off[8] = take(fe_bytes);
   off[9] = take(vec_scratch_bytes(n));
-  off[10] = take(vec_dots_scratch_bytes(n, 4 * m));
+  off[10] = take(256 + (size_t)LB_BLOCKS * LB_NK * sizeof(double));
+  off[11] = take(fe_slope_scratch_bytes());
   return o;
 }
 
