@@ -390,6 +390,9 @@ dsm_status dsm_vec_dot(long long n, const float *d_x, const float *d_y, double *
 /* y[k] += a * x[k] with a = sign * d_a[0] * (d_b ? d_b[0] : 1)  (device scalars) */
 dsm_status dsm_vec_axpy_dev(long long n, double sign, const double *d_a, const double *d_b,
                             const float *d_x, float *d_y, void *cuda_stream);
+/* y[k] = d_a[0] * x[k]  (device scalar) */
+dsm_status dsm_vec_scale_dev(long long n, const double *d_a, const float *d_x, float *d_y,
+                             void *cuda_stream);
 /* y[k] = a * x[k] + b * y[k] with host scalars */
 dsm_status dsm_vec_axpby(long long n, double a, const float *d_x, double b, float *d_y,
                          void *cuda_stream);

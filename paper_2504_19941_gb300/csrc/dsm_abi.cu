@@ -1255,6 +1255,12 @@ dsm_status dsm_vec_axpy_dev(long long n, double sign, const double *d_a, const d
   return cuda_status(vec_axpy_dev(n, sign, d_a, d_b, d_x, d_y, (cudaStream_t)cuda_stream));
 }
 
+dsm_status dsm_vec_scale_dev(long long n, const double *d_a, const float *d_x, float *d_y,
+                             void *cuda_stream) {
+  if (n < 0 || !d_a || !d_x || !d_y) return DSM_E_INVAL;
+  return cuda_status(vec_scale_dev(n, d_a, d_x, d_y, (cudaStream_t)cuda_stream));
+}
+
 dsm_status dsm_vec_axpby(long long n, double a, const float *d_x, double b, float *d_y,
                          void *cuda_stream) {
   if (n < 0 || !d_x || !d_y) return DSM_E_INVAL;

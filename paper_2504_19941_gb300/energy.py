@@ -3,7 +3,7 @@
 ``FreeEnergy`` evaluates the discrete free energy and its gradient with
 ``dsm_fe_energy_grad`` (FP32 fields, FP64 energy).  ``Energy`` exposes it to
 autograd: the forward pass returns E and keeps the hand-written adjoint dE/dC,
-the backward pass scales it by the incoming gradient (``dsm_vec_axpy_dev``).
+the backward pass scales it by the incoming gradient (``dsm_vec_scale_dev``).
 ``lbfgs`` minimises E over one component with the library's native L-BFGS loop
 (``dsm_lbfgs_minimize``: the compact form of the L-BFGS matrix, a strong-Wolfe
 line search, FP64 dot products; its readings are stated in ``include/dsm.h``).
@@ -32,17 +32,19 @@ class FreeEnergy:
                  energy=None, grad=None):
         """Returns (E as a 1-element float64 device tensor, gradient w.r.t. the
         active field as a float32 device tensor)."""
-        if energy is None:
-            energy = torch.empty(1, dtype=torch.float64, device=self.device)
-        if grad is None:
-            grad = torch.empty(self.n, dtype=torch.float32, device=self.device)
         arg = _lib.tensor_arg
         c1 = arg(c1, self.n, torch.float32, self.device, "c1", copy=True)
         c2 = arg(c2, self.n, torch.float32, self.device, "c2", copy=True)
         if mask is not None:
             mask = arg(mask, self.n, None, self.device, "mask", copy=True, itemsize=1)
-        energy = arg(energy, 1, torch.float64, self.device, "energy")
-        grad = arg(grad, self.n, torch.float32, self.device, "grad")
+        if energy is None:
+            energy = torch.empty(1, dtype=torch.float64, device=self.device)
+        else:
+            energy = arg(energy, 1, torch.float64, self.device, "energy")
+        if grad is None:
+            grad = torch.empty(self.n, dtype=torch.float32, device=self.device)
+        else:
+            grad = arg(grad, self.n, torch.float32, self.device, "grad")
         _lib.dsm_fe_energy_grad(self.params, c1, c2, mask, active, dP, kcs, V0, fg, energy, grad,
                                 self.terms, self.scratch, self.sb, self.stream)
         return energy, grad
@@ -65,8 +67,7 @@ class Energy(torch.autograd.Function):
     def forward(ctx, c_active, c_other, fe: FreeEnergy, active: int = 2, mask=None, dP=0.0,
                 kcs=0.0, V0=0.0, fg=0.0):
         c1, c2 = (c_other, c_active) if active == 2 else (c_active, c_other)
-        E, grad = fe(c1.detach().contiguous(), c2.detach().contiguous(), active=active,
-                     mask=mask, dP=dP, kcs=kcs, V0=V0, fg=fg)
+        E, grad = fe(c1, c2, active=active, mask=mask, dP=dP, kcs=kcs, V0=V0, fg=fg)
         ctx.save_for_backward(grad)
         ctx.fe = fe
         return E.reshape(())
@@ -75,10 +76,8 @@ class Energy(torch.autograd.Function):
     def backward(ctx, gout):
         (grad,) = ctx.saved_tensors
         out = torch.empty_like(grad)
-        n = grad.numel()
-        go = gout.detach().to(torch.float64).reshape(1).contiguous()
-        _lib.dsm_vec_axpby(n, 0.0, grad, 0.0, out, ctx.fe.stream)          # out = 0
-        _lib.dsm_vec_axpy_dev(n, 1.0, go, None, grad, out, ctx.fe.stream)  # out += gout grad
+        go = gout if gout.dtype == torch.float64 else gout.to(torch.float64)
+        _lib.dsm_vec_scale_dev(grad.numel(), go, grad, out, ctx.fe.stream)  # out = gout grad
         return out, None, None, None, None, None, None, None, None
 
 
