@@ -1666,6 +1666,11 @@ inline int mom_zrun(int nx, int ny, int nz, long long resident) {
 }
 
 inline int mom_blocks(long long n) {
+// Several translation units include this file, and each has kernels of its own
+// of the same name and template arguments: what follows is local to the unit,
+// so that an attribute set once is set on the unit's own kernel.
+namespace {
+
   const long long b = (n + 255) / 256;
   return (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
 }
@@ -1872,3 +1877,5 @@ struct MomOps {
 };
 
 }  // namespace dsm
+}  // namespace
+
