@@ -76,6 +76,34 @@ __host__ __device__ constexpr int lat_index(int cx, int cy, int cz) {
   return k;
 }
 
+// A kernel launched so that it may be resident before the kernel ahead of it in
+// the stream ends.  Its blocks call pdl_wait before they touch memory: it returns
+// when the kernel ahead has ended and its writes are visible (which holds for
+// those further ahead too, as each of them waited likewise).  pdl_next lets the
+// next launch become resident in its turn.  What is gained is the gap between
+// dependent launches, not any overlap of the work.
+__device__ __forceinline__ void pdl_next() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       const A &...args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // --------------------------------------------------------------------------
 // Population storage.  For the 16-bit precisions the hydrodynamic population is
 // stored as its offset from the rest weight, f_i - w_i, and the order-parameter

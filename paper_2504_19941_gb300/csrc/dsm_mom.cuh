@@ -1089,6 +1089,8 @@ __global__ void __launch_bounds__(256) mom_solid_kernel(const __grid_constant__ 
     const T v = a.c1[h.plus<L>(i)], w = T(L::w(i));
     lap += w * (v - c1);
     if (L::cx(i)) g[0] += w * T(L::cx(i)) * v;
+  pdl_next();
+  pdl_wait();
     if (L::cy(i)) g[1] += w * T(L::cy(i)) * v;
     if (L::cz(i)) g[2] += w * T(L::cz(i)) * v;
     lk |= (v >= T(0.5) ? 1u : 0u) << i;
@@ -1686,16 +1688,11 @@ struct MomOps {
     } else {
       Mom1<T> m1 = {};
       // small lattices: 64-thread tiles, so that the work spreads over the SMs
-      if ((long long)r.nx * r.ny < 2ll * 152 * 256) {
-        using SM = M2Smem<T, 16, 4>;
-        mom_step2_kernel<T, 16, 4, 2><<<dim3((r.nx + 15) / 16, (r.ny + 3) / 4), dim3(16, 4),
-                                        SM::total, st>>>(mom_typed<T>(r), m1);
-      } else {
-        using SM = M2Smem<T, 32, 8>;
-        mom_step2_kernel<T, 32, 8, 2><<<dim3((r.nx + 31) / 32, (r.ny + 7) / 8), dim3(32, 8),
-                                        SM::total, st>>>(mom_typed<T>(r), m1);
-      }
-      return cudaGetLastError();
+      if ((long long)r.nx * r.ny < 2ll * 152 * 256)
+        return launch_pdl(mom_step2_kernel<T, 16, 4, 2>, dim3((r.nx + 15) / 16, (r.ny + 3) / 4),
+                          dim3(16, 4), M2Smem<T, 16, 4>::total, st, mom_typed<T>(r), m1);
+      return launch_pdl(mom_step2_kernel<T, 32, 8, 2>, dim3((r.nx + 31) / 32, (r.ny + 7) / 8),
+                        dim3(32, 8), M2Smem<T, 32, 8>::total, st, mom_typed<T>(r), m1);
     }
   }
   static int resident() {
@@ -1768,11 +1765,11 @@ struct MomOps {
       } else if (what == 2) {
         mom_relax_c_kernel<T><<<g, b, 0, st>>>(a, m1, (T *)c);
       } else if ((long long)r.nx * r.ny < 2ll * 152 * 256) {
-        mom_step2_kernel<T, 16, 4, 1><<<dim3((r.nx + 15) / 16, (r.ny + 3) / 4), dim3(16, 4),
-                                        M2Smem<T, 16, 4>::total, st>>>(a, m1);
+        return launch_pdl(mom_step2_kernel<T, 16, 4, 1>, dim3((r.nx + 15) / 16, (r.ny + 3) / 4),
+                          dim3(16, 4), M2Smem<T, 16, 4>::total, st, a, m1);
       } else {
-        mom_step2_kernel<T, 32, 8, 1><<<dim3((r.nx + 31) / 32, (r.ny + 7) / 8), dim3(32, 8),
-                                        M2Smem<T, 32, 8>::total, st>>>(a, m1);
+        return launch_pdl(mom_step2_kernel<T, 32, 8, 1>, dim3((r.nx + 31) / 32, (r.ny + 7) / 8),
+                          dim3(32, 8), M2Smem<T, 32, 8>::total, st, a, m1);
       }
       return cudaGetLastError();
     }
@@ -1876,6 +1873,6 @@ struct MomOps {
   }
 };
 
-}  // namespace dsm
 }  // namespace
 
+}  // namespace dsm
