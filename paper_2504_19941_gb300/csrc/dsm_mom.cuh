@@ -1060,6 +1060,8 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
 template <class T, int TX, int TY, int STAGE>
 __global__ void __launch_bounds__(TX *TY)
     mom_step2_kernel(const __grid_constant__ MomArgs<T> a, const __grid_constant__ Mom1<T> m1) {
+  pdl_next();
+  pdl_wait();
   mom_tile2<T, TX, TY, STAGE>(a, m1, blockIdx.x * TX, blockIdx.y * TY, zsm);
 }
 
@@ -1089,8 +1091,6 @@ __global__ void __launch_bounds__(256) mom_solid_kernel(const __grid_constant__ 
     const T v = a.c1[h.plus<L>(i)], w = T(L::w(i));
     lap += w * (v - c1);
     if (L::cx(i)) g[0] += w * T(L::cx(i)) * v;
-  pdl_next();
-  pdl_wait();
     if (L::cy(i)) g[1] += w * T(L::cy(i)) * v;
     if (L::cz(i)) g[2] += w * T(L::cz(i)) * v;
     lk |= (v >= T(0.5) ? 1u : 0u) << i;
