@@ -59,6 +59,10 @@ struct dsm_lattice {
   // represent it; mstepped, mom and stepped since set_fluid
   bool mok, mom, mcp, mstat, mfit, mstepped;
   int mc, mzrun;
+  // single-pass step of D2Q9 (dsm_tile2.cuh): tok, the parameters allow it; tp,
+  // the state is f[cur] and the quads in g[cur ^ 1]; tcan, the canonical copy
+  // of that state (made for reads, which leave the quads valid) is up to date
+  bool tok, tp, tcan;
   // observables ring (dsm_set_observables_ring): caller-owned device records,
   // one appended by dsm_step after each step that is a multiple of ring_every
   double *ring = nullptr;
@@ -280,7 +284,9 @@ cudaError_t z_pack(dsm_lattice *h) {
 
 // Padded state -> canonical g_eq state (A, u planes and C of the last
 // collision), before any call that reads the state in its canonical layout.
+cudaError_t t_copy(dsm_lattice *h);
 cudaError_t z_unpack(dsm_lattice *h) {
+  if (h->tp) return t_copy(h);
   if (!h->zpacked) return cudaSuccess;
   LBRaw a = raw_of(h, h->cur);
   cudaError_t e = h->tab.zunpack(a, h->Qz[h->zc], h->Uz[h->zc], h->Cb[h->cur], h->stream);
@@ -289,10 +295,67 @@ cudaError_t z_unpack(dsm_lattice *h) {
   return cudaSuccess;
 }
 
+// ---- single-pass step of D2Q9 ---------------------------------------------------
+// It applies with tau_g = 1 and faces that are periodic or mirrors (at a wall
+// g would bounce back, which no image node gives), in the automatic forms of g
+// and of the step, where the step on moments does not.
+bool t_eligible(const dsm_params *p) {
+  if (p->lattice != DSM_D2Q9 || p->tau_g != 1.0) return false;
+  const int n[2] = {p->nx, p->ny};
+  for (int a = 0; a < 2; a++) {
+    const int lo = p->face[2 * a], hi = p->face[2 * a + 1];
+    if (lo == DSM_FACE_WALL || hi == DSM_FACE_WALL) return false;
+    if (lo == DSM_FACE_MIRROR && n[a] < 2) return false;  // the halo has two images
+  }
+  return true;
+}
+
+// Canonical planes of a state held as quads: (A, u) in M, C in Cb[cur], and for
+// lattices that keep g as populations (mirrors) those in g[cur].
+cudaError_t t_copy(dsm_lattice *h) {
+  if (h->tcan) return cudaSuccess;
+  LBRaw a = raw_of(h, h->cur ^ 1);  // g_out = g[cur]
+  cudaError_t e = h->tab.tpack(a, h->Cb[h->cur], h->g[h->cur ^ 1], 0, h->stream);
+  if (e == cudaSuccess && !h->eq) {
+    a.Cprev = h->Cb[h->cur];
+    e = h->tab.materialize(a, h->stream);
+  }
+  if (e != cudaSuccess) return e;
+  h->g_implicit = h->eq;
+  h->tcan = true;
+  return cudaSuccess;
+}
+
+// One step of a lattice in this form.  A state given as populations takes its
+// first step in two passes, which leave (A, u) and C.
+cudaError_t t_step(dsm_lattice *h) {
+  LBRaw a = raw_of(h, h->cur);
+  cudaError_t e = cudaSuccess;
+  if (!h->tp && !h->g_implicit) {
+    a.eq = 1;
+    e = h->tab.moments(a, h->stream);
+    if (e == cudaSuccess) e = h->tab.node(a, 2, MODE_STEP, h->stream);
+    if (e == cudaSuccess) e = h->tab.tpack(a, h->Cb[h->cur ^ 1], h->g[h->cur], 1, h->stream);
+  } else {
+    if (!h->tp) e = h->tab.tpack(a, h->Cb[h->cur], h->g[h->cur ^ 1], 1, h->stream);
+    a.Qz = h->g[h->cur];
+    if (e == cudaSuccess) e = h->tab.tstep(a, h->g[h->cur ^ 1], h->stream);
+  }
+  if (e != cudaSuccess) return e;
+  h->tp = true;
+  h->tcan = false;
+  return cudaSuccess;
+}
+
 // ---- step on moments ----------------------------------------------------------
-// It applies to FP32 and FP64 lattices with every relaxation time 1, equal
-// densities and periodic faces, whatever their size, in the automatic storage
-// form of g; dsm_set_step_form chooses one pass or two.
+// It applies to lattices with every relaxation time 1, equal densities and
+// periodic faces in the automatic storage form of g: FP32 and FP64 ones of any
+// size, and those with 16-bit populations where the padded buffers of the
+// population form's single pass exist (3D, nx >= 32, ny >= 8), in whose place
+// the solid's data goes.  dsm_set_step_form chooses one pass or two.  With
+// 16-bit populations the moments are FP32 reals all the same: 36 B per node are
+// fewer than the 38 B of the populations and the 20 B of (A, C, u) that they
+// replace, and nothing is rounded to 16 bits any more.
 bool m_eligible(const dsm_params *p) {
   return (p->precision == DSM_F32 || p->precision == DSM_F64) && p->tau2 == 1.0 &&
          p->tau3 == 1.0 && p->tau_g == 1.0 && p->rho2 == p->rho3 && !has_walls(p);
@@ -368,7 +431,7 @@ cudaError_t m_leave(dsm_lattice *h) {
 }
 
 // A new state arrives by other means.
-void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mstat = h->mfit = false; }
+void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mstat = h->mfit = h->tp = h->tcan = false; }
 
 // C of the next step of a state held as moments, into Cb[0].
 cudaError_t m_c(dsm_lattice *h) {
@@ -389,6 +452,10 @@ cudaError_t m_enter(dsm_lattice *h) {
   h->mstepped = true;
   h->mcp = false;
   return cudaSuccess;
+}
+
+bool t_active(const dsm_lattice *h) {
+  return h->tok && !m_active(h) && h->g_form == DSM_G_AUTO && h->step_form == DSM_STEP_AUTO;
 }
 
 int m_zrun(dsm_lattice *h) {
@@ -645,6 +712,7 @@ dsm_status dsm_create(const dsm_params *p, void *d_workspace, size_t bytes, void
   h->g_form = DSM_G_AUTO;
   h->eq = p->tau_g == 1.0 && !has_walls(p);
   h->mok = m_eligible(p) && t.mom_step;
+  h->tok = t_eligible(p) && t.tstep;
   // no solid yet: C1 = 0 everywhere; clear the error word and the mask
   cudaError_t e = cudaMemsetAsync(h->C1, 0, pitch * t.real_bytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->mask, 0, pitch, h->stream);
@@ -773,8 +841,8 @@ dsm_status dsm_step(dsm_lattice *h, long long nsteps) {
   TraceRange trace_range("dsm_step");
   if (!h || nsteps < 0) return DSM_E_INVAL;
   if (!h->has_fluid || h->latched) return DSM_E_STATE;
-  const bool mom = m_active(h), single = !mom && z_active(h);
-  if (!single && z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  const bool mom = m_active(h), single = !mom && z_active(h), tile = t_active(h);
+  if (!single && !tile && z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
   if (!mom && m_leave(h) != cudaSuccess) return DSM_E_CUDA;
   for (long long t = 0; t < nsteps; t++) {
     cudaError_t e;
@@ -791,7 +859,10 @@ dsm_status dsm_step(dsm_lattice *h, long long nsteps) {
       e = h->tab.zstep(a, h->maps[h->zc], h->zrun > 0 ? h->zrun : z_auto_run(h), h->stream);
       if (e != cudaSuccess) return DSM_E_CUDA;
       h->zc ^= 1;
+    } else if (tile) {
+      if (t_step(h) != cudaSuccess) return DSM_E_CUDA;
     } else {
+      h->tp = h->tcan = false;
       // moments pass, then the fused pass (also the first step of a state given
       // as populations)
       LBRaw a = raw_of(h, h->cur);
@@ -900,6 +971,7 @@ dsm_status dsm_step_collide(dsm_lattice *h) {
   }
   LBRaw a = raw_of(h, h->cur);
   if (h->tab.node(a, 2, MODE_STEP, h->stream) != cudaSuccess) return DSM_E_CUDA;
+  h->tp = h->tcan = false;
   h->cur ^= 1;
   h->step++;
   h->g_implicit = h->eq;
@@ -1001,6 +1073,7 @@ dsm_status dsm_set_g_storage(dsm_lattice *h, int form) {
   const bool eq = form == DSM_G_AUTO && h->prm.tau_g == 1.0 && !has_walls(&h->prm);
   if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
   if (!eq && m_leave(h) != cudaSuccess) return DSM_E_CUDA;
+  if (form == DSM_G_POPULATIONS) h->tp = h->tcan = false;  // (the canonical copy is the state)
   if (h->g_implicit && !eq) {
     // write the current g_eq out as populations of the current buffer
     LBRaw a = raw_of(h, h->cur ^ 1);  // g_out = current buffer
@@ -1025,8 +1098,9 @@ dsm_status dsm_get_g_storage(dsm_lattice *h, int *form, int *implicit_now) {
 // Raw state (checkpoint): a 256-byte header, then the current buffer's f, g,
 // 16-bit g_0, C of the last collision and the g_eq planes, each region
 // 256-byte aligned; a state held as moments (implicit = 2) has them in the
-// place of f, and the density they belong to in the header.  Restoring it
-// continues the run bitwise.
+// place of f, and the density they belong to in the header; one held as f and
+// quads (implicit = 3) has the quads in the place of g.  Restoring it continues
+// the run bitwise.
 namespace {
 constexpr unsigned kStateMagic = 0x53534d44u;  // "DSMS"
 struct StateHeader {
@@ -1068,7 +1142,7 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
   if (!h->has_fluid) return DSM_E_STATE;
   const StateLayout L = state_layout(h);
   if (bytes < L.total || ((uintptr_t)d_dst & 255u)) return DSM_E_WORKSPACE;
-  if (z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
+  if (!h->tp && z_unpack(h) != cudaSuccess) return DSM_E_CUDA;
   StateHeader hd;
   memset(&hd, 0, sizeof(hd));
   hd.magic = kStateMagic;
@@ -1078,7 +1152,7 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
   hd.nx = h->prm.nx;
   hd.ny = h->prm.ny;
   hd.nz = h->prm.nz;
-  hd.implicit = h->mom ? 2 : h->g_implicit ? 1 : 0;
+  hd.implicit = h->mom ? 2 : h->tp ? 3 : h->g_implicit ? 1 : 0;
   hd.rho = h->sp.rho3;
   hd.step = h->step;
   hd.pitch = h->pitch;
@@ -1095,6 +1169,12 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
     return cuda_status(e);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + L.f, h->f[h->cur], pop, cudaMemcpyDeviceToDevice, st);
+  if (h->tp) {
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(d + L.g, h->g[h->cur ^ 1], 4 * real, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return cuda_status(e);
+  }
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + L.g, h->g[h->cur], pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && h->tab.k16)
     e = cudaMemcpyAsync(d + L.g0, h->g0[h->cur], h->pitch * sizeof(float), cudaMemcpyDeviceToDevice, st);
@@ -1116,7 +1196,8 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
   if (e != cudaSuccess) return DSM_E_CUDA;
   if (hd.magic != kStateMagic || hd.version != 1 || hd.lattice != h->kind ||
       hd.precision != h->prm.precision || hd.nx != h->prm.nx || hd.ny != h->prm.ny ||
-      hd.nz != h->prm.nz || hd.pitch != h->pitch || hd.implicit < 0 || hd.implicit > 2 ||
+      hd.nz != h->prm.nz || hd.pitch != h->pitch || hd.implicit < 0 || hd.implicit > 3 ||
+      (hd.implicit == 3 && !h->tok) ||
       (hd.implicit == 2 && (h->tab.k16 || !(hd.rho > 0.0))) || hd.step < 0)
     return DSM_E_INVAL;
   const char *d = (const char *)d_src;
@@ -1149,6 +1230,20 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
     return DSM_OK;
   }
   e = cudaMemcpyAsync(h->f[0], d + L.f, pop, cudaMemcpyDeviceToDevice, st);
+  if (hd.implicit == 3) {
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->g[1], d + L.g, 4 * real, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, st);
+    if (e != cudaSuccess) return DSM_E_CUDA;
+    h->tp = true;
+    h->step = hd.step;
+    h->g_implicit = h->eq;
+    h->zpacked = false;
+    h->has_fluid = true;
+    h->latched = false;
+    h->moments_ready = false;
+    return DSM_OK;
+  }
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->g[0], d + L.g, pop, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && h->tab.k16)
     e = cudaMemcpyAsync(h->g0[0], d + L.g0, h->pitch * sizeof(float), cudaMemcpyDeviceToDevice, st);
@@ -1417,6 +1512,7 @@ dsm_status dsm_batch_step(dsm_lattice *const *hs, int n, const long long *nsteps
       h->mcp = false;
       h->mstepped = true;
     } else {
+      h->tp = h->tcan = false;
       h->cur ^= (int)(left[i] & 1);
       h->g_implicit = h->eq;
       h->mfit = h->mok && h->eq;

@@ -328,7 +328,11 @@ struct LBTable {
   cudaError_t (*zpack)(const LBRaw &r, void *Qz0, void *Qz1, void *Uz0, void *Uz1, void *C1z,
                        cudaStream_t);
   cudaError_t (*zunpack)(const LBRaw &r, const void *Qz, const void *Uz, void *Cout, cudaStream_t);
-  // step on moments (FP32 and FP64; null for 16-bit storage): one step with
+  // single-pass step of D2Q9 (dsm_tile2.cuh; null in 3D): one step from the
+  // quads qin into r.Qz; the quads from (pack) or into r.M and C
+  cudaError_t (*tstep)(const LBRaw &r, const void *qin, cudaStream_t);
+  cudaError_t (*tpack)(const LBRaw &r, void *C, void *q, int pack, cudaStream_t);
+  // step on moments (null for 16-bit storage in 2D): one step with
   // zrun planes per block (3D), its resident blocks per SM, the two passes (C
   // of the step, then the rest: step, field or observables), and the
   // conversions around it

@@ -460,12 +460,31 @@ __global__ void __launch_bounds__(256) moments_eq_kernel(LBArgs<T, S> a) {
 // a collision of the g_eq form stores what fixes g (A = mu - 3/2 C u.u, u):
 // global memory, as the per-lattice and batched launches keep them.  The
 // single-pass step (dsm_zstep.cuh) reads both from shared memory instead.
+// Density map rho = rho3 + (rho2 - rho3) C2/(C2 + C3), the ratio clamped to
+// [0, 1] and 0 where C2 + C3 = 1 - C1 <= 1e-6 (inside the solid).  (FP32: the
+// volume fraction, clamped to [0, 1] right after, needs no correctly rounded
+// quotient -- the fast reciprocal-and-multiply division, within 2 ulp, replaces
+// a full IEEE division.)
+template <class T>
+__device__ __forceinline__ T rho_map(const ConstT<T> &K_, T cc, T s1) {
+  const T den = T(1) - s1;
+  T ph = T(0);
+  if (den > T(1e-6)) {
+    if constexpr (sizeof(T) == 4) ph = __fdividef(cc, den);
+    else ph = cc / den;
+    ph = ph < T(0) ? T(0) : (ph > T(1) ? T(1) : ph);
+  }
+  return K_.rho3 + K_.drho * ph;
+}
+
 struct GlobalIO {
   // wall links fixed in one rolled loop (fewer registers next to the
   // neighbourhood loads in flight); the f pulls of a solid node are issued
   // with the rest, before its C1 is known
   static constexpr bool kUnrollWall = false;
   static constexpr bool kSolidFirst = false;
+  static constexpr bool kFetched = false;  // io.f holds the pulled f
+  static constexpr bool kRho = false;      // io.rho gives the neighbours' densities
   template <class L, class T, class S>
   __device__ __forceinline__ T C(const LBArgs<T, S> &a, const Hood &h, int i) const {
     return __ldg(a.C + h.plus<L>(i));
@@ -500,7 +519,7 @@ __device__ __forceinline__ void node_body(const LBArgs<T, S> &a, int x, int y, i
   // the pulled g enter only the g collision (C comes from the moments pass)
   constexpr bool LOAD_G = MODE == MODE_STEP && !EQ;
   static_assert(!EQ || STAGE == 2, "g as g_eq is a stage-2 form");
-  static_assert(!(EQ && FC), "g as g_eq implies periodic faces");
+  static_assert(!(EQ && FC) || K == 0, "g as g_eq: periodic faces, or mirrors in 2D");
   if (MODE != MODE_OBS && !valid) return;
   if (!valid) x = y = z = 0;
   Hood h;
@@ -531,7 +550,8 @@ __device__ __forceinline__ void node_body(const LBArgs<T, S> &a, int x, int y, i
       if (!LOAD_G) g[j] = T(0);
       else if (Store<S>::k16 && j == 0) g[j] = T(a.g0_in[n]);
       else g[j] = load_g<T, S>(a.gin[j], src);
-      if constexpr (IO::kSolidFirst) f[j] = T(L::w(j));
+      if constexpr (IO::kFetched) f[j] = io.f[j];
+      else if constexpr (IO::kSolidFirst) f[j] = T(L::w(j));
       else f[j] = load_f<T, S>(a.fin[j], src, j, L::w(j));
     }
     // the pulled f of a solid node (C1 >= 1/2) are never used: its collision
@@ -574,26 +594,33 @@ __device__ __forceinline__ void node_body(const LBArgs<T, S> &a, int x, int y, i
       // Eq. [eqn:fefrozen]), taken as its exact derivative in C2:
       //   mu = k2 b(C) + k3 b(C1 + C) - a^2 k2 L[C] - a^2 k3 L[C1 + C]
       mu = K_.k2 * bwell(C) + K_.k3 * bwell(c1 + C) - K_.a2k2 * lapC - K_.a2k3 * lapS;
-      // density map rho = rho3 + (rho2 - rho3) C2/(C2 + C3), the ratio clamped
-      // to [0, 1] and 0 where C2 + C3 = 1 - C1 <= 1e-6 (inside the solid)
-      // (FP32: the volume fraction, clamped to [0, 1] right after, needs no
-      // correctly rounded quotient -- the fast reciprocal-and-multiply division,
-      // within 2 ulp, replaces a full IEEE division at every neighbour)
-      auto rho_of = [&](T cc, T s1) -> T {
-        const T den = T(1) - s1;
-        T ph = T(0);
-        if (den > T(1e-6)) {
-          if constexpr (sizeof(T) == 4) ph = __fdividef(cc, den);
-          else ph = cc / den;
-          ph = ph < T(0) ? T(0) : (ph > T(1) ? T(1) : ph);
+      // density: where the node's view has it, each node's rho was formed once
+      // (kRho); else at every neighbour here
+      rho = K_.rho3;
+      if constexpr (RC && IO::kRho) {
+        // differences of opposite neighbours, of C and of rho as one pair
+        Pr<T> gx = pr(T(0), T(0)), gy = gx, gz = gx;
+        rho = io.template rho<L>(0);
+#pragma unroll
+        for (int i = 1; i < Q; i += 2) {
+          const T w = T(L::w(i));
+          const Pr<T> d = pr_fma(pr(Cn[i + 1], io.template rho<L>(i + 1)), pr(T(-1), T(-1)),
+                                 pr(Cn[i], io.template rho<L>(i)));
+          if (L::cx(i)) gx = pr_fma(pr(w * T(L::cx(i)), w * T(L::cx(i))), d, gx);
+          if (L::cy(i)) gy = pr_fma(pr(w * T(L::cy(i)), w * T(L::cy(i))), d, gy);
+          if (L::cz(i)) gz = pr_fma(pr(w * T(L::cz(i)), w * T(L::cz(i))), d, gz);
         }
-        return K_.rho3 + K_.drho * ph;
-      };
-      rho = RC ? rho_of(C, c1) : K_.rho3;
-      if (RC) {
+        gC[0] = T(3) * gx.a;
+        gC[1] = T(3) * gy.a;
+        gC[2] = T(3) * gz.a;
+        gR[0] = T(3) * gx.b;
+        gR[1] = T(3) * gy.b;
+        gR[2] = T(3) * gz.b;
+      } else if constexpr (RC) {
+        rho = rho_map(K_, C, c1);
 #pragma unroll
         for (int i = 1; i < Q; i++) {
-          const T r = T(L::w(i)) * rho_of(Cn[i], C1n[i]);
+          const T r = T(L::w(i)) * rho_map(K_, Cn[i], C1n[i]);
           if (L::cx(i)) gR[0] += r * T(L::cx(i));
           if (L::cy(i)) gR[1] += r * T(L::cy(i));
           if (L::cz(i)) gR[2] += r * T(L::cz(i));
@@ -1215,6 +1242,7 @@ inline dim3 lb_grid(int kind, int nx, int ny, int nz) {
 }  // namespace dsm
 
 #include "dsm_mom.cuh"
+#include "dsm_tile2.cuh"
 
 namespace dsm {
 
@@ -1325,8 +1353,9 @@ struct LBOps {
   }
   template <int STAGE, int MODE, bool EQ = false>
   static void node_launch(const LBRaw &r, cudaStream_t st) {
-    // (g held as g_eq implies periodic faces)
-    if (!EQ && r.p.walls) node_launch_fc<STAGE, MODE, false, true>(r, st);
+    // (g held as g_eq implies periodic faces; a 2D step can give it with mirrors)
+    if (EQ && K == 0 && r.p.walls) node_launch_fc<STAGE, MODE, EQ, K == 0 || !EQ>(r, st);
+    else if (!EQ && r.p.walls) node_launch_fc<STAGE, MODE, false, true>(r, st);
     else node_launch_fc<STAGE, MODE, EQ, false>(r, st);
   }
   static cudaError_t node(const LBRaw &r, int stage, int mode, cudaStream_t st) {
@@ -1499,8 +1528,35 @@ struct LBOps {
       return cudaGetLastError();
     }
   }
+  static cudaError_t tstep(const LBRaw &r, const void *qin, cudaStream_t st) {
+    if constexpr (K != 0) {
+      return cudaErrorNotSupported;
+    } else {
+      // small lattices: 64-thread tiles, so that the work spreads over the SMs
+      if ((long long)r.nx * r.ny < 2ll * 152 * 256) return tstep_tile<16, 4>(r, qin, st);
+      return tstep_tile<32, 8>(r, qin, st);
+    }
+  }
+  template <int TX, int TY>
+  static cudaError_t tstep_tile(const LBRaw &r, const void *qin, cudaStream_t st) {
+    const dim3 g((r.nx + TX - 1) / TX, (r.ny + TY - 1) / TY), b(TX, TY);
+    const int mx = r.p.face[0] != 0, my = r.p.face[2] != 0;
+    const auto k = r.p.rho_contrast
+                       ? (r.p.walls ? tile2_kernel<T, S, TX, TY, true, true>
+                                    : tile2_kernel<T, S, TX, TY, true, false>)
+                       : (r.p.walls ? tile2_kernel<T, S, TX, TY, false, true>
+                                    : tile2_kernel<T, S, TX, TY, false, false>);
+    return launch_pdl(k, g, b, 0, st, typed<T, S>(r), (const T *)qin, mx, my);
+  }
+  static cudaError_t tpack(const LBRaw &r, void *C, void *q, int pack, cudaStream_t st) {
+    const int blocks = (int)((r.N + 255) / 256 < 152 * 16 ? (r.N + 255) / 256 : 152 * 16);
+    tile2_pack_kernel<T><<<blocks, 256, 0, st>>>(r.N, r.pitch, (T *)r.M, (T *)C, (T *)q, pack);
+    return cudaGetLastError();
+  }
   static LBTable table() {
     LBTable t;
+    t.tstep = K == 0 ? &tstep : nullptr;
+    t.tpack = &tpack;
     t.zstep = &zstep;
     t.zresident = &zresident;
     t.zpack = &zpack;

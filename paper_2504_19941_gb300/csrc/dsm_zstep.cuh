@@ -144,6 +144,8 @@ template <class T>
 struct ZIO {
   static constexpr bool kUnrollWall = true;
   static constexpr bool kSolidFirst = true;
+  static constexpr bool kFetched = false;
+  static constexpr bool kRho = false;
   unsigned co[3], c1o[3];
   int x, y, z;
   template <class L, class T_, class S>
