@@ -357,16 +357,19 @@ cudaError_t t_step(dsm_lattice *h) {
 // fewer than the 38 B of the populations and the 20 B of (A, C, u) that they
 // replace, and nothing is rounded to 16 bits any more.
 bool m_eligible(const dsm_params *p) {
-  return (p->precision == DSM_F32 || p->precision == DSM_F64) && p->tau2 == 1.0 &&
-         p->tau3 == 1.0 && p->tau_g == 1.0 && p->rho2 == p->rho3 && !has_walls(p);
+  const bool k16 = p->precision != DSM_F32 && p->precision != DSM_F64;
+  return (!k16 || z_eligible(p)) && p->tau2 == 1.0 && p->tau3 == 1.0 && p->tau_g == 1.0 &&
+         p->rho2 == p->rho3 && !has_walls(p);
 }
 bool m_active(const dsm_lattice *h) {
   return h->mok && h->eq;
 }
 
 // The moments use buffers the g_eq form leaves idle: buffer b in g[b]; the
-// solid's pairs and link bits behind them, its link fractions in f[0].  The
-// canonical copy of a state held as moments goes to buffer 1.
+// solid's pairs and link bits behind them, its link fractions in f[0].  With
+// 16-bit populations the fractions take f[0] and f[1] (72 of 76 B per node), the
+// wall sums Qz[0], the solid's pairs, link bits and list Qz[1].  The canonical
+// copy of a state held as moments goes to buffer 1 (and ends the solid's data).
 MomRaw m_raw(const dsm_lattice *h, int src) {
   MomRaw r;
   memset(&r, 0, sizeof(r));
@@ -392,6 +395,12 @@ MomRaw m_raw(const dsm_lattice *h, int src) {
   if (h->kind == DSM_D3Q19) {
     r.list = (char *)r.lk + plane;
     r.wall = (char *)r.sol + 2 * plane;
+    if (h->tab.k16 && h->zok) {
+      r.wall = h->Qz[0];
+      r.sol = h->Qz[1];
+      r.lk = (char *)h->Qz[1] + 2 * plane;
+      r.list = (char *)h->Qz[1] + 3 * plane;
+    }
   }
   r.c1 = h->C1;
   r.err = h->err;
@@ -402,6 +411,7 @@ MomRaw m_raw(const dsm_lattice *h, int src) {
   r.rho = h->sp.rho3;
   for (int a = 0; a < 3; a++) r.body[a] = h->sp.body[a];
   r.alpha_s = h->sp.alpha_s;
+  r.step = (unsigned)h->step;
   return r;
 }
 
@@ -1198,7 +1208,7 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
       hd.precision != h->prm.precision || hd.nx != h->prm.nx || hd.ny != h->prm.ny ||
       hd.nz != h->prm.nz || hd.pitch != h->pitch || hd.implicit < 0 || hd.implicit > 3 ||
       (hd.implicit == 3 && !h->tok) ||
-      (hd.implicit == 2 && (h->tab.k16 || !(hd.rho > 0.0))) || hd.step < 0)
+      (hd.implicit == 2 && (!h->tab.mom_expand || !(hd.rho > 0.0))) || hd.step < 0)
     return DSM_E_INVAL;
   const char *d = (const char *)d_src;
   const size_t pop = (size_t)h->q * h->pitch * h->tab.store_bytes;

@@ -290,6 +290,7 @@ struct MomRaw {
   const void *c1;
   int *err;
   double k[3], ak[3], kl, akl, rho, body[3], alpha_s;
+  unsigned step;  // steps taken so far
 };
 // canonical planes of a state: f, A, u, C (pitch apart), or populations f and
 // g (N apart, in C)

@@ -1572,7 +1572,9 @@ struct LBOps {
     t.materialize = &materialize;
     t.mom_step = nullptr;
     t.mom_relax = nullptr;
-    if constexpr (!Store<S>::k16) MomOps<K, T>::table(t);
+    t.mom_expand = nullptr;
+    // (16-bit storage in 2D has no room for the moments)
+    if constexpr (!Store<S>::k16 || K == 1) MomOps<K, T, 1, S>::table(t);
     t.q = Lat<K>::Q;
     t.real_bytes = sizeof(T);
     t.store_bytes = sizeof(S);
