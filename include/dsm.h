@@ -224,9 +224,12 @@ dsm_status dsm_set_body_force(dsm_lattice *h, const double *body);
 enum { DSM_STEP_AUTO = 0, DSM_STEP_TWO_PASS = 1 };
 dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun);
 
-/* Whether dsm_step currently runs the one-pass step (*single_pass = 1) and
- * with how many z planes per block (*zrun; 0 for the two-pass step).  Either
- * pointer may be NULL. */
+/* Whether the one-pass step applies to the lattice's size, form and faces
+ * (*single_pass = 1) and with how many z planes per block (*zrun; 0 for the
+ * two-pass step).  The automatic form takes the fastest kernels for the same
+ * step where others are faster: moments in the place of populations where every
+ * relaxation time is 1, two passes with a density contrast in FP32 arithmetic.
+ * Either pointer may be NULL. */
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun);
 
 /* Observables of the current state; synchronises the stream.  Returns

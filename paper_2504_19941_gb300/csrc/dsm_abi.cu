@@ -267,8 +267,17 @@ int z_auto_run(dsm_lattice *h) {
   return run;
 }
 
-bool z_active(const dsm_lattice *h) {
+bool z_form(const dsm_lattice *h) {
   return h->zok && h->eq && h->step_form == DSM_STEP_AUTO;
+}
+// In FP32 arithmetic with a density contrast two passes are the faster form of
+// the automatic step: rho at a node's 18 neighbours, each a quotient, leaves the
+// single pass out of issue slots with 24 warps per SM (250 x 130 x 101: 303 us per
+// step, 184 + 45 in two passes; rho planes formed once per node in shared memory
+// spilled, 378 us, and as a plane of the moments pass changed nothing, 181 + 52).
+// FP64, bound by its pipe, keeps the single pass.
+bool z_active(const dsm_lattice *h) {
+  return z_form(h) && !(h->sp.rho_contrast && h->tab.real_bytes == 4);
 }
 
 // Canonical g_eq state -> padded buffers (buffer 0), and padded C1.
@@ -944,7 +953,7 @@ dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun) {
 
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun) {
   if (!h) return DSM_E_INVAL;
-  const bool single = z_active(h);
+  const bool single = z_form(h);
   if (single_pass) *single_pass = single ? 1 : 0;
   if (zrun) *zrun = single ? (h->zrun > 0 ? h->zrun : m_active(h) ? m_zrun(h) : z_auto_run(h)) : 0;
   return DSM_OK;
