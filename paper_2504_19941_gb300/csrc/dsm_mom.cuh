@@ -54,9 +54,11 @@ struct MomArgs {
   long long N, pitch;
   MomBuf<T> in, out;
   const T *sol;        // pairs (C1, L[C1]) of the frozen solid
-  const unsigned *lk;  // bit i: x + c_i is solid (fluid nodes next to the solid; else 0)
+  // of the nodes next to the solid, by node in 2D (lk: 0 elsewhere), in the order of
+  // list in 3D:
+  const unsigned *lk;  // bit i: x + c_i is solid
   const T *qpl;        // plane j - 1: link fraction of the wall link pulled in direction j
-  const unsigned char *near;  // 3D: lk != 0
+  const unsigned char *near;  // 3D: next to the solid
   unsigned *list;      // 3D: the nodes next to the solid, their count
   int *count;
   T *wall;             // 3D: quads, what their wall links add to (S, M)
@@ -200,16 +202,20 @@ __device__ __forceinline__ void mom_walls(const MomArgs<T> &a, unsigned lk, long
 // 3D: the wall sums of every node next to the solid, ahead of the step.  In the
 // step itself a wall node's loads (its link fractions, then the far nodes) would
 // follow one another while its block waits at the plane's barrier.  Here a
-// thread has all of a node's loads of one kind in flight: the link fractions
-// of nine links, then the moments at the far end of each (at the node itself
-// where the link needs none).
+// thread has all of a node's loads of one kind in flight: its index, link bits and
+// the fractions of all its links (which lie in the order of the list: 1/2 where
+// there is no link), then the node's moments and those at the far end of nine
+// links each (at the node itself where the link needs none).
 template <class T>
 __device__ __forceinline__ void mom_wall_nodes(const MomArgs<T> &a, int first, int stride) {
   using L = Lat<1>;
   const int cnt = *a.count;
   for (int k = first; k < cnt; k += stride) {
     const int n = chk(a.err, (int)a.list[k], a.N);
-    const unsigned lk = a.lk[n];
+    const unsigned lk = a.lk[k];
+    T q[L::Q - 1];
+#pragma unroll
+    for (int j = 1; j < L::Q; j++) q[j - 1] = a.qpl[(long long)(j - 1) * a.pitch + k];
     const MomNode<T> own = mom_load<L>(a.in, n);
     const int x = n % a.nx, y = n / a.nx % a.ny, z = n / (a.nx * a.ny);
     Hood h;
@@ -218,22 +224,16 @@ __device__ __forceinline__ void mom_wall_nodes(const MomArgs<T> &a, int first, i
     T S = T(0), M[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int j0 = 1; j0 < L::Q; j0 += 9) {
-      T q[9];
       MomNode<T> far[9];
 #pragma unroll
       for (int e = 0; e < 9; e++) {
         const int j = j0 + e;
-        q[e] = (lk >> L::opp(j)) & 1u ? a.qpl[(long long)(j - 1) * a.pitch + n] : T(0.5);
-      }
-#pragma unroll
-      for (int e = 0; e < 9; e++) {
-        const int j = j0 + e;
-        far[e] = mom_load<L>(a.in, q[e] < T(0.5) && !((lk >> j) & 1u) ? h.plus<L>(j) : n);
+        far[e] = mom_load<L>(a.in, q[j - 1] < T(0.5) && !((lk >> j) & 1u) ? h.plus<L>(j) : n);
       }
 #pragma unroll
       for (int e = 0; e < 9; e++) {
         const int j = j0 + e, i = L::opp(j);
-        if ((lk >> i) & 1u) mom_wall_add<L>(a, lk, j, q[e], own, far[e], S, M);
+        if ((lk >> i) & 1u) mom_wall_add<L>(a, lk, j, q[j - 1], own, far[e], S, M);
       }
     }
     Quad<T> r;
@@ -1129,10 +1129,15 @@ __global__ void __launch_bounds__(256) mom_solid_kernel(const __grid_constant__ 
   s.v[0] = c1;
   s.v[1] = T(6) * lap;
   reinterpret_cast<Duo<T> *>(const_cast<T *>(a.sol))[n] = s;
-  const_cast<unsigned *>(a.lk)[n] = lk;
-  if (K == 1) const_cast<unsigned char *>(a.near)[n] = lk != 0;
+  if (K == 0) const_cast<unsigned *>(a.lk)[n] = lk;
+  else const_cast<unsigned char *>(a.near)[n] = lk != 0;
   if (!lk) return;
-  if (K == 1) a.list[atomicAdd(a.count, 1)] = n;
+  int k = n;
+  if (K == 1) {
+    k = atomicAdd(a.count, 1);
+    a.list[k] = n;
+    const_cast<unsigned *>(a.lk)[k] = lk;
+  }
 #pragma unroll
   for (int d = 0; d < 3; d++) g[d] *= T(3);
   const T cc = c1 < T(1e-9) ? T(1e-9) : c1;
@@ -1141,9 +1146,10 @@ __global__ void __launch_bounds__(256) mom_solid_kernel(const __grid_constant__ 
 #pragma unroll
   for (int j = 1; j < Q; j++) {
     const int i = L::opp(j);
-    if ((lk >> i) & 1u)
-      const_cast<T *>(a.qpl)[(long long)(j - 1) * a.pitch + n] =
-          link_fraction<L, T>(xs, gn, g[0], g[1], g[2], i);
+    const bool link = (lk >> i) & 1u;
+    if (link || K == 1)
+      const_cast<T *>(a.qpl)[(long long)(j - 1) * a.pitch + k] =
+          link ? link_fraction<L, T>(xs, gn, g[0], g[1], g[2], i) : T(0.5);
   }
 }
 
@@ -1290,10 +1296,19 @@ __global__ void __launch_bounds__(256)
   T M[3];
 #pragma unroll
   for (int e = 0; e < 3; e++) M[e] = fm(T(L::w(1)), Ma[e], ml(T(L::w(L::Q - 1)), Md[e]));
-  const unsigned lk = a.lk[n];
-  if (lk)
-    mom_walls<L>(
-        a, lk, n, [&](int j) { return mom_load<L>(a.in, j == 0 ? n : h.plus<L>(j)); }, S, M);
+  if constexpr (K == 1) {  // summed ahead (mom_wall_nodes)
+    if (a.near[n]) {
+      const Quad<T> w = reinterpret_cast<const Quad<T> *>(a.wall)[n];
+      S = ad(S, w.v[0]);
+#pragma unroll
+      for (int e = 0; e < 3; e++) M[e] = ad(M[e], w.v[1 + e]);
+    }
+  } else {
+    const unsigned lk = a.lk[n];
+    if (lk)
+      mom_walls<L>(
+          a, lk, n, [&](int j) { return mom_load<L>(a.in, j == 0 ? n : h.plus<L>(j)); }, S, M);
+  }
   const MomOut<T, NF> o = mom_collide<L::D, T, NF>(a, s.v[0], s.v[1], C, lap, g, S, M);
   const bool solid = s.v[0] >= T(0.5);
   if constexpr (MODE == MODE_STEP) {
@@ -1780,6 +1795,7 @@ struct MomOps {
     const MomArgs<T> a = mom_typed<T>(r);
     const T *c = (const T *)cn;
     T *o = (T *)fields;
+    if (K == 1) mom_wall_kernel<T><<<152 * 8, 128, 0, st>>>(a);
     if (mode == MODE_STEP)
       mom_node_kernel<K, T, NF, MODE_STEP><<<g, b, 0, st>>>(a, c, cstride, o, field, index, partials);
     else if (mode == MODE_FIELDS)
