@@ -246,7 +246,9 @@ __device__ __forceinline__ void mom_wall_nodes(const MomArgs<T> &a, int first, i
 }
 template <class T>
 __global__ void __launch_bounds__(128) mom_wall_kernel(const __grid_constant__ MomArgs<T> a) {
+  pdl_wait();
   mom_wall_nodes(a, blockIdx.x * 128 + threadIdx.x, gridDim.x * 128);
+  pdl_next();
 }
 
 // mu, F and the new moments of one node from this step's C, its stencils and
@@ -805,8 +807,10 @@ template <class T, int NF, int TY, int RY, int BPS, bool DI>
 __global__ void __launch_bounds__(M3_X *TY / RY, sizeof(T) == 8 ? 1 : BPS)
     mom_step3_kernel(const __grid_constant__ MomArgs<T> a, int zrun) {
   const int z0 = blockIdx.z * zrun;
+  pdl_wait();
   mom_run3<T, NF, TY, RY, DI>(a, blockIdx.x * M3_X, blockIdx.y * TY, z0, min(z0 + zrun, a.nz),
                               a.step, zsm);
+  pdl_next();
 }
 
 // ---------------------------------------------------------------------------
@@ -1707,10 +1711,14 @@ struct Mom3 {
   static cudaError_t step(const MomRaw &r, int zrun, cudaStream_t st) {
     if (!prepare() || zrun < 1) return cudaErrorInvalidValue;
     const MomArgs<T> a = mom_typed<T>(r);
-    mom_wall_kernel<T><<<152 * 8, 128, 0, st>>>(a);
-    kernel()<<<dim3((r.nx + M3_X - 1) / M3_X, (r.ny + TY - 1) / TY, (r.nz + zrun - 1) / zrun),
-               dim3(M3_X, TY / RY), M3Smem<T, NF, TY>::total, st>>>(a, zrun);
-    return cudaGetLastError();
+    // Each lets the next launch in when its blocks are done (pdl_next at their end):
+    // 101^3 46.3 -> 42.1 us per step, 256 x 256 x 192 279 -> 275.  Let in at their
+    // start, the next launch's blocks took SM space from those still to run (51.1).
+    const cudaError_t e = launch_pdl(mom_wall_kernel<T>, dim3(152 * 8), dim3(128), 0, st, a);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel(),
+                      dim3((r.nx + M3_X - 1) / M3_X, (r.ny + TY - 1) / TY, (r.nz + zrun - 1) / zrun),
+                      dim3(M3_X, TY / RY), M3Smem<T, NF, TY>::total, st, a, zrun);
   }
 };
 
