@@ -54,10 +54,11 @@ struct dsm_lattice {
   int zrun_auto;
   // step on moments (dsm_mom.cuh): mok, the parameters allow it; mom, the
   // current state is held as moments (buffer mc); mcp, Cb[0] holds the C of its
-  // next step; mstat, the frozen solid's data is made; mfit, the canonical
+  // next step, mpk: the other buffer holds that step (made for reads); mstat, the
+  // frozen solid's data is made; mfit, the canonical
   // state is the result of a step with every relaxation time 1, so moments
   // represent it; mstepped, mom and stepped since set_fluid
-  bool mok, mom, mcp, mstat, mfit, mstepped;
+  bool mok, mom, mcp, mpk, mstat, mfit, mstepped;
   int mc, mzrun;
   // single-pass step of D2Q9 (dsm_tile2.cuh): tok, the parameters allow it; tp,
   // the state is f[cur] and the quads in g[cur ^ 1]; tcan, the canonical copy
@@ -444,13 +445,13 @@ cudaError_t m_leave(dsm_lattice *h) {
   if (e != cudaSuccess) return e;
   h->cur = 1;
   h->g_implicit = true;
-  h->mom = h->mcp = h->mstat = false;
+  h->mom = h->mcp = h->mpk = h->mstat = false;
   h->mfit = true;
   return cudaSuccess;
 }
 
 // A new state arrives by other means.
-void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mstat = h->mfit = h->tp = h->tcan = false; }
+void m_drop(dsm_lattice *h) { h->mom = h->mcp = h->mpk = h->mstat = h->mfit = h->tp = h->tcan = false; }
 
 // C of the next step of a state held as moments, into Cb[0].
 cudaError_t m_c(dsm_lattice *h) {
@@ -469,7 +470,7 @@ cudaError_t m_enter(dsm_lattice *h) {
   h->mc = 0;
   h->mom = true;
   h->mstepped = true;
-  h->mcp = false;
+  h->mcp = h->mpk = false;
   return cudaSuccess;
 }
 
@@ -516,7 +517,7 @@ cudaError_t m_collide(dsm_lattice *h) {
                         h->stream);
   if (e != cudaSuccess) return e;
   h->mc ^= 1;
-  h->mcp = false;
+  h->mcp = h->mpk = false;
   h->mstepped = true;
   return cudaSuccess;
 }
@@ -531,9 +532,22 @@ cudaError_t m_step(dsm_lattice *h) {
   if (e == cudaSuccess) e = h->tab.mom_step(m_raw(h, h->mc), m_zrun(h), h->stream);
   if (e != cudaSuccess) return e;
   h->mc ^= 1;
-  h->mcp = false;
+  h->mcp = h->mpk = false;
   h->mstepped = true;
   return cudaSuccess;
+}
+
+// The next step of a state held as moments, into the other buffer, for the reads
+// that take their values from it: in 3D, where the automatic form steps.
+bool m_peeks(const dsm_lattice *h) {
+  return h->kind == DSM_D3Q19 && h->step_form == DSM_STEP_AUTO;
+}
+cudaError_t m_peek(dsm_lattice *h) {
+  if (h->mpk) return cudaSuccess;
+  cudaError_t e = m_statics(h);
+  if (e == cudaSuccess) e = h->tab.mom_step(m_raw(h, h->mc), m_zrun(h), h->stream);
+  if (e == cudaSuccess) h->mpk = true;
+  return e;
 }
 
 // Read and clear nothing: report the latched device error word.
@@ -582,6 +596,14 @@ namespace {
 // canonical state, then the deterministic final reduction.
 cudaError_t obs_launch(dsm_lattice *h) {
   cudaError_t e;
+  if (h->mom && m_peeks(h)) {
+    e = m_peek(h);
+    if (e == cudaSuccess)
+      e = h->tab.mom_peek(m_raw(h, h->mc ^ 1), MODE_OBS, 0, nullptr, h->partials, h->stream);
+    if (e != cudaSuccess) return e;
+    obs_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, h->obs_blocks, h->obs);
+    return cudaGetLastError();
+  }
   if (h->mom) {
     e = m_statics(h);
     if (e == cudaSuccess) e = m_c(h);
@@ -839,7 +861,7 @@ dsm_status dsm_set_fluid(dsm_lattice *h, const void *d_c2) {
     if (e == cudaSuccess) e = h->tab.mom_init(m_raw(h, 1), d_c2, 0, h->stream);  // writes buffer 0
     h->mc = 0;
     h->mom = true;
-    h->mcp = h->mfit = h->mstepped = false;
+    h->mcp = h->mpk = h->mfit = h->mstepped = false;
   } else {
     m_drop(h);
     LBRaw r = raw_of(h, 1);  // writes buffer 0
@@ -937,6 +959,7 @@ dsm_status dsm_set_body_force(dsm_lattice *h, const double *body) {
   for (int a = 0; a < 3; a++)
     if (!isfinite(body[a])) return DSM_E_INVAL;
   for (int a = 0; a < 3; a++) h->prm.body_force[a] = body[a];
+  h->mpk = false;
   h->sp.body[0] = body[0];
   h->sp.body[1] = body[1];
   h->sp.body[2] = h->kind == DSM_D2Q9 ? 0.0 : body[2];
@@ -1039,6 +1062,12 @@ dsm_status dsm_get_field(dsm_lattice *h, int field, void *d_dst) {
     return cuda_status(e);
   }
   if (!h->has_fluid) return DSM_E_STATE;
+  if (h->mom && m_peeks(h)) {
+    e = field == DSM_FIELD_RHO || field == DSM_FIELD_TAU ? m_statics(h) : m_peek(h);
+    if (e == cudaSuccess)
+      e = h->tab.mom_peek(m_raw(h, h->mc ^ 1), MODE_FIELDS, field, d_dst, nullptr, h->stream);
+    return cuda_status(e);
+  }
   if (h->mom) {
     if (field == DSM_FIELD_C2 && !h->mcp)
       return cuda_status(h->tab.mom_c(m_raw(h, h->mc), d_dst, 0, h->stream));
@@ -1528,7 +1557,7 @@ dsm_status dsm_batch_step(dsm_lattice *const *hs, int n, const long long *nsteps
     if (left[i] == 0) continue;
     if (m_active(h)) {
       h->mc ^= (int)(left[i] & 1);
-      h->mcp = false;
+      h->mcp = h->mpk = false;
       h->mstepped = true;
     } else {
       h->tp = h->tcan = false;

@@ -342,6 +342,9 @@ struct LBTable {
   cudaError_t (*mom_c)(const MomRaw &r, void *c, long long cstride, cudaStream_t);
   cudaError_t (*mom_node)(const MomRaw &r, const void *c, long long cstride, int mode, int field,
                           int index, void *fields, double *partials, cudaStream_t);
+  // a field or the observables of the state whose next step r.in holds (3D)
+  cudaError_t (*mom_peek)(const MomRaw &r, int mode, int field, void *fields, double *partials,
+                          cudaStream_t);
   cudaError_t (*mom_relax)(const MomRaw &r, const MomRelax &m, int what, void *c, cudaStream_t);
   cudaError_t (*mom_solid)(const MomRaw &r, cudaStream_t);
   cudaError_t (*mom_init)(const MomRaw &r, const void *c, long long cstride, cudaStream_t);
