@@ -341,8 +341,8 @@ __device__ __forceinline__ void cp_async_bytes(unsigned dst, const void *src) {
 // The kernel it replaced for these lattices (populations f, tensor-memory
 // loads, dsm_zstep.cuh) takes 0.572 ms there: 196 B and 1189 instructions per
 // node against 81 B and 425.
-// With the wall pass, whole steps: 256 x 256 x 192 0.572 -> 0.264 ms, 101^3
-// 76.4 -> 46.5 us.
+// With the wall pass, whole steps: 256 x 256 x 192 0.572 -> 0.256 ms, 101^3
+// 76.4 -> 42.0 us.
 // ---------------------------------------------------------------------------
 constexpr int M3_X = 32, M3_HX = M3_X + 4, M3_HP = M3_HX + 1, M3_CX = M3_X + 2, M3_RING = 3;
 
@@ -817,9 +817,10 @@ __global__ void __launch_bounds__(M3_X *TY / RY, sizeof(T) == 8 ? 1 : BPS)
 // 2D step (D2Q9).  A block stages a TX x TY tile with a two-node halo, sums
 // this step's C on the tile and a one-node halo and the streamed f on the
 // tile, and collides.  One launch and 65 B per node in FP32 where the two passes
-// over populations took two and 128: 4096^2 0.427 -> 0.291 ms per step, 128 x 64
-// in FP64 (bound by the FP64 pipe and the launch) 24.6 -> 12.3 us.  STAGE 1 is the relaxation of the solid itself (C is
-// C1; rho = tau = tau_g = 1).  Beyond a mirror face the halo holds the image
+// over populations took two and 128: 4096^2 0.427 -> 0.283 ms per step, 128 x 64
+// in FP64 (bound by the FP64 pipe and the launch) 24.6 -> 10.4 us.  32 x 16 tiles:
+// 0.375 ms.  STAGE 1 is the relaxation of the solid itself (C is C1; rho = tau =
+// tau_g = 1).  Beyond a mirror face the halo holds the image
 // nodes with the normal components of u and G reversed, which gives both the
 // streaming's specular reflection and the stencils' zero normal gradient.
 // ---------------------------------------------------------------------------
@@ -872,16 +873,23 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
     }
     return c;
   };
+  // a tile whose halo lies within the lattice needs no map (4096^2 291 -> 283 us per
+  // step; the relaxation, whose tiles are lighter, is 5 % faster with it: 13.1 us
+  // against 13.7 at 1750 x 450)
+  const bool inner = STAGE == 2 && x0 >= 2 && y0 >= 2 && x0 + TX + 2 <= nx && y0 + TY + 2 <= ny;
   int flip[PER];
 #pragma unroll
   for (int r = 0; r < PER; r++) {
     const int k = tid + r * NT;
     flip[r] = 0;
     if ((r + 1) * NT <= SM::NS || k < SM::NS) {
-      int fx, fy;
-      const int gx = map(x0 - 2 + k % HX, nx, STAGE == 1 ? m1.mirror[0] : 0, fx);
-      const int gy = map(y0 - 2 + k / HX, ny, STAGE == 1 ? m1.mirror[1] : 0, fy);
-      flip[r] = (fx < 0 ? 1 : 0) | (fy < 0 ? 2 : 0);
+      int gx = x0 - 2 + k % HX, gy = y0 - 2 + k / HX;
+      if (!inner) {
+        int fx, fy;
+        gx = map(gx, nx, STAGE == 1 ? m1.mirror[0] : 0, fx);
+        gy = map(gy, ny, STAGE == 1 ? m1.mirror[1] : 0, fy);
+        flip[r] = (fx < 0 ? 1 : 0) | (fy < 0 ? 2 : 0);
+      }
       const long long n = chk(a.err, gx + (long long)nx * gy, a.N);
       cp_async_bytes<4 * sizeof(T)>(sbase + k * (4 * sizeof(T)), a.in.q1 + 4 * n);
       cp_async_bytes<2 * sizeof(T)>(sbase + SM::o2 + k * (2 * sizeof(T)), a.in.q2 + 2 * n);
@@ -905,7 +913,7 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
     }
   }
   cp_async_wait<0>();
-  if (STAGE == 1) {
+  if (STAGE == 1 && !inner) {
 #pragma unroll
     for (int r = 0; r < PER; r++) {
       if (flip[r]) {
