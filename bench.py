@@ -57,6 +57,14 @@ def lu_bytes_single(prec: str):
     real = 8 if prec == "f64" else 4
     st = {"f64": 8, "f32": 4, "bf16": 2, "f16": 2}[prec]
     return 2 * 19 * st + 2 * 5 * real + real
+
+
+def lu_bytes_moments(prec: str, nfluid: int = 2):
+    """Algorithmic bytes per lattice update of the D3Q19 step on moments (every
+    relaxation time 1, equal densities, periodic): read and write 9 reals, 2 more
+    per further fluid, read the solid's (C1, L[C1]) and a byte.  FP32: 81 B."""
+    real = 8 if prec == "f64" else 4
+    return 2 * (9 + 2 * (nfluid - 2)) * real + 2 * real + 1
 SHAPE = (256, 256, 192)
 WORKLOAD = "D3Q19 FP32 pillar-slab 256x256x192 (12.58M nodes), plain method, stage-2 LB step"
 
@@ -342,7 +350,11 @@ def run_gpu(args, rank, world):
         one_step()
     torch.cuda.synchronize()
     g_eq = lat.g_implicit
-    if single:
+    # (the automatic form's kernels: include/dsm.h, dsm_step_info)
+    moments = single and args.rho3 == 1.0 and args.tau3 == 1.0
+    if moments:
+        k2_b, k1_b = lu_bytes_moments(store), 0
+    elif single:
         k2_b, k1_b = lu_bytes_single(store), 0
     else:
         k2_b, k1_b = lu_bytes(lattice, store, g_eq)
@@ -403,7 +415,7 @@ def run_gpu(args, rank, world):
     default = (shape == SHAPE and lattice == "D3Q19" and args.rho3 == 1.0 and args.tau3 == 1.0
                and not faces and store == "f32")
     if single:
-        traffic = measured_traffic("zstep_kernel_d3q19_f32") if default else None
+        traffic = measured_traffic("zstep_kernel_d3q19_f32") if default and not moments else None
     else:
         traffic = (measured_traffic("node_kernel_d3q19_f32_geq" if g_eq else "node_kernel_d3q19_f32")
                    if default else None)
@@ -427,9 +439,13 @@ def run_gpu(args, rank, world):
                                     lattice, args.rho3, args.tau3, faces),
                "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak, "traffic": traffic,
-                            "kernel": ("zstep_kernel<f32,f32%s> (one pass per step, %d z planes "
-                                       "per block)" % (",density contrast" if args.rho3 != 1.0 else "",
-                                                       _lib.dsm_step_info(h)[1]))
+                            "kernel": "mom_wall_kernel, mom_step3_kernel (step on moments, %d z "
+                                      "planes per block)" % _lib.dsm_step_info(h)[1]
+                                      if moments else
+                                      "moments_eq_tiled_kernel, node_kernel<D3Q19,f32,stage2,step,"
+                                      "g_eq,density contrast>" if single and args.rho3 != 1.0 else
+                                      "zstep_kernel<f32,f32> (one pass per step, %d z planes "
+                                      "per block)" % _lib.dsm_step_info(h)[1]
                                       if single else
                                       "node_kernel<%s,f32,stage2,step,%s%s>" %
                                       (lattice, "g_eq" if g_eq else "populations",
@@ -441,7 +457,8 @@ def run_gpu(args, rank, world):
                             "measured_frac": (traffic / n * lups_gpu / 1e9 / peak) if traffic else None,
                             "b_min_per_lu": b_min, "useful_frac": b_min * lups_gpu / 1e9 / peak},
                "clocks": clk.summary(), "e2e": e2e,
-               "gpu_launches": (1 if single else 2) * args.steps,
+               "gpu_launches": (1 if single and not moments and args.rho3 == 1.0 else 2)
+                               * args.steps,
                "cpu_baseline": cb,
                "observables": {"mass_c2": obs["mass_c2"], "max_u": obs["max_u"]}}
         print(json.dumps(out), flush=True)
@@ -559,7 +576,7 @@ def run_precision(args, rank, world):
         lat.set_fluid(torch.as_tensor(case.c2, dtype=torch.float32, device=dev))
         lat.set_step_form(args.step_form, args.zrun)
         t_step, t_k2 = _time_steps(lat, args.steps, args.warmup)
-        bmin = (lu_bytes_single(prec) if lat.single_pass
+        bmin = (lu_bytes_moments(prec) if lat.single_pass
                 else lu_bytes("D3Q19", prec, lat.g_implicit)[0])
         ob = lat.observables()
         out[prec] = {"MLUPS": lat.n / t_step / 1e6, "ms_per_step": t_step * 1e3,
@@ -641,7 +658,7 @@ def run_ramp(args, rank, world):
             torch.cuda.empty_cache()
     t_max, lups = aggregate(t_total, lu_total, dist)
     value = lups / 1e6
-    achieved = lu_bytes_single("f32") * value * 1e6 / 1e9
+    achieved = lu_bytes_moments("f32") * value * 1e6 / 1e9
     if rank == 0:
         print(json.dumps({
             "metric": "cfg2 pressure ramp: critical pressure per contact angle; ramp MLUPS",
@@ -657,8 +674,8 @@ def run_ramp(args, rank, world):
                                  "and the field reads of the detector"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "zstep_kernel<f32,f32> (one pass per step)",
-                         "bytes_per_lu": lu_bytes_single("f32"), "peak_source": peak_kind},
+                         "kernel": "mom_wall_kernel, mom_step3_kernel (step on moments)",
+                         "bytes_per_lu": lu_bytes_moments("f32"), "peak_source": peak_kind},
             "clocks": clk.summary(), "runs": runs}), flush=True)
     if dist:
         dist.destroy_process_group()
@@ -986,8 +1003,9 @@ def run_multi(args, rank, world):
     peak, peak_kind = _peaks()
     nf = nfl - 1
     single = ml.single_pass
-    b = 180 + 16 * nf if ml.g_implicit else 2 * 19 * 4 * (nf + 1) + 4 + 80 * nf
-    launches = 1 if single else (nf + 1 if ml.g_implicit else 2)
+    b = (lu_bytes_moments("f32", nfl) if single else
+         180 + 16 * nf if ml.g_implicit else 2 * 19 * 4 * (nf + 1) + 4 + 80 * nf)
+    launches = 2 if single else (nf + 1 if ml.g_implicit else 2)
     names = {3: "three", 4: "four"}
     if rank == 0:
         print(json.dumps({
