@@ -305,12 +305,24 @@ cudaError_t z_unpack(dsm_lattice *h) {
   return cudaSuccess;
 }
 
+// FP64 lattices in 2D that are neither so small that at most two of their 64-node
+// tiles fall to an SM nor large enough for tiles of 256 nodes on every SM stay with
+// two passes over populations: the FP64 pipe is the bound there, and the halo of a
+// tile costs it more sums of C.  One launch against two passes, us per step:
+// 128 x 64 11.1 and 24.7, 160 x 121 22.1 and 26.7, 256 x 96 33.7 and 28.8 (34.9 with
+// tiles of 256), 256 x 128 42.3 and 32.9 (40.0), 512 x 512 87 and 140.
+bool f64_tiles(const dsm_params *p) {
+  if (p->precision != DSM_F64 || p->lattice != DSM_D2Q9) return true;
+  const long long n = (long long)p->nx * p->ny;
+  return n <= 2ll * 152 * 64 || n >= 2ll * 152 * 256;
+}
+
 // ---- single-pass step of D2Q9 ---------------------------------------------------
 // It applies with tau_g = 1 and faces that are periodic or mirrors (at a wall
 // g would bounce back, which no image node gives), in the automatic forms of g
 // and of the step, where the step on moments does not.
 bool t_eligible(const dsm_params *p) {
-  if (p->lattice != DSM_D2Q9 || p->tau_g != 1.0) return false;
+  if (p->lattice != DSM_D2Q9 || p->tau_g != 1.0 || !f64_tiles(p)) return false;
   const int n[2] = {p->nx, p->ny};
   for (int a = 0; a < 2; a++) {
     const int lo = p->face[2 * a], hi = p->face[2 * a + 1];
@@ -366,9 +378,15 @@ cudaError_t t_step(dsm_lattice *h) {
 // 16-bit populations the moments are FP32 reals all the same: 36 B per node are
 // fewer than the 38 B of the populations and the 20 B of (A, C, u) that they
 // replace, and nothing is rounded to 16 bits any more.
+// Small FP64 lattices in 3D keep their populations: their runs of one plane form
+// four planes' sums for it on the FP64 pipe (16^3: 53 us per step in two passes, 87
+// on moments; 32^3: 86 and 84; 64^3: 351 and 272).
 bool m_eligible(const dsm_params *p) {
+  if (p->precision == DSM_F64 && p->lattice == DSM_D3Q19 &&
+      (long long)p->nx * p->ny * p->nz < 32768)
+    return false;
   const bool k16 = p->precision != DSM_F32 && p->precision != DSM_F64;
-  return (!k16 || z_eligible(p)) && p->tau2 == 1.0 && p->tau3 == 1.0 && p->tau_g == 1.0 &&
+  return (!k16 || z_eligible(p)) && f64_tiles(p) && p->tau2 == 1.0 && p->tau3 == 1.0 && p->tau_g == 1.0 &&
          p->rho2 == p->rho3 && !has_walls(p);
 }
 bool m_active(const dsm_lattice *h) {
@@ -495,7 +513,7 @@ int m_zrun(dsm_lattice *h) {
 // Whether dsm_relax_solid runs on moments: D2Q9 in FP32 or FP64, each axis
 // periodic, or a mirror on both sides (a wall's bounce-back has no image node).
 bool m_relax_of(const dsm_lattice *h, MomRelax *m) {
-  if (h->kind != DSM_D2Q9 || !h->tab.mom_relax) return false;
+  if (h->kind != DSM_D2Q9 || !h->tab.mom_relax || !f64_tiles(&h->prm)) return false;
   const int n[2] = {h->prm.nx, h->prm.ny};
   for (int a = 0; a < 2; a++) {
     const int lo = h->prm.face[2 * a], hi = h->prm.face[2 * a + 1];
