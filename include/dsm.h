@@ -228,7 +228,8 @@ dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun);
  * (*single_pass = 1) and with how many z planes per block (*zrun; 0 for the
  * two-pass step).  The automatic form takes the fastest kernels for the same
  * step where others are faster: moments in the place of populations where every
- * relaxation time is 1, two passes with a density contrast in FP32 arithmetic.
+ * relaxation time is 1, two passes with a density contrast in FP32 arithmetic
+ * from 180000 nodes up.
  * Either pointer may be NULL. */
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun);
 

@@ -276,9 +276,11 @@ bool z_form(const dsm_lattice *h) {
 // single pass out of issue slots with 24 warps per SM (250 x 130 x 101: 303 us per
 // step, 184 + 45 in two passes; rho planes formed once per node in shared memory
 // spilled, 378 us, and as a plane of the moments pass changed nothing, 181 + 52).
-// FP64, bound by its pipe, keeps the single pass.
+// FP64, bound by its pipe, keeps the single pass, and so do lattices too small to
+// pay for a second launch (20 steps and two fields, single pass and two: 40 x 40 x 64
+// 552 and 587 us, 64^3 737 and 684, 120 x 100 x 80 2138 and 1898).
 bool z_active(const dsm_lattice *h) {
-  return z_form(h) && !(h->sp.rho_contrast && h->tab.real_bytes == 4);
+  return z_form(h) && !(h->sp.rho_contrast && h->tab.real_bytes == 4 && h->N >= 180000);
 }
 
 // Canonical g_eq state -> padded buffers (buffer 0), and padded C1.
