@@ -25,31 +25,132 @@ __device__ __forceinline__ T bw(T c) {
 // dE/dC2 = d2 - d3 (+ constraint + fg h),  dE/dC1 = d1 - d3 + 2 beta (C1 - 1/2) chi,
 // d_n = kappa_n b(C_n) - a^2 kappa_n L[C_n],  C3 = 1 - C1 - C2.
 // ---------------------------------------------------------------------------
+// The minimiser's evaluations, and every one in 2D.  The order of these sums is
+// part of the minimiser's result (L-BFGS amplifies the last place of E into the
+// iterates), so it stays as it is: threads own the nodes of fixed bricks.  128^3:
+// 43 us where fe_march_kernel, whose sums run along z, takes 32.
+template <int K>
+__global__ void __launch_bounds__(256) fe_kernel(FEArgs a, int gx, int gy, int nbricks) {
+  using L = Lat<K>;
+  constexpr int Q = L::Q;
+  FF acc[FE_K];
+#pragma unroll
+  for (int k = 0; k < FE_K; k++) acc[k] = FF{0.0f, 0.0f};
+  // resident blocks walk the node bricks (blockDim-shaped boxes) in a fixed
+  // grid-stride order, so each block leaves one partial sum; the brick
+  // coordinates advance by the stride's own (x, y, z) digits with carries
+  // instead of three divisions per brick
+  const int G = gridDim.x;
+  const int sx = G % gx, sy = (G / gx) % gy, sz = G / (gx * gy);
+  int bx = blockIdx.x % gx, by = (blockIdx.x / gx) % gy, bz = blockIdx.x / (gx * gy);
+  for (int b = blockIdx.x; b < nbricks; b += G) {
+    if (b != blockIdx.x) {
+      bx += sx;
+      by += sy;
+      bz += sz;
+      if (bx >= gx) {
+        bx -= gx;
+        by++;
+      }
+      if (by >= gy) {
+        by -= gy;
+        bz++;
+      }
+    }
+    const int x = bx * blockDim.x + threadIdx.x;
+    const int y = by * blockDim.y + threadIdx.y;
+    const int z = bz * blockDim.z + threadIdx.z;
+    if (!(x < a.nx && y < a.ny && z < a.nz)) continue;
+    const int xm = x == 0 ? a.lo[0] : x - 1, xp = x + 1 == a.nx ? a.hi[0] : x + 1;
+    const int ym = y == 0 ? a.lo[1] : y - 1, yp = y + 1 == a.ny ? a.hi[1] : y + 1;
+    const int zm = z == 0 ? a.lo[2] : z - 1, zp = z + 1 == a.nz ? a.hi[2] : z + 1;
+    const int s = a.nx * a.ny;
+    const int ox[3] = {xm, x, xp}, oy[3] = {ym * a.nx, y * a.nx, yp * a.nx},
+              oz[3] = {zm * s, z * s, zp * s};
+    const int n = x + y * a.nx + z * s;
+    const float k1 = a.kappa[0], k2 = a.kappa[1], k3 = a.kappa[2];
+    const float c1 = a.c1[n], c2 = a.c2[n], c3 = 1.0f - c1 - c2;
+    // C3 = 1 - C1 - C2, so its differences are -(d1 + d2): L[C3] = -L[C1] - L[C2]
+    // and its pair sum is p1 + p2 + 2 x12 with x12 = sum_i w_i d1 d2
+    float l1 = 0.f, l2 = 0.f, p1 = 0.f, p2 = 0.f, x12 = 0.f;
+#pragma unroll
+    for (int i = 1; i < Q; i++) {
+      const int m = ox[L::cx(i) + 1] + oy[L::cy(i) + 1] + oz[L::cz(i) + 1];
+      const float w = float(L::w(i));
+      const float d1 = __ldg(a.c1 + m) - c1, d2 = __ldg(a.c2 + m) - c2;
+      const float t1 = w * d1, t2 = w * d2;
+      l1 += t1;
+      l2 += t2;
+      p1 = fmaf(t1, d1, p1);
+      p2 = fmaf(t2, d2, p2);
+      x12 = fmaf(t1, d2, x12);
+    }
+    const float p3 = p1 + p2 + 2.0f * x12;
+    l1 *= 6.f;
+    l2 *= 6.f;
+    const float l3 = -(l1 + l2);
+    const float A2 = a.a2;
+    // per-node densities in FP32, accumulated with carried rounding errors
+    const float q1 = c1 * (1.0f - c1), q2 = c2 * (1.0f - c2), q3 = c3 * (1.0f - c3);
+    acc[0] = ff_add(acc[0], FF{0.5f * (k1 * q1 * q1 + k2 * q2 * q2 + k3 * q3 * q3), 0.0f});
+    acc[1] = ff_add(acc[1], FF{1.5f * A2 * (k1 * p1 + k2 * p2 + k3 * p3), 0.0f});
+    const bool inS = a.mask ? a.mask[n] != 0 : false;
+    const bool chi = (inS && c1 < 0.5f) || (!inS && c1 > 0.5f);
+    if (a.active == 1 && chi) acc[2] = ff_add(acc[2], FF{a.beta * (c1 - 0.5f) * (c1 - 0.5f), 0.0f});
+    const int hgt = (a.d == 2) ? y : z;
+    acc[3] = ff_add(acc[3], FF{a.fg * c2 * (float)hgt, 0.0f});
+    acc[4] = ff_add(acc[4], FF{c2, 0.0f});
+    const float dd1 = k1 * bw(c1) - A2 * k1 * l1;
+    const float dd2 = k2 * bw(c2) - A2 * k2 * l2;
+    const float dd3 = k3 * bw(c3) - A2 * k3 * l3;
+    float gr;
+    if (a.active == 2) gr = dd2 - dd3 + a.const_grad + a.fg * (float)hgt;
+    else gr = dd1 - dd3 + (chi ? 2.0f * a.beta * (c1 - 0.5f) : 0.0f);
+    a.grad[n] = gr;
+  }
+  const int sums[FE_K] = {0, 0, 0, 0, 0};
+  block_reduce_ff<FE_K>(acc, sums, a.partials + (long long)blockIdx.x * FE_K);
+}
+
+// Sum the per-block partials, a warp per sum (the tree of 256 threads);
+// assemble E and the constraint.
+__global__ void __launch_bounds__(32 * FE_K)
+    fe_finalize_kernel(const double *partials, int nb, double dP, double kcs, double V0,
+                       double *energy, double *terms, double *dEcs) {
+  __shared__ double sh[FE_K];
+  const double t = warp_sum256(partials + (threadIdx.x >> 5), nb, FE_K);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double V = sh[4];
+    const double Ecs = (kcs == 0.0) ? -dP * V : 0.5 * kcs * (V - V0) * (V - V0);
+    const double E = sh[0] + sh[1] + sh[2] + Ecs + sh[3];
+    if (energy) energy[0] = E;
+    if (terms) {
+      terms[0] = sh[0];
+      terms[1] = sh[1];
+      terms[2] = sh[2];
+      terms[3] = Ecs;
+      terms[4] = sh[3];
+      terms[5] = V;
+    }
+    dEcs[0] = (kcs == 0.0) ? -dP : kcs * (V - V0);
+  }
+}
+
 // s + v with the rounding error carried in lo (no renormalisation)
 __device__ __forceinline__ void acc_sum(FF &s, float v) {
   const FF t = two_sum(s.hi, v);
   s.hi = t.hi;
   s.lo += t.lo;
 }
-// The exact product a b (TwoProd: p + e, e from one FMA) added to the pair s:
-// TwoSum into s.hi, both rounding errors into s.lo.  FP64 accuracy from FP32
-// instructions, without renormalising the pair at every element.
-__device__ __forceinline__ void acc_prod(FF &s, float a, float b) {
-  const float p = a * b;
-  const float pe = fmaf(a, b, -p);
-  const FF t = two_sum(s.hi, p);
-  s.hi = t.hi;
-  s.lo += t.lo + pe;
-}
-
 // Energy densities and gradient of node n at height hgt from its stencil sums:
 // l, sum_i w_i d_i, and p, sum_i w_i d_i d_i, of C1 and C2, x12 the mixed one.
 // C3 = 1 - C1 - C2, so its differences are -(d1 + d2): L[C3] = -L[C1] - L[C2]
 // and its pair sum is p1 + p2 + 2 x12.
-template <bool SLOPE>
 __device__ __forceinline__ void fe_node(const FEArgs &a, long long n, int hgt, float c1, float c2,
                                         float l1, float l2, float p1, float p2, float x12,
-                                        FF (&acc)[SLOPE ? FE_KS : FE_K]) {
+                                        FF (&acc)[FE_K]) {
   const float k1 = a.kappa[0], k2 = a.kappa[1], k3 = a.kappa[2], A2 = a.a2;
   const float c3 = 1.0f - c1 - c2;
   const float p3 = p1 + p2 + 2.0f * x12;
@@ -75,69 +176,6 @@ __device__ __forceinline__ void fe_node(const FEArgs &a, long long n, int hgt, f
   if (a.active == 2) gr = dd2 - dd3 + a.const_grad + a.fg * (float)hgt;
   else gr = dd1 - dd3 + (chi ? 2.0f * a.beta * (c1 - 0.5f) : 0.0f);
   a.grad[n] = gr;
-  if constexpr (SLOPE) {
-    acc_prod(acc[FE_K], gr, a.dir[n]);
-  }
-}
-
-// Sum the per-block partials (k of the nk of every block, in block order);
-// assemble E, the constraint and the slope.  Called by one block.
-template <int NK>
-__device__ __forceinline__ void fe_finish(const double *partials, int nb, const FEFin &fin) {
-  __shared__ double tot[NK];
-  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int lane = tid & 31, nw = (blockDim.x * blockDim.y * blockDim.z) >> 5;
-  for (int k = tid >> 5; k < NK; k += nw) {  // a warp per sum
-    double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += ((volatile const double *)partials)[(long long)b * NK + k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) tot[k] = s;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const double V = tot[4];
-    const double Ecs = (fin.kcs == 0.0) ? -fin.dP * V : 0.5 * fin.kcs * (V - fin.V0) * (V - fin.V0);
-    const double dV = (fin.kcs == 0.0) ? -fin.dP : fin.kcs * (V - fin.V0);
-    if (fin.energy) fin.energy[0] = tot[0] + tot[1] + tot[2] + Ecs + tot[3];
-    if (fin.terms) {
-      fin.terms[0] = tot[0];
-      fin.terms[1] = tot[1];
-      fin.terms[2] = tot[2];
-      fin.terms[3] = Ecs;
-      fin.terms[4] = tot[3];
-      fin.terms[5] = V;
-    }
-    fin.dEcs[0] = dV;
-    if constexpr (NK > FE_K)
-      if (fin.slope) fin.slope[0] = tot[FE_K];
-  }
-}
-__global__ void __launch_bounds__(256) fe_finalize_kernel(const double *partials, int nb, FEFin fin) {
-  fe_finish<FE_K>(partials, nb, fin);
-}
-
-// Block sums of an evaluation; with fin.counter the last block of the grid (the
-// one that counts itself last: every partial is then visible) finishes.  No
-// block waits for another.
-template <int NK>
-__device__ __forceinline__ void fe_close(const FF (&acc)[NK], double *partials, const FEFin &fin) {
-  int sums[NK];
-#pragma unroll
-  for (int k = 0; k < NK; k++) sums[k] = 0;
-  block_reduce_ff<NK>(acc, sums, partials + (long long)blockIdx.x * NK);
-  if (!fin.counter) return;
-  __shared__ bool last;
-  __syncthreads();
-  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  if (tid == 0) {
-    __threadfence();
-    last = atomicAdd(fin.counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  fe_finish<NK>(partials, gridDim.x, fin);
-  if (tid == 0) *fin.counter = 0u;
 }
 
 // 3D: a block takes 32 x 8 tiles and runs of z planes in grid-stride order, a
@@ -153,16 +191,15 @@ __device__ __forceinline__ void fe_close(const FF (&acc)[NK], double *partials, 
 // with the points read through L1 instead of staged: 36.7.
 constexpr int FE_TX = 32, FE_TY = 8, FE_RY = 2, FE_RING = 4;
 constexpr int FE_HX = FE_TX + 2, FE_HY = FE_TY + 2, FE_NS = FE_HX * FE_HY;
-template <bool SLOPE>
 __global__ void __launch_bounds__(FE_TX *FE_TY / FE_RY, 4)
-    fe_march_kernel(FEArgs a, int tx, int ty, int items, int zrun, FEFin fin) {
+    fe_march_kernel(FEArgs a, int tx, int ty, int items, int zrun) {
   using L = Lat<1>;
-  constexpr int NK = SLOPE ? FE_KS : FE_K, R = FE_RY, NT = FE_TX * FE_TY / R;
+  constexpr int R = FE_RY, NT = FE_TX * FE_TY / R;
   constexpr int PER = (FE_NS + NT - 1) / NT;
   __shared__ float2 sm[FE_RING][FE_NS];  // (C1, C2)
-  FF acc[NK];
+  FF acc[FE_K];
 #pragma unroll
-  for (int k = 0; k < NK; k++) acc[k] = FF{0.0f, 0.0f};
+  for (int k = 0; k < FE_K; k++) acc[k] = FF{0.0f, 0.0f};
   const int plane = a.nx * a.ny;
   const int tid = threadIdx.x + FE_TX * threadIdx.y;
   const int k0 = (threadIdx.y * R) * FE_HX + threadIdx.x;  // corner of the nodes' points
@@ -233,8 +270,8 @@ __global__ void __launch_bounds__(FE_TX *FE_TY / FE_RY, 4)
           pp = __ffma2_rn(t, d, pp);
           x12 = fmaf(t.x, d.y, x12);
         }
-        fe_node<SLOPE>(a, (long long)z * plane + (long long)a.nx * (y + j) + x, z, c.x, c.y, l.x,
-                       l.y, pp.x, pp.y, x12, acc);
+        fe_node(a, (long long)z * plane + (long long)a.nx * (y + j) + x, z, c.x, c.y, l.x, l.y,
+                pp.x, pp.y, x12, acc);
       }
     };
     __syncthreads();  // the last item's planes are read
@@ -255,41 +292,8 @@ __global__ void __launch_bounds__(FE_TX *FE_TY / FE_RY, 4)
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   }
-  fe_close<NK>(acc, a.partials, fin);
-}
-
-// 2D: resident blocks walk 32 x 8 bricks in grid-stride order.
-template <bool SLOPE>
-__global__ void __launch_bounds__(256) fe_kernel2(FEArgs a, int gx, int nbricks, FEFin fin) {
-  using L = Lat<0>;
-  constexpr int NK = SLOPE ? FE_KS : FE_K;
-  FF acc[NK];
-#pragma unroll
-  for (int k = 0; k < NK; k++) acc[k] = FF{0.0f, 0.0f};
-  for (int b = blockIdx.x; b < nbricks; b += gridDim.x) {
-    const int x = b % gx * 32 + threadIdx.x, y = b / gx * 8 + threadIdx.y;
-    if (!(x < a.nx && y < a.ny)) continue;
-    const int ox[3] = {x == 0 ? a.lo[0] : x - 1, x, x + 1 == a.nx ? a.hi[0] : x + 1};
-    const int oy[3] = {(y == 0 ? a.lo[1] : y - 1) * a.nx, y * a.nx,
-                       (y + 1 == a.ny ? a.hi[1] : y + 1) * a.nx};
-    const int n = x + y * a.nx;
-    const float c1 = a.c1[n], c2 = a.c2[n];
-    float l1 = 0.f, l2 = 0.f, p1 = 0.f, p2 = 0.f, x12 = 0.f;
-#pragma unroll
-    for (int i = 1; i < L::Q; i++) {
-      const int m = ox[L::cx(i) + 1] + oy[L::cy(i) + 1];
-      const float w = float(L::w(i));
-      const float d1 = __ldg(a.c1 + m) - c1, d2 = __ldg(a.c2 + m) - c2;
-      const float t1 = w * d1, t2 = w * d2;
-      l1 += t1;
-      l2 += t2;
-      p1 = fmaf(t1, d1, p1);
-      p2 = fmaf(t2, d2, p2);
-      x12 = fmaf(t1, d2, x12);
-    }
-    fe_node<SLOPE>(a, n, y, c1, c2, l1, l2, p1, p2, x12, acc);
-  }
-  fe_close<NK>(acc, a.partials, fin);
+  const int sums[FE_K] = {0, 0, 0, 0, 0};
+  block_reduce_ff<FE_K>(acc, sums, a.partials + (long long)blockIdx.x * FE_K);
 }
 
 __global__ void add_dev_scalar_kernel(long long n, const double *c, float *g) {
@@ -382,39 +386,37 @@ size_t fe_scratch_bytes(int kind, int nx, int ny, int nz) {
   return (size_t)round_up(fe_blocks(kind, nx, ny, nz) * FE_K * sizeof(double), 256) + 256;
 }
 
-// blocks of one evaluation, at most `most` (one partial sum per block)
-template <bool SLOPE>
-static int fe_run(int kind, const FEArgs &a, const FEFin &fin, long long most, cudaStream_t st) {
-  if (kind == 0) {
-    const dim3 g = fe_bricks(0, a.nx, a.ny, 1);
-    const long long bricks = (long long)g.x * g.y, nb = bricks < most ? bricks : most;
-    fe_kernel2<SLOPE><<<(unsigned)nb, fe_block(0), 0, st>>>(a, g.x, (int)bricks, fin);
-    return (int)nb;
-  }
-  // runs of z planes so that the tiles fill the blocks once, but no shorter than
-  // four planes (each run reads two more)
-  const int tx = (a.nx + FE_TX - 1) / FE_TX, ty = (a.ny + FE_TY - 1) / FE_TY;
-  long long runs = most / ((long long)tx * ty);
-  if (runs < 1) runs = 1;
-  if (runs > (a.nz + 3) / 4) runs = (a.nz + 3) / 4;
-  const int zrun = (int)((a.nz + runs - 1) / runs);
-  const long long items = (long long)tx * ty * ((a.nz + zrun - 1) / zrun);
-  const long long nb = items < most ? items : most;
-  fe_march_kernel<SLOPE><<<(unsigned)nb, dim3(FE_TX, FE_TY / FE_RY), 0, st>>>(a, tx, ty, (int)items,
-                                                                              zrun, fin);
-  return (int)nb;
-}
-
 cudaError_t fe_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
-                      double *terms, void *scratch, cudaStream_t st) {
+                      double *terms, void *scratch, cudaStream_t st, bool fixed_order,
+                      const double **defer) {
   const long long most = fe_blocks(kind, a.nx, a.ny, a.nz);
   double *partials = (double *)scratch;
   double *dEcs = (double *)((char *)scratch + round_up(most * FE_K * sizeof(double), 256));
   a.partials = partials;
   a.const_grad = (kcs == 0.0) ? (float)(-dP) : 0.0f;
-  const FEFin fin = {dP, kcs, V0, energy, terms, dEcs, nullptr, nullptr};
-  const int nb = fe_run<false>(kind, a, fin, most, st);
-  fe_finalize_kernel<<<1, 256, 0, st>>>(partials, nb, fin);
+  long long nb = most;  // partial sums, one per block
+  if (kind == 0 || fixed_order) {
+    const dim3 g = fe_bricks(kind, a.nx, a.ny, a.nz);
+    const int nbricks = (int)((long long)g.x * g.y * g.z);
+    if (kind == 0) fe_kernel<0><<<(unsigned)nb, fe_block(0), 0, st>>>(a, g.x, g.y, nbricks);
+    else fe_kernel<1><<<(unsigned)nb, fe_block(1), 0, st>>>(a, g.x, g.y, nbricks);
+  } else {
+    // runs of z planes so that the tiles fill the blocks once, but no shorter than
+    // four planes (each run reads two more)
+    const int tx = (a.nx + FE_TX - 1) / FE_TX, ty = (a.ny + FE_TY - 1) / FE_TY;
+    long long runs = most / ((long long)tx * ty);
+    if (runs < 1) runs = 1;
+    if (runs > (a.nz + 3) / 4) runs = (a.nz + 3) / 4;
+    const int zrun = (int)((a.nz + runs - 1) / runs);
+    const long long items = (long long)tx * ty * ((a.nz + zrun - 1) / zrun);
+    nb = items < most ? items : most;
+    fe_march_kernel<<<(unsigned)nb, dim3(FE_TX, FE_TY / FE_RY), 0, st>>>(a, tx, ty, (int)items, zrun);
+  }
+  fe_finalize_kernel<<<1, 32 * FE_K, 0, st>>>(partials, (int)nb, dP, kcs, V0, energy, terms, dEcs);
+  if (defer) {  // the caller adds the constraint's constant (null: none)
+    *defer = (kcs != 0.0 && a.active == 2) ? dEcs : nullptr;
+    return cudaGetLastError();
+  }
   if (kcs != 0.0 && a.active == 2) {
     const long long N = (long long)a.nx * a.ny * a.nz;
     long long blocks = (N + 255) / 256;
@@ -422,28 +424,6 @@ cudaError_t fe_launch(int kind, FEArgs a, double dP, double kcs, double V0, doub
     add_dev_scalar_kernel<<<(int)blocks, 256, 0, st>>>(N, dEcs, a.grad);
   }
   return cudaGetLastError();
-}
-
-size_t fe_slope_scratch_bytes() {
-  return 512 + (FE_MAX_BLOCKS * FE_KS + VEC_BLOCKS) * sizeof(double);
-}
-
-cudaError_t fe_slope_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
-                            double *slope, void *scratch, cudaStream_t st) {
-  double *cst = (double *)((char *)scratch + 256);
-  unsigned *counter = (unsigned *)scratch;
-  a.partials = (double *)((char *)scratch + 512);
-  a.const_grad = (kcs == 0.0) ? (float)(-dP) : 0.0f;
-  const FEFin fin = {dP, kcs, V0, energy, nullptr, cst, slope, counter};
-  if (kcs == 0.0 || a.active == 1) {
-    fe_run<true>(kind, a, fin, FE_MAX_BLOCKS, st);
-    return cudaGetLastError();
-  }
-  // the constraint's constant is known only after every block's sums: a second
-  // pass adds it to the gradient and takes the slope
-  fe_run<false>(kind, a, fin, FE_MAX_BLOCKS, st);
-  return vec_trial_slope((long long)a.nx * a.ny * a.nz, cst, a.grad, a.dir, slope,
-                         (double *)((char *)scratch + 512) + FE_MAX_BLOCKS * FE_KS, counter, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -627,6 +607,17 @@ cudaError_t fe_multi_launch(int kind, FEMArgs a, const FEMCons &cons, double *en
 
 static int vec_grid(long long n);
 
+// The exact product a b (TwoProd: p + e, e from one FMA) added to the pair s:
+// TwoSum into s.hi, both rounding errors into s.lo.  FP64 accuracy from FP32
+// instructions, without renormalising the pair at every element.
+__device__ __forceinline__ void acc_prod(FF &s, float a, float b) {
+  const float p = a * b;
+  const float pe = fmaf(a, b, -p);
+  const FF t = two_sum(s.hi, p);
+  s.hi = t.hi;
+  s.lo += t.lo + pe;
+}
+
 // The last block of a grid sums the grid's partials in block order (as
 // dot_finalize_kernel does) into out[0] and rearms the counter: each block
 // publishes its partial, counts itself, and the block that counts last (every
@@ -699,8 +690,10 @@ __global__ void __launch_bounds__(256) trial_slope_kernel(long long n, const dou
 }
 
 cudaError_t vec_trial_slope(long long n, const double *c, float *g, const float *d, double *out,
-                            double *partials, unsigned *counter, cudaStream_t st) {
+                            void *scratch, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
+  double *partials = (double *)scratch;
+  unsigned *counter = vec_scratch_counter(scratch);
   trial_slope_kernel<<<vec_grid(n), 256, 0, st>>>(n, c, g, d, partials, counter, out);
   return cudaGetLastError();
 }
@@ -842,8 +835,6 @@ static int vec_grid(long long n) {
   long long b = (n + 255) / 256;
   return (int)(b < VEC_BLOCKS ? (b > 0 ? b : 1) : VEC_BLOCKS);
 }
-
-int vec_blocks(long long n) { return vec_grid(n); }
 
 size_t vec_scratch_bytes(long long) { return VEC_BLOCKS * sizeof(double) + 256; }
 

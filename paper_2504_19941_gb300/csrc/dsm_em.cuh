@@ -22,7 +22,6 @@ struct FEArgs {
   const float *c1, *c2;
   const unsigned char *mask;
   float *grad;
-  const float *dir;  // direction of the slope (null: none)
   double *partials;
 };
 
@@ -62,27 +61,14 @@ dsm_status fem_args_of(const dsm_params *p, int nfluid, const double *kappa, con
 cudaError_t fe_multi_launch(int kind, FEMArgs a, const FEMCons &cons, double *energy,
                             double *terms, void *scratch, cudaStream_t st);
 
-// What one energy evaluation leaves besides the gradient: E and its terms
-// (null: not wanted), and the constraint's derivative dE/dV (dEcs).  With dir,
-// also the slope of the gradient along dir.
-// counter (zero before and after): the evaluation's last block sums the
-// partials; null: a second launch does.
-struct FEFin {
-  double dP, kcs, V0;
-  double *energy, *terms, *dEcs, *slope;
-  unsigned *counter;
-};
-constexpr int FE_KS = FE_K + 1;  // partials of an evaluation with a slope
-
 long long fe_blocks(int kind, int nx, int ny, int nz);
 size_t fe_scratch_bytes(int kind, int nx, int ny, int nz);
+// fixed_order: the sums in the minimiser's order (fe_kernel).
+// defer: when given, the constraint's constant is not added to the gradient;
+// *defer receives its device address (null when there is none).
 cudaError_t fe_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
-                      double *terms, void *scratch, cudaStream_t st);
-// Energy, complete gradient and its slope along a.dir.  scratch:
-// fe_slope_scratch_bytes() bytes, its first 256 zero before and after.
-size_t fe_slope_scratch_bytes();
-cudaError_t fe_slope_launch(int kind, FEArgs a, double dP, double kcs, double V0, double *energy,
-                            double *slope, void *scratch, cudaStream_t st);
+                      double *terms, void *scratch, cudaStream_t st, bool fixed_order = false,
+                      const double **defer = nullptr);
 
 constexpr int LINCOMB_MAX = 64;  // most vectors one dsm_vec_lincomb combines
 struct LinCoef {
@@ -92,14 +78,17 @@ struct LinCoef {
 
 size_t vec_scratch_bytes(long long n);
 size_t vec_dots_scratch_bytes(long long n, int nv);
-// elements a grid-stride vector pass of n elements has in flight per step
-int vec_blocks(long long n);
 cudaError_t vec_dots(long long n, int nv, const float *V, long long stride, const float *x,
                      double *out, void *scratch, cudaStream_t st);
-// g += c[0] if c is given, out[0] = g.d, one launch (counter: zero before and
-// after; partials: VEC_BLOCKS doubles).
+// A trial point's gradient and slope: g += c[0] if c is given, out[0] = g.d,
+// one launch (scratch: vec_scratch_bytes(n), whose counter word starts and
+// ends at zero).
 cudaError_t vec_trial_slope(long long n, const double *c, float *g, const float *d, double *out,
-                            double *partials, unsigned *counter, cudaStream_t st);
+                            void *scratch, cudaStream_t st);
+// the counter word of a vec_scratch_bytes scratch (behind the block partials)
+inline unsigned *vec_scratch_counter(void *scratch) {
+  return (unsigned *)((char *)scratch + VEC_BLOCKS * sizeof(double));
+}
 cudaError_t vec_lincomb(long long n, int nv, const float *V, long long stride, const double *coef,
                         const float *x, double cx, float *y, cudaStream_t st);
 cudaError_t vec_dot(long long n, const float *x, const float *y, double *out, const double *scale,

@@ -17,18 +17,24 @@
 // ring of stored pairs) and the compact-form solve live on the device, in one
 // small state block; the host drives only the line search, whose decisions need
 // the trial's energy and slope.  An iteration whose first trial is accepted is
-// three or four launches: the direction and the first trial point
-// (lb_dir_kernel), the trial's energy, gradient and slope (fe_slope_launch: two
-// with a volume constraint), and, once the host has taken it, the new pair with every dot product of the update, whose last block
-// folds them into the state and solves for the next direction (lb_pair_kernel).  Each trial
+// five launches: the direction and the first trial point (lb_dir_kernel), the
+// trial's energy and gradient (two, fe_launch), its slope (trial_slope_kernel),
+// and, once the host has taken it, the new pair with every dot product of the
+// update, whose last block folds them into the state and solves for the next
+// direction (lb_pair_kernel).  Each trial
 // reads one block of six doubles (slope, energy, the direction's initial
 // slope, |g|^2 of the current point, the pairs in use, the next pair's slot),
 // so an iteration whose first trial is accepted reads the host once.
+//
+// The iteration amplifies the last place of an energy or of a dot product (one
+// unit in E moves the point after 25 iterations by up to 1e-2), so the iterates
+// are results only as long as every sum keeps its order: energies are summed over
+// fixed bricks (fe_kernel), dot products in the order of dot_kernel, whatever
+// kernel takes them.
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 #include <vector>
 
 #include "dsm_em.cuh"
@@ -311,7 +317,7 @@ __global__ void __launch_bounds__(256) lb_dir_kernel(long long n, int nv, const 
     }
     stv<W>(d + k, acc);
 #pragma unroll
-    for (int u = 0; u < W; u++) xx.v[u] += acc.v[u];
+    for (int u = 0; u < W; u++) xx.v[u] = __fadd_rn(xx.v[u], acc.v[u]);
     stv<W>(xt + k, xx);
   }
 }
@@ -319,15 +325,17 @@ __global__ void __launch_bounds__(256) lb_dir_kernel(long long n, int nv, const 
 // The accepted step's update in one pass over the vectors: the pair (s = step d,
 // y = gt - g into slot nxt), every stored vector against the new gradient gt
 // (v < hi is s_v, else y_{v-hi}; slots hi.. have never held a pair), and y.y,
-// gt.gt, s.s, all as carried-error sums.  gt is read once for all of them, W
-// elements of a vector per load, five vectors' loads in flight.  The grid's last
-// block sums the partials into dots and, on the update's last launch, folds them
-// into the state and solves for the next direction (lb_step).  128^3, m = 10:
-// 50.6 us, where seven launches (the pair in two, 20 dot products one vector per
-// block row at 59 us, three squares, two sums, the solve) took 91.  Bound by
-// latency (16 warps per SM at 118 registers); two block rows of ten vectors took
-// 70.9, staging in shared memory by asynchronous copies 56.
-constexpr int LB_NV = 20, LB_NK = LB_NV + 3, LB_BLOCKS = 152 * 2, LB_NT = 256;
+// gt.gt, s.s, all as carried-error sums.  Each sum is dot_kernel's to the bit: its
+// grid, its elements per thread and their order, its block's and its last sum's
+// trees.  So that loads are 16 bytes wide all the same, a thread holds four
+// neighbouring threads' sums of a quarter of the vectors: warps 2w and 2w + 1 take
+// vectors 5w .. 5w + 4 and one of the three squares.  The grid's last block sums the
+// partials into dots and, on the update's last launch, folds them into the state
+// and solves for the next direction (lb_step).  128^3, m = 10, caches cold: 68 us,
+// where seven launches (the pair in two, 20 dot products one vector per block row,
+// three squares, two sums, the solve) take 105; 193 MB of vectors, 28 us of copying.
+constexpr int LB_NV = 20, LB_NK = LB_NV + 3, LB_NT = 256;
+constexpr int LB_G = 4, LB_GV = LB_NV / LB_G;  // groups of threads, their vectors
 struct LbPair {
   long long n;
   int m, hi, v0, cnt, nxt, last;
@@ -345,71 +353,119 @@ __device__ __forceinline__ void lb_acc(FF &s, float a, float b) {
   s.hi = t.hi;
   s.lo += t.lo + p.lo;
 }
-template <bool PAIR, int W>
+// four elements from k on (not ALIGNED: those below n, 0 beyond, which add nothing)
+template <bool ALIGNED>
+__device__ __forceinline__ Pack<4> lb_ld(const float *p, long long k, long long n) {
+  if constexpr (ALIGNED) {
+    return ld<4>(p + k);
+  } else {
+    Pack<4> r;
+#pragma unroll
+    for (int c = 0; c < 4; c++) r.v[c] = k + c < n ? p[k + c] : 0.0f;
+    return r;
+  }
+}
+template <bool ALIGNED>
+__device__ __forceinline__ void lb_st(float *p, long long k, long long n, const Pack<4> &a) {
+  if constexpr (ALIGNED) {
+    stv<4>(p + k, a);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; c++)
+      if (k + c < n) p[k + c] = a.v[c];
+  }
+}
+template <bool SQUARES, bool ALIGNED>
 __global__ void __launch_bounds__(LB_NT, 2) lb_pair_kernel(const __grid_constant__ LbPair a) {
-  __shared__ FF sh[LB_NT / 32][32];
+  __shared__ FF sh[LB_NT / 32][LB_NK];
   __shared__ LbStepShared hs;
   __shared__ bool last;
-  FF acc[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int grp = threadIdx.x / (LB_NT / LB_G), q = threadIdx.x % (LB_NT / LB_G);
+  // this group's vectors: how many, where they are read, and which are the new pair's
+  // s and y (made from d and g here, not read back; -1: another group's)
+  const float *src[LB_GV];
+  const int cnt = a.cnt - grp * LB_GV;
+  int js = -1, jy = -1;
 #pragma unroll
-  for (int j = 0; j < 32; j++) acc[j] = FF{0.0f, 0.0f};
+  for (int j = 0; j < LB_GV; j++) {
+    const int v = a.v0 + grp * LB_GV + j;
+    const int slot = v < a.hi ? v : a.m + v - a.hi;
+    if (slot == a.nxt) js = j;
+    if (slot == a.m + a.nxt) jy = j;
+    src[j] = js == j ? a.d : jy == j ? a.g : a.V + (long long)slot * a.n;
+  }
+  FF acc[8][4];  // (of 8 sums, so that they halve over 8 lanes; the last two stay 0)
+#pragma unroll
+  for (int j = 0; j < 8; j++)
+#pragma unroll
+    for (int c = 0; c < 4; c++) acc[j][c] = FF{0.0f, 0.0f};
   const long long G = (long long)gridDim.x * LB_NT;
-  auto vec = [&](int j) {  // vector v0 + j
-    const int v = a.v0 + j;
-    return (long long)(v < a.hi ? v : a.m + v - a.hi) * a.n;
-  };
-  for (long long i = blockIdx.x * (long long)LB_NT + threadIdx.x; i < a.n / W; i += G) {
-    const long long k = W * i;
-    const Pack<W> gg = ld<W>(a.gt + k);
-    if (PAIR) {
-      Pack<W> ss = ld<W>(a.d + k), yy = ld<W>(a.g + k);
+  const long long T = blockIdx.x * (long long)LB_NT + 4 * q;
+  constexpr int U = 2;  // elements a grid apart in flight
+  for (long long k0 = T; k0 < a.n; k0 += U * G) {
+    Pack<4> gg[U], vv[U][LB_GV], ex[U];
 #pragma unroll
-      for (int u = 0; u < W; u++) {
-        ss.v[u] = a.step * ss.v[u];
-        yy.v[u] = gg.v[u] - yy.v[u];
-        lb_acc(acc[LB_NV], yy.v[u], yy.v[u]);
-        lb_acc(acc[LB_NV + 1], gg.v[u], gg.v[u]);
-        lb_acc(acc[LB_NV + 2], ss.v[u], ss.v[u]);
-      }
-      stv<W>(a.V + a.nxt * a.n + k, ss);  // (read again below by this thread)
-      stv<W>(a.V + (a.m + a.nxt) * a.n + k, yy);
+    for (int u = 0; u < U; u++) {
+      const long long k = k0 + u * G;
+      if (k >= a.n) break;
+      gg[u] = lb_ld<ALIGNED>(a.gt, k, a.n);
+#pragma unroll
+      for (int j = 0; j < LB_GV; j++)
+        if (j < cnt) vv[u][j] = lb_ld<ALIGNED>(src[j], k, a.n);
+      if (SQUARES && (grp == 0 || grp == 2)) ex[u] = lb_ld<ALIGNED>(grp == 0 ? a.g : a.d, k, a.n);
     }
 #pragma unroll
-    for (int j0 = 0; j0 < LB_NV; j0 += 5) {
-      if (j0 + 5 <= a.cnt) {
-        Pack<W> vv[5];
+    for (int u = 0; u < U; u++) {
+      const long long k = k0 + u * G;
+      if (k >= a.n) break;
 #pragma unroll
-        for (int e = 0; e < 5; e++) vv[e] = ld<W>(a.V + vec(j0 + e) + k);
+      for (int j = 0; j < LB_GV; j++) {
+        if (j >= cnt) continue;
+        if (js == j) {
 #pragma unroll
-        for (int e = 0; e < 5; e++)
+          for (int c = 0; c < 4; c++) vv[u][j].v[c] = a.step * vv[u][j].v[c];
+          lb_st<ALIGNED>(a.V + a.nxt * a.n, k, a.n, vv[u][j]);
+        }
+        if (jy == j) {
 #pragma unroll
-          for (int u = 0; u < W; u++) lb_acc(acc[j0 + e], vv[e].v[u], gg.v[u]);
-      } else {
+          for (int c = 0; c < 4; c++) vv[u][j].v[c] = gg[u].v[c] - vv[u][j].v[c];
+          lb_st<ALIGNED>(a.V + (a.m + a.nxt) * a.n, k, a.n, vv[u][j]);
+        }
 #pragma unroll
-        for (int e = 0; e < 5; e++)
-          if (j0 + e < a.cnt) {
-            const Pack<W> vv = ld<W>(a.V + vec(j0 + e) + k);
+        for (int c = 0; c < 4; c++) lb_acc(acc[j][c], vv[u][j].v[c], gg[u].v[c]);
+      }
+      if (SQUARES && grp < 3) {  // y.y, gt.gt, s.s
 #pragma unroll
-            for (int u = 0; u < W; u++) lb_acc(acc[j0 + e], vv.v[u], gg.v[u]);
-          }
+        for (int c = 0; c < 4; c++) {
+          const float v = grp == 0   ? gg[u].v[c] - ex[u].v[c]
+                          : grp == 1 ? gg[u].v[c]
+                                     : a.step * ex[u].v[c];
+          lb_acc(acc[LB_GV][c], v, v);
+        }
       }
     }
   }
-  // 32 sums across the warp by halving: lane l ends with sum l (31 pair sums
-  // instead of 5 x 23)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // block_reduce_ff's tree over the 32 threads whose sums eight lanes hold: 16, 8 and
+  // 4 apart are lanes 4, 2 and 1 apart (by halving: lane l of the eight ends with
+  // sum l), 2 and 1 apart lie in one thread
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 4; o > 0; o >>= 1) {
     const bool up = lane & o;
 #pragma unroll
-    for (int e = 0; e < o; e++) {
-      const FF keep = up ? acc[e + o] : acc[e], send = up ? acc[e] : acc[e + o];
-      const FF got = {__shfl_xor_sync(0xffffffffu, send.hi, o),
-                      __shfl_xor_sync(0xffffffffu, send.lo, o)};
-      acc[e] = ff_add(keep, got);
-    }
+    for (int e = 0; e < o; e++)
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const FF keep = up ? acc[e + o][c] : acc[e][c], send = up ? acc[e][c] : acc[e + o][c];
+        const FF got = {__shfl_xor_sync(0xffffffffu, send.hi, o),
+                        __shfl_xor_sync(0xffffffffu, send.lo, o)};
+        acc[e][c] = ff_add(keep, got);
+      }
   }
-  sh[warp][lane] = acc[0];
+  const FF mine = ff_add(ff_add(acc[0][0], acc[0][2]), ff_add(acc[0][1], acc[0][3]));
+  const int sum = lane & 7;  // of the group; its place among the block's
+  if (sum < LB_GV) sh[q >> 3][grp * LB_GV + sum] = mine;
+  else if (sum == LB_GV && grp < 3) sh[q >> 3][LB_NV + grp] = mine;
   __syncthreads();
   if (threadIdx.x < LB_NK) {
     FF r = sh[0][threadIdx.x];
@@ -425,25 +481,17 @@ __global__ void __launch_bounds__(LB_NT, 2) lb_pair_kernel(const __grid_constant
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int j = warp; j < LB_NK; j += LB_NT / 32) {  // a warp per sum
-    const volatile double *p = a.partials + (long long)j * gridDim.x;
-    double t = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) t += p[b];
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  for (int j = warp; j < LB_NK; j += LB_NT / 32) {
+    const double t = warp_sum256(a.partials + (long long)j * gridDim.x, gridDim.x, 1);
     if (lane == 0) {
       const int v = a.v0 + j;
       if (j < a.cnt) a.dots[v < a.hi ? v : a.m + v - a.hi] = t;
-      else if (PAIR && j >= LB_NV) a.dots[2 * a.m + j - LB_NV] = t;
+      else if (SQUARES && j >= LB_NV) a.dots[2 * a.m + j - LB_NV] = t;
     }
   }
   __syncthreads();
   if (threadIdx.x == 0) *a.counter = 0u;
   if (a.last && warp == 0) lb_step(a.s, a.dots, a.m, a.sy, hs);
-}
-template <bool PAIR, int W>
-cudaError_t lb_pair_launch(const LbPair &a, int grid, cudaStream_t st) {
-  lb_pair_kernel<PAIR, W><<<grid, LB_NT, 0, st>>>(a);
-  return cudaGetLastError();
 }
 
 // drop the stored pairs (after a line search that found no step)
@@ -484,7 +532,7 @@ struct Minimiser {
   float *xb[2], *gb[2], *d, *hist;
   double *E[2], *dots, *vout;  // vout: the state's read-back block
   LbState *state;
-  void *fe_scr, *vec_scr, *dots_scr, *slope_scr;
+  void *fe_scr, *vec_scr, *dots_scr;
   int hi = 0;  // slots that have held a pair
 
   cudaError_t evaluate(const float *x, double *e_out, float *g_out) {
@@ -498,7 +546,7 @@ struct Minimiser {
     a.c1 = active == 2 ? fixed : x;
     a.c2 = active == 2 ? x : fixed;
     a.grad = g_out;
-    return fe_launch(kind, a, dP, kcs, V0, e_out, nullptr, fe_scr, st);
+    return fe_launch(kind, a, dP, kcs, V0, e_out, nullptr, fe_scr, st, true);
   }
   // device doubles -> host (pageable copy, waits for the stream)
   cudaError_t read(double *h, const double *dv, int count) {
@@ -508,6 +556,8 @@ struct Minimiser {
   }
   // energy and slope at the trial point xt = x + a d (made: xt is there
   // already), read back with the rest of the state's block (rb: 6 doubles).
+  // Two fluids: the energy goes straight into the block, and the constraint's
+  // constant is added to the gradient in the same pass that takes the slope.
   cudaError_t trial(double a, const float *x, float *xt, double *Et, float *gt, double *rb,
                     bool made) {
     cudaError_t e = made ? cudaSuccess : vec_lincomb(n, 1, d, n, &a, x, 1.0, xt, st);
@@ -521,8 +571,10 @@ struct Minimiser {
       b.c1 = active == 2 ? fixed : xt;
       b.c2 = active == 2 ? xt : fixed;
       b.grad = gt;
-      b.dir = d;
-      if (e == cudaSuccess) e = fe_slope_launch(kind, b, dP, kcs, V0, vout + 1, vout, slope_scr, st);
+      const double *cst = nullptr;
+      if (e == cudaSuccess)
+        e = fe_launch(kind, b, dP, kcs, V0, vout + 1, nullptr, fe_scr, st, true, &cst);
+      if (e == cudaSuccess) e = vec_trial_slope(n, cst, gt, d, vout, vec_scr, st);
     }
     if (e == cudaSuccess) e = read(rb, vout, 6);
     return e;
@@ -545,15 +597,19 @@ struct Minimiser {
     a.dots = dots;
     a.s = state;
     a.hi = hi = std::max(hi, nxt + 1);
-    const int w = n % 4 == 0 ? 4 : 1;  // (every vector starts n reals after another)
-    const int grid = (int)std::min<long long>((n / w + LB_NT - 1) / LB_NT, LB_BLOCKS);
+    const int grid = (int)std::min<long long>((n + LB_NT - 1) / LB_NT, VEC_BLOCKS);
     for (int v = 0; v < 2 * hi; v += LB_NV) {
       a.v0 = v;
       a.cnt = std::min(LB_NV, 2 * hi - v);
       a.last = v + LB_NV >= 2 * hi;
-      const cudaError_t e =
-          v == 0 ? (w == 4 ? lb_pair_launch<true, 4>(a, grid, st) : lb_pair_launch<true, 1>(a, grid, st))
-                 : (w == 4 ? lb_pair_launch<false, 4>(a, grid, st) : lb_pair_launch<false, 1>(a, grid, st));
+      if (n % 4 == 0) {  // (every vector starts n reals after another)
+        if (v == 0) lb_pair_kernel<true, true><<<grid, LB_NT, 0, st>>>(a);
+        else lb_pair_kernel<false, true><<<grid, LB_NT, 0, st>>>(a);
+      } else {
+        if (v == 0) lb_pair_kernel<true, false><<<grid, LB_NT, 0, st>>>(a);
+        else lb_pair_kernel<false, false><<<grid, LB_NT, 0, st>>>(a);
+      }
+      const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -564,7 +620,7 @@ struct Minimiser {
 
 // The L-BFGS loop over M.n-vectors (x in d_x, overwritten), workspace w laid
 // out by lbfgs_layout_n.
-static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *d_x, double tol,
+static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[11], float *d_x, double tol,
                      long long max_iter, dsm_lbfgs_info *info) {
   const int m = M.m;
   M.xb[0] = d_x;
@@ -581,7 +637,6 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
   M.fe_scr = w + off[8];
   M.vec_scr = w + off[9];
   M.dots_scr = w + off[10];
-  M.slope_scr = w + off[11];
   const long long n = M.n;
   cudaStream_t st = M.st;
   // 16-byte loads: every vector of the workspace starts a multiple of n reals
@@ -598,7 +653,7 @@ static dsm_status run_lbfgs(Minimiser &M, char *w, const size_t off[12], float *
   CK(cudaMemsetAsync(M.hist, 0, (size_t)2 * m * n * sizeof(float), st));
   CK(cudaMemsetAsync(M.dots, 0, (size_t)(2 * m + 3) * sizeof(double), st));
   CK(cudaMemsetAsync(M.dots_scr, 0, 256, st));
-  CK(cudaMemsetAsync(M.slope_scr, 0, 256, st));
+  CK(cudaMemsetAsync(vec_scratch_counter(M.vec_scr), 0, sizeof(unsigned), st));
   lb_init_kernel<<<1, 1, 0, st>>>(M.state);
   CK(cudaGetLastError());
   int cur = 0;  // x = xb[cur], g = gb[cur], E = E[cur]
@@ -770,7 +825,7 @@ dsm_status dsm_lbfgs_compact(int k, const double *SY, const double *YY, const do
 
 // Workspace of an L-BFGS run over n-vectors whose energy needs fe_bytes of
 // scratch.
-static size_t lbfgs_layout_n(long long n, int m, size_t fe_bytes, size_t off[12]) {
+static size_t lbfgs_layout_n(long long n, int m, size_t fe_bytes, size_t off[11]) {
   size_t o = 0;
   auto take = [&](size_t bytes) {
     size_t at = o;
@@ -787,12 +842,11 @@ static size_t lbfgs_layout_n(long long n, int m, size_t fe_bytes, size_t off[12]
   off[7] = take(sizeof(LbState));                 // the pair bookkeeping on the device
   off[8] = take(fe_bytes);
   off[9] = take(vec_scratch_bytes(n));
-  off[10] = take(256 + (size_t)LB_BLOCKS * LB_NK * sizeof(double));
-  off[11] = take(fe_slope_scratch_bytes());
+  off[10] = take(256 + (size_t)VEC_BLOCKS * LB_NK * sizeof(double));
   return o;
 }
 
-static size_t lbfgs_layout(const dsm_params *p, int m, size_t off[12]) {
+static size_t lbfgs_layout(const dsm_params *p, int m, size_t off[11]) {
   return lbfgs_layout_n((long long)p->nx * p->ny * p->nz, m,
                         fe_scratch_bytes(p->lattice, p->nx, p->ny, p->nz), off);
 }
@@ -800,7 +854,7 @@ static size_t lbfgs_layout(const dsm_params *p, int m, size_t off[12]) {
 dsm_status dsm_lbfgs_workspace_bytes(const dsm_params *p, int m, size_t *bytes) {
   if (!p || !bytes || m < 1 || 2 * m > LINCOMB_MAX) return DSM_E_INVAL;
   if (p->nx < 1 || p->ny < 1 || p->nz < 1) return DSM_E_INVAL;
-  size_t off[12];
+  size_t off[11];
   *bytes = lbfgs_layout(p, m, off);
   return DSM_OK;
 }
@@ -823,7 +877,7 @@ dsm_status dsm_lbfgs_minimize(const dsm_params *p, const float *d_fixed,
   double kap[3];
   dsm_status s = dsm_kappa(p, kap);
   if (s != DSM_OK) return s;
-  size_t off[12];
+  size_t off[11];
   if (work_bytes < lbfgs_layout(p, m, off) || ((uintptr_t)d_work & 255u)) return DSM_E_WORKSPACE;
   memset(info, 0, sizeof(*info));
 
@@ -849,7 +903,7 @@ dsm_status dsm_lbfgs_multi_workspace_bytes(const dsm_params *p, int nfluid, int 
   if (p->nx < 1 || p->ny < 1 || p->nz < 1) return DSM_E_INVAL;
   if (p->lattice != DSM_D2Q9 && p->lattice != DSM_D3Q19) return DSM_E_INVAL;
   if (nfluid < 2 || nfluid > FEM_MAX_NF + 1) return DSM_E_INVAL;
-  size_t off[12];
+  size_t off[11];
   const long long nodes = (long long)p->nx * p->ny * p->nz;
   *bytes = lbfgs_layout_n(nodes * (nfluid - 1), m,
                           fe_multi_scratch_bytes(p->lattice, p->nx, p->ny, p->nz, nfluid - 1),
@@ -869,7 +923,7 @@ dsm_status dsm_lbfgs_minimize_multi(const dsm_params *p, int nfluid, const doubl
   dsm_status s = fem_args_of(p, nfluid, kappa, dP, kcs, V0, &M.fm, &M.fcons);
   if (s != DSM_OK) return s;
   const long long nodes = (long long)p->nx * p->ny * p->nz;
-  size_t off[12];
+  size_t off[11];
   const size_t need = lbfgs_layout_n(
       nodes * (nfluid - 1), m, fe_multi_scratch_bytes(p->lattice, p->nx, p->ny, p->nz, nfluid - 1),
       off);

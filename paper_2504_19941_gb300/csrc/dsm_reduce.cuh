@@ -82,4 +82,29 @@ __device__ __forceinline__ void block_reduce_ff(const float (&v)[NV], const int 
   block_reduce_ff<NV>(p, is_max, out);
 }
 
+// Sum of p[0], p[stride], .. (n of them) by one warp, returned in lane 0, equal to
+// the bit to 256 threads that each add every 256th and a shared-memory
+// tree over them (last_block_sum): lane l has the threads l, l + 32, ..
+__device__ __forceinline__ double warp_sum256(const double *p, int n, int stride) {
+  const int lane = threadIdx.x & 31;
+  double t[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) t[i] = 0.0;
+  for (int b = lane; b < n + lane; b += 256) {
+    double v[8];  // all in flight (from L2: other blocks have written them)
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+      v[i] = b + 32 * i < n ? __ldcg(p + (long long)(b + 32 * i) * stride) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) t[i] += v[i];
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < o; i++) t[i] += t[i + o];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_down_sync(0xffffffffu, t[0], o);
+  return t[0];
+}
+
 }  // namespace dsm
