@@ -490,7 +490,7 @@ cudaError_t m_enter(dsm_lattice *h) {
   h->mc = 0;
   h->mom = true;
   h->mstepped = true;
-  h->mcp = h->mpk = false;
+  h->mcp = h->mpk = h->tp = h->tcan = false;
   return cudaSuccess;
 }
 
@@ -881,7 +881,7 @@ dsm_status dsm_set_fluid(dsm_lattice *h, const void *d_c2) {
     if (e == cudaSuccess) e = h->tab.mom_init(m_raw(h, 1), d_c2, 0, h->stream);  // writes buffer 0
     h->mc = 0;
     h->mom = true;
-    h->mcp = h->mpk = h->mfit = h->mstepped = false;
+    h->mcp = h->mpk = h->mfit = h->mstepped = h->tp = h->tcan = false;
   } else {
     m_drop(h);
     LBRaw r = raw_of(h, 1);  // writes buffer 0
@@ -1547,7 +1547,7 @@ dsm_status dsm_batch_step(dsm_lattice *const *hs, int n, const long long *nsteps
       h->cur ^= 1;
       h->step++;
       h->g_implicit = h->mfit = true;
-      h->moments_ready = false;
+      h->moments_ready = h->tp = h->tcan = false;
       left[i]--;
     }
     if (left[i] == 0) continue;

@@ -1,0 +1,67 @@
+"""A state's form when it changes hands: checkpoints restored into lattices of
+other relaxation times or faces, which hold and step their state otherwise.
+Everything compared here is the same operations on the same numbers: equal bits.
+"""
+import pytest
+
+import synthetic as S
+from dsm_helpers import gpu_lattice
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2504_19941_gb300 import _lib  # noqa: E402
+
+
+def _case(shape=(45, 13), **kw):
+    sd = S.sphere_sd(shape, [s / 3 for s in shape], 4.0)
+    c2 = S.drop_c2(shape, [s / 2 for s in shape], 4.0, 1.0, sd, 1.0).ravel()
+    case = S.Case("forms", "D2Q9" if len(shape) == 2 else "D3Q19", shape, sd.ravel(),
+                  c2 + S.perturbation(3, sd.size), theta_deg=70.0, g23=0.01, g12=0.01,
+                  alpha_s=1.0, body=(1e-6, -2e-6, 0.0))
+    for k, v in kw.items():
+        setattr(case, k, v)
+    return case
+
+
+def _equal(a, b):
+    return all(torch.equal(u, v) for u, v in zip(a.populations(), b.populations()))
+
+
+def _batch(lat, n):
+    nb = _lib.dsm_batch_scratch_bytes([lat.h])
+    _lib.dsm_batch_step([lat.h], [n], torch.empty(nb, dtype=torch.uint8, device="cuda"), nb)
+
+
+def _quads():
+    # held as f and quads (A, C, u) by a lattice with two viscosities
+    donor = gpu_lattice(_case(tau3=0.6), "f64")
+    donor.step(4)
+    return donor.state()
+
+
+def _restored(st, **kw):
+    lat = gpu_lattice(_case(**kw), "f64")
+    lat.set_state(st)
+    return lat
+
+
+def test_a_batched_step_on_moments_ends_the_quads():
+    st = _quads()
+    ref, lat = _restored(st), _restored(st)
+    ref.step(1)
+    _batch(lat, 1)
+    assert _equal(lat, ref)
+    assert _equal(_restored(lat.state()), ref)
+
+
+def test_a_new_fluid_on_moments_ends_the_quads():
+    lat, new = _restored(_quads()), gpu_lattice(_case(), "f64")
+    for x in (lat, new):
+        x.set_step_form("two_pass")
+        x.set_fluid(torch.as_tensor(_case().c2, dtype=x.real, device="cuda"))
+        x.field("mu")
+        x.step(1)
+    assert _equal(lat, new)
