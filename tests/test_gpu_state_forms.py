@@ -58,9 +58,11 @@ def test_a_batched_step_on_moments_ends_the_quads():
 
 
 def test_a_new_fluid_on_moments_ends_the_quads():
-    lat, new = _restored(_quads()), gpu_lattice(_case(), "f64")
+    lat, new = gpu_lattice(_case(), "f64"), gpu_lattice(_case(), "f64")
+    lat.set_step_form("two_pass")
+    new.set_step_form("two_pass")
+    lat.set_state(_quads())
     for x in (lat, new):
-        x.set_step_form("two_pass")
         x.set_fluid(torch.as_tensor(_case().c2, dtype=x.real, device="cuda"))
         x.field("mu")
         x.step(1)
