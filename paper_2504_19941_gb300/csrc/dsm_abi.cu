@@ -1265,7 +1265,7 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
   if (hd.magic != kStateMagic || hd.version != 1 || hd.lattice != h->kind ||
       hd.precision != h->prm.precision || hd.nx != h->prm.nx || hd.ny != h->prm.ny ||
       hd.nz != h->prm.nz || hd.pitch != h->pitch || hd.implicit < 0 || hd.implicit > 3 ||
-      (hd.implicit == 3 && !h->tok) ||
+      (hd.implicit == 3 && h->kind != DSM_D2Q9) ||
       (hd.implicit == 2 && (!h->tab.mom_expand || !(hd.rho > 0.0))) || hd.step < 0)
     return DSM_E_INVAL;
   const char *d = (const char *)d_src;
@@ -1310,6 +1310,10 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
     h->has_fluid = true;
     h->latched = false;
     h->moments_ready = false;
+    if (!h->tok) {  // a handle that never steps from quads: the canonical planes
+      if (t_copy(h) != cudaSuccess) return DSM_E_CUDA;
+      h->tp = h->tcan = false;
+    }
     return DSM_OK;
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->g[0], d + L.g, pop, cudaMemcpyDeviceToDevice, st);
