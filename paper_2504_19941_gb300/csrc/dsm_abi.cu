@@ -1176,6 +1176,7 @@ struct StateHeader {
   int lattice, precision, nx, ny, nz, implicit;
   long long step, pitch;
   double rho;
+  int rest;  // implicit = 2: not stepped since dsm_set_fluid
 };
 struct StateLayout {
   size_t f, g, g0, C, M, total;
@@ -1222,6 +1223,7 @@ dsm_status dsm_get_state(dsm_lattice *h, void *d_dst, size_t bytes) {
   hd.nz = h->prm.nz;
   hd.implicit = h->mom ? 2 : h->tp ? 3 : h->g_implicit ? 1 : 0;
   hd.rho = h->sp.rho3;
+  hd.rest = h->mom && !h->mstepped;
   hd.step = h->step;
   hd.pitch = h->pitch;
   char *d = (char *)d_dst;
@@ -1277,7 +1279,8 @@ dsm_status dsm_set_state(dsm_lattice *h, const void *d_src, size_t bytes) {
     e = cudaMemcpyAsync(h->g[0], d + L.f, mom_reals(h->kind) * real, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int) * 4, st);
     h->mc = 0;
-    h->mom = h->mstepped = true;
+    h->mom = true;
+    h->mstepped = !hd.rest;
     if (e == cudaSuccess && (!m_active(h) || hd.rho != h->sp.rho3)) {
       // a handle that holds its state otherwise: expanded with the density the
       // moments belong to

@@ -86,3 +86,15 @@ def test_quads_into_a_lattice_without_that_step(prec, kw):
             assert float((a - b).abs().max()) <= (1e-14 if prec == "f64" else 2.0 ** -11)
         lat.step(3)
         ref.step(3)
+
+
+@pytest.mark.parametrize("shape", [(45, 13), (33, 9, 5)])
+def test_a_state_at_rest_keeps_its_storage_form(shape):
+    # dsm_get_g_storage: g of a new fluid are populations until the first step
+    lat, other = gpu_lattice(_case(shape), "f32"), gpu_lattice(_case(shape), "f32")
+    other.step(2)
+    other.set_state(lat.state())
+    assert not lat.g_implicit and not other.g_implicit
+    lat.step(2)
+    other.step(2)
+    assert other.g_implicit and _equal(lat, other)
