@@ -350,7 +350,7 @@ def run_gpu(args, rank, world):
         one_step()
     torch.cuda.synchronize()
     g_eq = lat.g_implicit
-    # (the automatic form's kernels: include/dsm.h, dsm_step_info)
+    # (the automatic form's kernels: include/dsm.h, dsm_set_step_form)
     moments = single and args.rho3 == 1.0 and args.tau3 == 1.0
     if moments:
         k2_b, k1_b = lu_bytes_moments(store), 0
@@ -442,8 +442,6 @@ def run_gpu(args, rank, world):
                             "kernel": "mom_wall_kernel, mom_step3_kernel (step on moments, %d z "
                                       "planes per block)" % _lib.dsm_step_info(h)[1]
                                       if moments else
-                                      "moments_eq_tiled_kernel, node_kernel<D3Q19,f32,stage2,step,"
-                                      "g_eq,density contrast>" if single and args.rho3 != 1.0 else
                                       "zstep_kernel<f32,f32> (one pass per step, %d z planes "
                                       "per block)" % _lib.dsm_step_info(h)[1]
                                       if single else
@@ -457,7 +455,7 @@ def run_gpu(args, rank, world):
                             "measured_frac": (traffic / n * lups_gpu / 1e9 / peak) if traffic else None,
                             "b_min_per_lu": b_min, "useful_frac": b_min * lups_gpu / 1e9 / peak},
                "clocks": clk.summary(), "e2e": e2e,
-               "gpu_launches": (1 if single and not moments and args.rho3 == 1.0 else 2)
+               "gpu_launches": (1 if single and not moments else 2)
                                * args.steps,
                "cpu_baseline": cb,
                "observables": {"mass_c2": obs["mass_c2"], "max_u": obs["max_u"]}}

@@ -213,24 +213,26 @@ dsm_status dsm_set_body_force(dsm_lattice *h, const double *body);
  * as ONE pass: blocks march 32 x 8 tiles (the last ones ragged) up runs of z
  * planes, rebuild the C of
  * the step on chip from the staged (A, u, C) of the previous collision and
- * collide.  The results are the same step (the same per-node arithmetic, so
+ * collide.  Where every relaxation time is 1 and the densities are equal it marches
+ * the moments that fix the populations instead, on lattices of any size; D2Q9
+ * lattices with tau_g = 1 and periodic or mirror faces collide tile by tile in
+ * one launch; and with a density contrast in FP32 arithmetic lattices of 180000
+ * nodes and more run the two passes, the faster form there, unless zrun is given.
+ * The results are the same step (the same per-node arithmetic, so
  * equal to the two-pass step up to nothing but FP32 contraction order); the
  * state then lives in padded buffers of the workspace and is converted back
  * before any call that reads it (fields, observables, populations, checkpoint,
  * dsm_batch_step).  DSM_STEP_TWO_PASS always uses the two passes.
  *   zrun: z planes per block of the one-pass step, 0 = chosen from the lattice
  *   size and the GPU's resident blocks (a tuning knob; results do not depend on
- *   it).  DSM_E_INVAL for an unknown form or zrun < 0. */
+ *   it beyond that order).  DSM_E_INVAL for an unknown form or zrun < 0. */
 enum { DSM_STEP_AUTO = 0, DSM_STEP_TWO_PASS = 1 };
 dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun);
 
-/* Whether the one-pass step applies to the lattice's size, form and faces
- * (*single_pass = 1) and with how many z planes per block (*zrun; 0 for the
- * two-pass step).  The automatic form takes the fastest kernels for the same
- * step where others are faster: moments in the place of populations where every
- * relaxation time is 1, two passes with a density contrast in FP32 arithmetic
- * from 180000 nodes up.
- * Either pointer may be NULL. */
+/* Whether dsm_step marches runs of z planes in one pass (*single_pass = 1) and
+ * with how many z planes per block (*zrun; 0 where it does not).  Lattices that
+ * have no such runs (D2Q9, and D3Q19 narrower than a 32 x 8 tile) answer 0,
+ * in however many launches their step runs.  Either pointer may be NULL. */
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun);
 
 /* Observables of the current state; synchronises the stream.  Returns

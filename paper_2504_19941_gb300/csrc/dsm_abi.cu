@@ -278,9 +278,11 @@ bool z_form(const dsm_lattice *h) {
 // spilled, 378 us, and as a plane of the moments pass changed nothing, 181 + 52).
 // FP64, bound by its pipe, keeps the single pass, and so do lattices too small to
 // pay for a second launch (20 steps and two fields, single pass and two: 40 x 40 x 64
-// 552 and 587 us, 64^3 737 and 684, 120 x 100 x 80 2138 and 1898).
+// 552 and 587 us, 64^3 737 and 684, 120 x 100 x 80 2138 and 1898), and so does a
+// handle that is given its planes per block (dsm_set_step_form).
 bool z_active(const dsm_lattice *h) {
-  return z_form(h) && !(h->sp.rho_contrast && h->tab.real_bytes == 4 && h->N >= 180000);
+  return z_form(h) &&
+         !(h->zrun == 0 && h->sp.rho_contrast && h->tab.real_bytes == 4 && h->N >= 180000);
 }
 
 // Canonical g_eq state -> padded buffers (buffer 0), and padded C1.
@@ -996,7 +998,7 @@ dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun) {
 
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun) {
   if (!h) return DSM_E_INVAL;
-  const bool single = z_form(h);
+  const bool single = m_active(h) ? z_form(h) : z_active(h);
   if (single_pass) *single_pass = single ? 1 : 0;
   if (zrun) *zrun = single ? (h->zrun > 0 ? h->zrun : m_active(h) ? m_zrun(h) : z_auto_run(h)) : 0;
   return DSM_OK;
