@@ -828,8 +828,11 @@ dsm_status dsm_relax_solid(dsm_lattice *h, const unsigned char *d_mask, int step
       r.rho = 1.0;
     }
     e = h->tab.mom_relax(a[1], mr, 0, h->C1, h->stream);
-    for (int t = 0; t < steps && e == cudaSuccess; t++)
+    for (int t = 0; t < steps && e == cudaSuccess; t++) {
+      a[t & 1].step = (unsigned)t;
       e = h->tab.mom_relax(a[t & 1], mr, 1, nullptr, h->stream);
+    }
+    a[steps & 1].step = (unsigned)steps;
     if (e == cudaSuccess) e = h->tab.mom_relax(a[steps & 1], mr, 2, h->C1, h->stream);
     h->sp.beta = h->prm.beta;
     h->sp.omega = h->prm.omega;

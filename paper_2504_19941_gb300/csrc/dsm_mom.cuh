@@ -67,7 +67,7 @@ struct MomArgs {
   T k[MOM_NF], ak[MOM_NF];  // kappa and alpha^2 kappa of the free fluids
   T kl, akl;                // the dependent fluid's
   T rho, irho, body[3], alpha_s;
-  unsigned step;       // number of the step (DI: see mom_dither)
+  unsigned seed;       // MOM_SEED x the number of the step (mom_add)
 };
 
 // reals of one buffer per node, two fluids
@@ -86,21 +86,33 @@ template <class T>
 __device__ __forceinline__ T mom_bn(T v) {  // b(-v)
   return ml(v, fm(T(4.5), v, T(-3)));
 }
-// DI: C + d rounded without bias.  Where C is near 1, d is mostly less than half
-// a unit in C's last place and would round away, while the nodes with small C
-// that exchange with it keep what they receive: FP32 lattices gain about 6e-10 of
-// their liquid per step (96 x 64 x 48).  The lattices with 16-bit populations
-// conserve it better, and still do with a d to which a fraction in (-1/2, 1/2) of
-// that unit is added, a hash of the node and the step, so that it is the same in
-// every form of the step.
-__device__ __forceinline__ float mom_dither(float c, float d, int n, unsigned step) {
-  unsigned h = (unsigned)n * 0x9e3779b1u + step * 0x85ebca77u;
+// A step adds to each C a difference d, and two things in it would make an FP32
+// lattice gain or lose liquid steadily (24^3, 10000 steps: -5.1e-5 of it; with f as
+// populations, whose rounding shakes u and so d, -1.6e-5; as it is, 1e-8):
+//   - Where C is near 1, d is mostly less than half a unit in C's last place and
+//     would round away, while the nodes with small C that exchange with it keep what
+//     they receive.  mom_add adds a fraction in (-1/2, 1/2) of that unit to d: C + d
+//     rounded without bias.  The fraction is a hash of d and the step, no function of
+//     the node, so that every form and tile of the step rounds alike and fields keep
+//     their symmetries.
+//   - A leaves a node as 1 - w_0 and arrives as the weights, which in FP32 do not add
+//     up to it.  All of them are 2^k times the last one in any precision, so A leaves
+//     as mom_out (24 in 3D, 20 in 2D) times that weight.
+// 256 x 256 x 192: 275 -> 284 us per step for both.
+template <class L>
+__host__ __device__ constexpr int mom_out() {
+  return L::D == 3 ? 24 : 20;
+}
+constexpr unsigned MOM_SEED = 0x85ebca77u;
+__device__ __forceinline__ float mom_add(float c, float d, unsigned seed) {
+  unsigned h = (__float_as_uint(d) ^ seed) * 0x9e3779b1u;
   h = (h ^ (h >> 15)) * 0x2c1b3c6du;
   const float r = sb(__uint_as_float((h >> 9) | 0x3f800000u), 1.5f);
   const unsigned m = __float_as_uint(c) & 0x7fffffffu;
   const float e = __uint_as_float((m - (m != 0u)) & 0x7f800000u);  // 2^23 units (below c)
-  return fm(e, ml(r, 1.1920928955078125e-7f), d);
+  return ad(c, fm(e, ml(r, 1.1920928955078125e-7f), d));
 }
+__device__ __forceinline__ double mom_add(double c, double d, unsigned) { return ad(c, d); }
 
 template <class T>
 __device__ __forceinline__ T mom_well(T c) {
@@ -341,8 +353,8 @@ __device__ __forceinline__ void cp_async_bytes(unsigned dst, const void *src) {
 // The kernel it replaced for these lattices (populations f, tensor-memory
 // loads, dsm_zstep.cuh) takes 0.572 ms there: 196 B and 1189 instructions per
 // node against 81 B and 425.
-// With the wall pass, whole steps: 256 x 256 x 192 0.572 -> 0.256 ms, 101^3
-// 76.4 -> 42.0 us.
+// With the wall pass, whole steps: 256 x 256 x 192 0.572 -> 0.284 ms, 101^3
+// 76.4 -> 42.9 us.
 // ---------------------------------------------------------------------------
 constexpr int M3_X = 32, M3_HX = M3_X + 4, M3_HP = M3_HX + 1, M3_CX = M3_X + 2, M3_RING = 3;
 
@@ -374,9 +386,9 @@ __device__ __forceinline__ void mom_cross_b(T v, T uz, T &b0, T &bp, T &bm) {
   }
 }
 
-template <class T, int NF, int TY, int RY, bool DI>
+template <class T, int NF, int TY, int RY>
 __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, int z0, int z1,
-                                         unsigned step, unsigned char *sm) {
+                                         unsigned seed, unsigned char *sm) {
   using SM = M3Smem<T, NF, TY>;
   constexpr int NT = M3_X * TY / RY;
   constexpr int HP = M3_HP;  // staged row: nodes, pitch
@@ -489,10 +501,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
   // plane, h = 9/2 u_z^2 and s = u_z (3 + 9 v), b(v +- u_z) = b(v) + h +- s: the
   // links c_z = +-1 of a point share all but the sign of one term, and so do
   // their sums.  Row by row, each point read once for all R nodes.
-  // (DI: lx, ly, the first node in the tile; qz, the target plane's nodes)
-  int qz = 0;
-  auto links = [&](unsigned slot, int k, auto *gs, auto &Cd, auto joint, auto rows, int lx,
-                   int ly) {
+  auto links = [&](unsigned slot, int k, auto *gs, auto &Cd, auto joint, auto rows) {
     constexpr bool F = decltype(joint)::value;
     constexpr int R = decltype(rows)::value;
     T s0[R][NF], sE[R][NF], sQ[R][NF], gc[R][NF], out[R][NF], cn[R][NF];
@@ -516,7 +525,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
             const T uu = fm(uz, uz, fm(p.uy, p.uy, ml(p.ux, p.ux)));
 #pragma unroll
             for (int f = 0; f < NF; f++) {
-              out[j][f] = fm(ml(T(1.5), p.C[f]), uu, ml(T(1) - w0, p.A[f]));
+              out[j][f] = fm(ml(T(1.5), p.C[f]), uu, ml(T(mom_out<Lat<1>>()), ml(w2, p.A[f])));
               gP[j][f] = ml(w1, fm(p.C[f], h, p.A[f]));
               gR[j][f] = ml(w1, ml(p.C[f], z3));
               cn[j][f] = p.C[f];
@@ -614,14 +623,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
 #pragma unroll
         for (int f = 0; f < NF; f++) {
           const T P = fm(w2, ad(s0[j][f], sE[j][f]), gP[j][f]), Q = fm(w2, sQ[j][f], gR[j][f]);
-          T d = ad(gs[j].mid[f], sb(P, Q));
-          if constexpr (DI) {
-            int gx = x0 + lx, gy = y0 + ly + j;
-            gx += gx < 0 ? nx : gx >= nx ? -nx : 0;
-            gy += gy < 0 ? ny : gy >= ny ? -ny : 0;
-            d = mom_dither(gs[j].ck[f], d, qz + gx + nx * gy, step);
-          }
-          Cd[j][f] = ad(gs[j].ck[f], d);
+          Cd[j][f] = mom_add(gs[j].ck[f], ad(gs[j].mid[f], sb(P, Q)), seed);
           gs[j].mid[f] = ad(gs[j].up[f], fm(w1, s0[j][f], fm(w2, gc[j][f], -out[j][f])));
           gs[j].up[f] = ad(P, Q);
           gs[j].ck[f] = cn[j][f];
@@ -771,11 +773,10 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
     if (!S && q > z1 + 1) return;
     // ---- links of plane q
     T Cd[RY][NF];
-    if (DI) qz = wrap(q - 1, nz) * plane;
     typedef std::integral_constant<int, RY> Rows;
     typedef std::integral_constant<int, 1> One;
-    if (S || (q >= z0 - 1 && q <= z1)) links(s_cur, k0, g, Cd, std::true_type(), Rows(), tx, ty);
-    else links(s_cur, k0, g, Cd, std::false_type(), Rows(), tx, ty);
+    if (S || (q >= z0 - 1 && q <= z1)) links(s_cur, k0, g, Cd, std::true_type(), Rows());
+    else links(s_cur, k0, g, Cd, std::false_type(), Rows());
     if (S || q >= z0) {
 #pragma unroll
       for (int f = 0; f < NF; f++)
@@ -785,7 +786,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
     }
     if (extra) {
       T Ce[1][NF];
-      links(s_cur, ke, ge, Ce, std::false_type(), One(), ci - 1, cj - 1);
+      links(s_cur, ke, ge, Ce, std::false_type(), One());
       if (S || q >= z0) {
 #pragma unroll
         for (int f = 0; f < NF; f++)
@@ -803,13 +804,13 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
   cp_async_wait<0>();  // no copy outlives the run
 }
 
-template <class T, int NF, int TY, int RY, int BPS, bool DI>
+template <class T, int NF, int TY, int RY, int BPS>
 __global__ void __launch_bounds__(M3_X *TY / RY, sizeof(T) == 8 ? 1 : BPS)
     mom_step3_kernel(const __grid_constant__ MomArgs<T> a, int zrun) {
   const int z0 = blockIdx.z * zrun;
   pdl_wait();
-  mom_run3<T, NF, TY, RY, DI>(a, blockIdx.x * M3_X, blockIdx.y * TY, z0, min(z0 + zrun, a.nz),
-                              a.step, zsm);
+  mom_run3<T, NF, TY, RY>(a, blockIdx.x * M3_X, blockIdx.y * TY, z0, min(z0 + zrun, a.nz),
+                              a.seed, zsm);
   pdl_next();
 }
 
@@ -843,7 +844,7 @@ struct M2Smem {
 
 template <class T, int TX, int TY, int STAGE>
 __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1, int x0, int y0,
-                                          unsigned char *sm) {
+                                          unsigned seed, unsigned char *sm) {
   using SM = M2Smem<T, TX, TY>;
   using L = Lat<0>;
   constexpr int NT = TX * TY, PER = (SM::NS + NT - 1) / NT, HX = SM::HX;
@@ -944,7 +945,7 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
     const Quad<T> p = Q1(k0);
     const T c = p.v[1];
     const T uu = fm(p.v[3], p.v[3], ml(p.v[2], p.v[2]));
-    const T out = fm(ml(T(1.5), c), uu, ml(T(1) - w0, p.v[0]));
+    const T out = ml(ml(T(1.5), c), uu);
     T ga, gb, fS, fX, fY;
     {
       const Quad<T> m = Q1(k0 - 1), q = Q1(k0 + 1);
@@ -980,6 +981,7 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
       const Duo<T> gm = Q2(k0 - 1 + HX), gq = Q2(k0 + 1 - HX);
       const T bm = mom_b(sb(m.v[2], m.v[3])), bp = mom_bn(sb(q.v[2], q.v[3]));
       gb = ad(gb, ad(fm(m.v[1], bm, m.v[0]), fm(q.v[1], bp, q.v[0])));
+      gb = fm(T(-mom_out<L>()), p.v[0], gb);
       const T fa = fm(a.rho, bm, ad(DP(k0 - 1 + HX), sb(gm.v[0], gm.v[1])));
       const T fb = fm(a.rho, bp, sb(DP(k0 + 1 - HX), sb(gq.v[0], gq.v[1])));
       sa = ad(sa, ad(fa, fb));
@@ -988,7 +990,7 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
       M[1] = fm(w1, fY, ml(w2, sb(da, db)));
     }
     S = fm(w1, fS, fm(w2, sa, ml(w0, DP(k0))));
-    C = ad(c, fm(w1, ga, fm(w2, gb, -out)));
+    C = mom_add(c, fm(w1, ga, fm(w2, gb, -out)), seed);
     cn[c0i] = C;
   }
   constexpr int NE = SM::NC - NT;
@@ -1006,7 +1008,7 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
     const Quad<T> p = Q1(k);
     const T c = p.v[1];
     const T uu = fm(p.v[3], p.v[3], ml(p.v[2], p.v[2]));
-    const T out = fm(ml(T(1.5), c), uu, ml(T(1) - w0, p.v[0]));
+    const T out = ml(ml(T(1.5), c), uu);
     Quad<T> m = Q1(k - 1), q = Q1(k + 1);
     T ga = ad(fm(m.v[1], mom_b(m.v[2]), m.v[0]), fm(q.v[1], mom_bn(q.v[2]), q.v[0]));
     m = Q1(k - HX);
@@ -1020,7 +1022,8 @@ __device__ __forceinline__ void mom_tile2(const MomArgs<T> &a, const Mom1<T> &m1
     q = Q1(k + 1 - HX);
     gb = ad(gb, ad(fm(m.v[1], mom_b(sb(m.v[2], m.v[3])), m.v[0]),
                    fm(q.v[1], mom_bn(sb(q.v[2], q.v[3])), q.v[0])));
-    cn[cj * SM::CX + ci] = ad(c, fm(w1, ga, fm(w2, gb, -out)));
+    gb = fm(T(-mom_out<L>()), p.v[0], gb);
+    cn[cj * SM::CX + ci] = mom_add(c, fm(w1, ga, fm(w2, gb, -out)), seed);
   }
   __syncthreads();
   if (!inside) return;
@@ -1103,7 +1106,7 @@ __global__ void __launch_bounds__(TX *TY)
     mom_step2_kernel(const __grid_constant__ MomArgs<T> a, const __grid_constant__ Mom1<T> m1) {
   pdl_next();
   pdl_wait();
-  mom_tile2<T, TX, TY, STAGE>(a, m1, blockIdx.x * TX, blockIdx.y * TY, zsm);
+  mom_tile2<T, TX, TY, STAGE>(a, m1, blockIdx.x * TX, blockIdx.y * TY, a.seed, zsm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1192,7 +1195,7 @@ __device__ __forceinline__ void mom_store(const MomBuf<T> &b, long long n, T A, 
 }
 
 // C of the next step at one node, from its neighbours' (A, C, u)
-template <int K, class T, int NF, bool DI>
+template <int K, class T, int NF>
 __global__ void __launch_bounds__(256)
     mom_c_kernel(const __grid_constant__ MomArgs<T> a, T *out, long long ostride) {
   using L = Lat<K>;
@@ -1204,7 +1207,7 @@ __global__ void __launch_bounds__(256)
   h.init(x, y, z, a.nx, a.ny, a.nz);
   h.guard(a.err);
   const int n = h.g(h.ox[1] + h.oy[1] + h.oz[1]);
-  T sa[NF], sd[NF], out0[NF], ck[NF];
+  T sa[NF], sd[NF], out0[NF], ak[NF], ck[NF];
 #pragma unroll
   for (int i = 0; i < L::Q; i++) {
     const int m = i == 0 ? n : h.minus<L>(i);
@@ -1222,7 +1225,8 @@ __global__ void __launch_bounds__(256)
       }
       if (i == 0) {
         ck[f] = C;
-        out0[f] = fm(ml(T(1.5), C), uu, ml(T(1.0 - L::w(0)), A));
+        out0[f] = ml(ml(T(1.5), C), uu);
+        ak[f] = A;
         sa[f] = sd[f] = T(0);
       } else if (L::w(i) == L::w(1)) {
         sa[f] = ad(sa[f], fm(C, b, A));
@@ -1233,9 +1237,9 @@ __global__ void __launch_bounds__(256)
   }
 #pragma unroll
   for (int f = 0; f < NF; f++) {
-    T d = fm(T(L::w(1)), sa[f], fm(T(L::w(L::Q - 1)), sd[f], -out0[f]));
-    if constexpr (DI) d = mom_dither(ck[f], d, n, a.step);
-    out[f * ostride + n] = ad(ck[f], d);
+    sd[f] = fm(T(-mom_out<L>()), ak[f], sd[f]);
+    const T d = fm(T(L::w(1)), sa[f], fm(T(L::w(L::Q - 1)), sd[f], -out0[f]));
+    out[f * ostride + n] = mom_add(ck[f], d, a.seed);
   }
 }
 
@@ -1526,8 +1530,9 @@ __global__ void __launch_bounds__(256)
     if (L::w(i) == L::w(1)) sa = ad(sa, g);
     else sd = ad(sd, g);
   }
-  const T o = fm(ml(T(1.5), q.v[1]), uu, ml(T(1.0 - L::w(0)), q.v[0]));
-  out[n] = ad(q.v[1], fm(T(L::w(1)), sa, fm(T(L::w(L::Q - 1)), sd, -o)));
+  sd = fm(T(-mom_out<L>()), q.v[0], sd);
+  const T d = fm(T(L::w(1)), sa, fm(T(L::w(L::Q - 1)), sd, -ml(ml(T(1.5), q.v[1]), uu)));
+  out[n] = mom_add(q.v[1], d, a.seed);
 }
 
 // canonical state planes: f (Q, storage type S), u (D), and A and C of each free
@@ -1680,7 +1685,7 @@ template <int K>
 constexpr int mom_batch_threads() {
   return K == 1 ? 128 : 256;
 }
-template <int K, class T, bool DI>
+template <int K, class T>
 __global__ void __launch_bounds__(mom_batch_threads<K>(), sizeof(T) == 8 ? 1 : 4)
     mom_batch_kernel(MomItem<T> *items, int nitems, const int *owner,
                      unsigned long long spin_limit) {
@@ -1704,10 +1709,10 @@ __global__ void __launch_bounds__(mom_batch_threads<K>(), sizeof(T) == 8 ? 1 : 4
       const int bx = b % meta[2], by = (b / meta[2]) % meta[3];
       if constexpr (K == 1) {
         const int z0 = b / (meta[2] * meta[3]) * meta[5];
-        mom_run3<T, 1, 8, 2, DI>(a, bx * M3_X, by * 8, z0, min(z0 + meta[5], a.nz),
-                                 a.step + (unsigned)t, zsm);
+        mom_run3<T, 1, 8, 2>(a, bx * M3_X, by * 8, z0, min(z0 + meta[5], a.nz),
+                             a.seed + MOM_SEED * (unsigned)t, zsm);
       } else {
-        mom_tile2<T, 32, 8, 2>(a, Mom1<T>{}, bx * 32, by * 8, zsm);
+        mom_tile2<T, 32, 8, 2>(a, Mom1<T>{}, bx * 32, by * 8, a.seed + MOM_SEED * (unsigned)t, zsm);
       }
       __syncthreads();  // the tile's shared memory is free
     }
@@ -1745,7 +1750,7 @@ MomArgs<T> mom_typed(const MomRaw &r) {
   a.rho = T(r.rho);
   a.irho = T(1.0 / r.rho);
   a.alpha_s = T(r.alpha_s);
-  a.step = r.step;
+  a.seed = MOM_SEED * r.step;
   return a;
 }
 
@@ -1755,9 +1760,9 @@ MomArgs<T> mom_typed(const MomRaw &r) {
 namespace {
 
 // The 3D step's launches for one set of template arguments.
-template <class T, int NF, int TY, int RY, int BPS, bool DI>
+template <class T, int NF, int TY, int RY, int BPS>
 struct Mom3 {
-  static constexpr auto kernel() { return mom_step3_kernel<T, NF, TY, RY, BPS, DI>; }
+  static constexpr auto kernel() { return mom_step3_kernel<T, NF, TY, RY, BPS>; }
   static bool prepare() {  // opt in to its dynamic shared memory, once
     static const bool ok =
         cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1816,8 +1821,7 @@ template <int K, class T, int NF = 1, class S = T>
 struct MomOps {
   // 3D: 32 x 8 tiles, two nodes per thread; blocks per SM by what the sums of
   // NF fluids leave of the registers (128, 168, 255 per thread)
-  static constexpr bool DI = Store<S>::k16;
-  using Step3 = Mom3<T, NF, 8, 2, (NF == 1 ? 4 : NF == 2 ? 3 : 2), DI>;
+  using Step3 = Mom3<T, NF, 8, 2, (NF == 1 ? 4 : NF == 2 ? 3 : 2)>;
   static cudaError_t step(const MomRaw &r, int zrun, cudaStream_t st) {
     if constexpr (K == 1) {
       return Step3::step(r, zrun, st);
@@ -1856,7 +1860,7 @@ struct MomOps {
     return cudaGetLastError();
   }
   static cudaError_t c_pass(const MomRaw &r, void *out, long long cstride, cudaStream_t st) {
-    mom_c_kernel<K, T, NF, DI><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0, st>>>(
+    mom_c_kernel<K, T, NF><<<lb_grid(K, r.nx, r.ny, r.nz), lb_block(K, r.nx, r.ny, r.nz), 0, st>>>(
         mom_typed<T>(r), (T *)out, cstride);
     return cudaGetLastError();
   }
@@ -1938,13 +1942,13 @@ struct MomOps {
   static cudaError_t batch(const MomBatchRaw *items, int n, void *scratch, size_t bytes,
                            unsigned long long spins, cudaStream_t st) {
     if (bytes < batch_bytes(n)) return cudaErrorInvalidValue;
-    static const bool ok = cudaFuncSetAttribute(mom_batch_kernel<K, T, DI>,
+    static const bool ok = cudaFuncSetAttribute(mom_batch_kernel<K, T>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)batch_smem()) == cudaSuccess;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!ok || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mom_batch_kernel<K, T, DI>,
+    if (!ok || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mom_batch_kernel<K, T>,
                                                              mom_batch_threads<K>(), batch_smem()) != cudaSuccess ||
         per_sm < 1)
       return cudaErrorInvalidValue;
@@ -2004,7 +2008,7 @@ struct MomOps {
       int cnt = m;
       unsigned long long lim = spins ? spins : kBarrierSpins;
       void *args[] = {(void *)&pi, (void *)&cnt, (void *)&po, (void *)&lim};
-      e = cudaLaunchCooperativeKernel((const void *)mom_batch_kernel<K, T, DI>,
+      e = cudaLaunchCooperativeKernel((const void *)mom_batch_kernel<K, T>,
                                       dim3((unsigned)owner.size()),
                                       dim3(32, mom_batch_threads<K>() / 32), args,
                                       batch_smem(), st);

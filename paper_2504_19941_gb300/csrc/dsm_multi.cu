@@ -684,6 +684,7 @@ struct dsm_mlattice {
   // Uz, pairs in Pz, quads (dP, G) in mq2; mcp, C[0] holds the C of its next step
   bool mok, mstat, mcp;
   int mc, mzrun;
+  long long msteps;  // taken since dsm_ml_set_fluids
   char *mq2[2], *msol, *mlk, *mnear, *mlist, *mwall;
   int *mcount;
 };
@@ -1071,6 +1072,7 @@ MomRaw mlm_raw(const dsm_mlattice *h, int src) {
   r.rho = h->rho[h->nf];
   for (int a = 0; a < 3; a++) r.body[a] = h->prm.body_force[a];
   r.alpha_s = h->prm.alpha_s > 0.0 ? h->prm.alpha_s : h->prm.alpha;
+  r.step = (unsigned)h->msteps;
   return r;
 }
 // dispatch over the free fluids
@@ -1086,6 +1088,7 @@ cudaError_t mlm_dispatch(const dsm_mlattice *h, Fn fn) {
 template <class T>
 cudaError_t mlm_init(dsm_mlattice *h) {
   h->mc = 0;
+  h->msteps = 0;
   h->mcp = false;
   return mlm_dispatch<T>(h, [&](auto k) {
     cudaError_t e = cudaSuccess;
@@ -1135,6 +1138,7 @@ cudaError_t mlm_step(dsm_mlattice *h) {
   }
   if (e == cudaSuccess) {
     h->mc ^= 1;
+    h->msteps++;
     h->mcp = false;
   }
   return e;
