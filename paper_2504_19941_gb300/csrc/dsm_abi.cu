@@ -382,13 +382,17 @@ cudaError_t t_step(dsm_lattice *h) {
 // 16-bit populations the moments are FP32 reals all the same: 36 B per node are
 // fewer than the 38 B of the populations and the 20 B of (A, C, u) that they
 // replace, and nothing is rounded to 16 bits any more.
-// Small FP64 lattices in 3D keep their populations: their runs of one plane form
-// four planes' sums for it on the FP64 pipe (16^3: 53 us per step in two passes, 87
-// on moments; 32^3: 86 and 84; 64^3: 351 and 272).
+// FP64 lattices in 3D, which the FP64 pipe bounds, keep their populations where a
+// run of planes has too much to sum beside its own nodes: small ones (16^3: 53 us per
+// step in two passes, 87 on moments; 32^3: 104 and 92; 64^3: 360 and 245), and those
+// narrower than a tile in x up to 80000 nodes (24 x 48 x 48 103 and 114, 31 x 64 x 64
+// 166 and 157) or in y (128 x 4 x 100 95 and 136, 300 x 5 x 100 229 and 241).
+bool m_f64_3d(const dsm_params *p) {
+  const long long n = (long long)p->nx * p->ny * p->nz;
+  return n >= 32768 && (z_tiles(p->nx, p->ny) || (n >= 80000 && p->ny >= 8));
+}
 bool m_eligible(const dsm_params *p) {
-  if (p->precision == DSM_F64 && p->lattice == DSM_D3Q19 &&
-      (long long)p->nx * p->ny * p->nz < 32768)
-    return false;
+  if (p->precision == DSM_F64 && p->lattice == DSM_D3Q19 && !m_f64_3d(p)) return false;
   const bool k16 = p->precision != DSM_F32 && p->precision != DSM_F64;
   return (!k16 || z_eligible(p)) && f64_tiles(p) && p->tau2 == 1.0 && p->tau3 == 1.0 && p->tau_g == 1.0 &&
          p->rho2 == p->rho3 && !has_walls(p);
@@ -509,8 +513,8 @@ int m_zrun(dsm_lattice *h) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int per_sm = h->tab.mom_resident();
-  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz,
-                      (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1));
+  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz, sms > 0 ? sms : 152, per_sm,
+                      h->prm.precision == DSM_F64);
   return h->mzrun;
 }
 

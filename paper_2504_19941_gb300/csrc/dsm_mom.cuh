@@ -1759,14 +1759,31 @@ MomArgs<T> mom_typed(const MomRaw &r) {
 // so that an attribute set once is set on the unit's own kernel.
 namespace {
 
+inline int mom_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 152;
+  }();
+  return sms;
+}
+// Dynamic shared memory of a launch of FP64 blocks no more than the SMs: so much that
+// no two share an SM (and its FP64 pipe) while others idle (48^3: 283 -> 157 us).
+template <class T>
+constexpr unsigned mom_spread(unsigned smem, long long blocks, int sms) {
+  return sizeof(T) == 8 && blocks <= sms && smem < 116u * 1024u ? 116u * 1024u : smem;
+}
+
 // The 3D step's launches for one set of template arguments.
 template <class T, int NF, int TY, int RY, int BPS>
 struct Mom3 {
   static constexpr auto kernel() { return mom_step3_kernel<T, NF, TY, RY, BPS>; }
+  static constexpr unsigned smem = M3Smem<T, NF, TY>::total;
   static bool prepare() {  // opt in to its dynamic shared memory, once
     static const bool ok =
         cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)M3Smem<T, NF, TY>::total) == cudaSuccess;
+                             (int)mom_spread<T>(smem, 0, 1)) == cudaSuccess;
     return ok;
   }
   static int resident() {
@@ -1784,9 +1801,9 @@ struct Mom3 {
     // start, the next launch's blocks took SM space from those still to run (51.1).
     const cudaError_t e = launch_pdl(mom_wall_kernel<T>, dim3(152 * 8), dim3(128), 0, st, a);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kernel(),
-                      dim3((r.nx + M3_X - 1) / M3_X, (r.ny + TY - 1) / TY, (r.nz + zrun - 1) / zrun),
-                      dim3(M3_X, TY / RY), M3Smem<T, NF, TY>::total, st, a, zrun);
+    const dim3 g((r.nx + M3_X - 1) / M3_X, (r.ny + TY - 1) / TY, (r.nz + zrun - 1) / zrun);
+    return launch_pdl(kernel(), g, dim3(M3_X, TY / RY),
+                      mom_spread<T>(smem, (long long)g.x * g.y * g.z, mom_sms()), st, a, zrun);
   }
 };
 
@@ -1795,14 +1812,18 @@ struct Mom3 {
 // than it advances (two of halo on each side, partly summed, and the first
 // copies).  101^3: 36.7 us with the 9 planes this gives, 42.4 / 37.5 / 43.2
 // with 6 / 13 / 17; 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96
-// (without the wall pass).
-inline int mom_zrun(int nx, int ny, int nz, long long resident) {
+// (without the wall pass).  FP64 blocks share their SM's FP64 pipe: two on an SM take
+// 1.85 times as long as one, which one block on each SM then beats with longer runs
+// (33 x 32 x 33 160 -> 115 us per step, 40^3 201 -> 136, 64^3 284 -> 245).
+inline int mom_zrun(int nx, int ny, int nz, int sms, int per_sm, bool f64) {
+  const long long resident = (long long)sms * (per_sm < 1 ? 1 : per_sm);
   const long long tiles = (long long)((nx + M3_X - 1) / M3_X) * ((ny + 7) / 8);
   double best = 1e300;
   int run = 1;
   for (int zr = 1; zr <= nz; zr++) {
     const long long blocks = tiles * ((nz + zr - 1) / zr);
-    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0);
+    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0) *
+                        (f64 && per_sm == 2 && blocks > sms ? 1.85 : 1.0);
     if (cost < best - 1e-9) {
       best = cost;
       run = zr;
@@ -1944,7 +1965,7 @@ struct MomOps {
     if (bytes < batch_bytes(n)) return cudaErrorInvalidValue;
     static const bool ok = cudaFuncSetAttribute(mom_batch_kernel<K, T>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)batch_smem()) == cudaSuccess;
+                                                (int)mom_spread<T>(batch_smem(), 0, 1)) == cudaSuccess;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1988,6 +2009,8 @@ struct MomOps {
           if (runs * tiles > nb && runs > 1) runs--;
           if (runs > nz) runs = nz;
           h.zrun = (nz + runs - 1) / runs;
+          if (m == 1 && sizeof(T) == 8)
+            h.zrun = mom_zrun(h.a[0].nx, h.a[0].ny, nz, sms, per_sm, true);
           h.runs = (nz + h.zrun - 1) / h.zrun;
         }
         const int tiles = h.tx * h.ty * h.runs;
@@ -2011,7 +2034,9 @@ struct MomOps {
       e = cudaLaunchCooperativeKernel((const void *)mom_batch_kernel<K, T>,
                                       dim3((unsigned)owner.size()),
                                       dim3(32, mom_batch_threads<K>() / 32), args,
-                                      batch_smem(), st);
+                                      K == 1 ? mom_spread<T>(batch_smem(), (long long)owner.size(), sms)
+                                             : batch_smem(),
+                                      st);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

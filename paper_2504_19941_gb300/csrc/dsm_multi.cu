@@ -1118,8 +1118,8 @@ int mlm_zrun(dsm_mlattice *h) {
     per_sm = k.resident();
     return cudaSuccess;
   });
-  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz,
-                      (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1));
+  h->mzrun = mom_zrun(h->prm.nx, h->prm.ny, h->prm.nz, sms > 0 ? sms : 152, per_sm,
+                      sizeof(T) == 8);
   return h->mzrun;
 }
 template <class T>

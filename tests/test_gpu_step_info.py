@@ -46,3 +46,31 @@ def test_step_info_is_the_form_that_runs(prec, shape, auto):
     fa, fg, ft = (x.populations()[0] for x in (lat, given, two))
     assert torch.equal(fa, fg if auto else ft)
     assert rel_err(fg.cpu().numpy(), ft.cpu().numpy()) < {"f64": 1e-13, "f32": 2e-6, "f16": 1e-3}[prec]
+
+
+def _form(lat):
+    """How the state is held: 1 f with g as g_eq, 2 moments, 3 f and quads."""
+    return int(lat.state()[:32].view(torch.int32)[7])
+
+
+def _plain(shape, prec, **kw):
+    sd = S.slab_sd(shape, len(shape) - 1, 0, 1)
+    case = S.Case("form", "D2Q9" if len(shape) == 2 else "D3Q19", shape, sd.ravel(),
+                  0.5 + S.perturbation(3, sd.size), theta_deg=90.0, g23=0.01, g12=0.01, alpha_s=1.0)
+    for k, v in kw.items():
+        setattr(case, k, v)
+    lat = gpu_lattice(case, prec)
+    lat.step(2)
+    return lat
+
+
+@pytest.mark.parametrize("shape,form,zrun", [
+    ((32, 32, 31), 1, None), ((32, 32, 32), 2, 1), ((33, 32, 33), 2, 2), ((40, 40, 40), 2, 3),
+    ((64, 64, 64), 2, 8), ((24, 48, 48), 1, 0), ((31, 64, 64), 2, 0), ((128, 4, 100), 1, 0),
+    ((300, 5, 100), 1, 0)])
+def test_fp64_in_3d_steps_on_moments_where_that_is_faster(shape, form, zrun):
+    # runs of planes: one block on each of 152 SMs, which share no FP64 pipe
+    lat = _plain(shape, "f64")
+    assert _form(lat) == form
+    if zrun is not None:
+        assert _lib.dsm_step_info(lat.h)[1] == zrun
