@@ -320,13 +320,35 @@ bool f64_tiles(const dsm_params *p) {
   const long long n = (long long)p->nx * p->ny;
   return n <= 2ll * 152 * 64 || n >= 2ll * 152 * 256;
 }
+// tiles of 16 x 4 nodes, which small FP64 lattices in 2D take
+long long small_tiles(const dsm_params *p) {
+  return ((p->nx + 15ll) / 16) * ((p->ny + 3ll) / 4);
+}
+// The same for the single pass over populations, whose halo costs more: up to 256
+// small tiles (tau contrast, 128 x 120, 240 tiles, 33.0 and 24.4 us per step; 160 x
+// 120, 300 tiles, 33.0 and 31.8, with mirrors and a density contrast 39.2 and 40.6;
+// 17 x 1100, 550 tiles, 37.3 and 44.4), and large ones with a density contrast
+// (512 x 400 185 and 153; without one 115 and 120).
+bool f64_quads(const dsm_params *p) {
+  if (p->precision != DSM_F64) return true;
+  return f64_tiles(p) &&
+         (small_tiles(p) <= 256 ||
+          (p->rho2 != p->rho3 && (long long)p->nx * p->ny >= 2ll * 152 * 256));
+}
+// And for the solid's relaxation, which has less to do per node: up to 360 small tiles
+// (40 x 480, 360 tiles, 21.2 and 13.2; 33 x 550, 414, 21.2 and 30.3) and from 90000
+// nodes up (340 x 240 48.0 and 51.1, 300 x 300 47.9 and 37.7).
+bool f64_relax(const dsm_params *p) {
+  if (p->precision != DSM_F64) return true;
+  return f64_tiles(p) && (small_tiles(p) <= 360 || (long long)p->nx * p->ny >= 90000);
+}
 
 // ---- single-pass step of D2Q9 ---------------------------------------------------
 // It applies with tau_g = 1 and faces that are periodic or mirrors (at a wall
 // g would bounce back, which no image node gives), in the automatic forms of g
 // and of the step, where the step on moments does not.
 bool t_eligible(const dsm_params *p) {
-  if (p->lattice != DSM_D2Q9 || p->tau_g != 1.0 || !f64_tiles(p)) return false;
+  if (p->lattice != DSM_D2Q9 || p->tau_g != 1.0 || !f64_quads(p)) return false;
   const int n[2] = {p->nx, p->ny};
   for (int a = 0; a < 2; a++) {
     const int lo = p->face[2 * a], hi = p->face[2 * a + 1];
@@ -521,7 +543,7 @@ int m_zrun(dsm_lattice *h) {
 // Whether dsm_relax_solid runs on moments: D2Q9 in FP32 or FP64, each axis
 // periodic, or a mirror on both sides (a wall's bounce-back has no image node).
 bool m_relax_of(const dsm_lattice *h, MomRelax *m) {
-  if (h->kind != DSM_D2Q9 || !h->tab.mom_relax || !f64_tiles(&h->prm)) return false;
+  if (h->kind != DSM_D2Q9 || !h->tab.mom_relax || !f64_relax(&h->prm)) return false;
   const int n[2] = {h->prm.nx, h->prm.ny};
   for (int a = 0; a < 2; a++) {
     const int lo = h->prm.face[2 * a], hi = h->prm.face[2 * a + 1];

@@ -74,3 +74,12 @@ def test_fp64_in_3d_steps_on_moments_where_that_is_faster(shape, form, zrun):
     assert _form(lat) == form
     if zrun is not None:
         assert _lib.dsm_step_info(lat.h)[1] == zrun
+
+
+@pytest.mark.parametrize("shape,contrast,form", [
+    ((128, 120), False, 3), ((160, 120), False, 1), ((17, 1100), True, 1), ((256, 128), True, 1),
+    ((512, 400), False, 1), ((512, 400), True, 3)])
+def test_fp64_in_2d_steps_from_quads_where_that_is_faster(shape, contrast, form):
+    kw = dict(tau3=0.6, **(dict(rho3=0.5) if contrast else {}))
+    assert _form(_plain(shape, "f64", **kw)) == form
+    assert _form(_plain(shape, "f32", **kw)) == 3
