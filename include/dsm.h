@@ -216,9 +216,7 @@ dsm_status dsm_set_body_force(dsm_lattice *h, const double *body);
  * collide.  Where every relaxation time is 1 and the densities are equal it marches
  * the moments that fix the populations instead, on lattices of any size; D2Q9
  * lattices with tau_g = 1 and periodic or mirror faces collide tile by tile in
- * one launch; and with a density contrast in FP32 arithmetic lattices of 180000
- * nodes and more run the two passes, the faster form there, unless zrun is given.
- * The results are the same step (the same per-node arithmetic, so
+ * one launch.  The results are the same step (the same per-node arithmetic, so
  * equal to the two-pass step up to nothing but FP32 contraction order); the
  * state then lives in padded buffers of the workspace and is converted back
  * before any call that reads it (fields, observables, populations, checkpoint,

@@ -245,6 +245,14 @@ bool z_maps(dsm_lattice *h) {
 // tiles * ceil(nz / zr) blocks, which run in waves of the resident blocks; a
 // wave lasts about zr planes plus the run's prologue (this step's C of two
 // extra planes and the first staged planes, about 0.7 of a plane).
+//
+// With a density contrast in FP32 arithmetic a node beside the solid takes a
+// multiple of another's time, and a lattice that is one wave of long runs waits for
+// the blocks that have most of them.  Runs of more than 12 planes become runs of 7,
+// which the SMs take as they come free.  us per step (before) over pillars and over a
+// flat wall: 250 x 130 x 101 210 (273) and 195 (211), 160 x 130 x 101 136 (186) and 128
+// (132), 128 x 128 x 101 115 (142) and 103 (99), 144^3 196 (231) and 187 (181).  Two
+// passes take 230 and 204, 151 and 134, 117 and 105, 214 and 191.
 int z_auto_run(dsm_lattice *h) {
   if (h->zrun_auto) return h->zrun_auto;
   int dev = 0, sms = 0;
@@ -264,25 +272,13 @@ int z_auto_run(dsm_lattice *h) {
       run = zr;
     }
   }
+  if (run > 12 && h->sp.rho_contrast && h->tab.real_bytes == 4) run = 7;
   h->zrun_auto = run;
   return run;
 }
 
-bool z_form(const dsm_lattice *h) {
-  return h->zok && h->eq && h->step_form == DSM_STEP_AUTO;
-}
-// In FP32 arithmetic with a density contrast two passes are the faster form of
-// the automatic step: rho at a node's 18 neighbours, each a quotient, leaves the
-// single pass out of issue slots with 24 warps per SM (250 x 130 x 101: 303 us per
-// step, 184 + 45 in two passes; rho planes formed once per node in shared memory
-// spilled, 378 us, and as a plane of the moments pass changed nothing, 181 + 52).
-// FP64, bound by its pipe, keeps the single pass, and so do lattices too small to
-// pay for a second launch (20 steps and two fields, single pass and two: 40 x 40 x 64
-// 552 and 587 us, 64^3 737 and 684, 120 x 100 x 80 2138 and 1898), and so does a
-// handle that is given its planes per block (dsm_set_step_form).
 bool z_active(const dsm_lattice *h) {
-  return z_form(h) &&
-         !(h->zrun == 0 && h->sp.rho_contrast && h->tab.real_bytes == 4 && h->N >= 180000);
+  return h->zok && h->eq && h->step_form == DSM_STEP_AUTO;
 }
 
 // Canonical g_eq state -> padded buffers (buffer 0), and padded C1.
@@ -1027,7 +1023,7 @@ dsm_status dsm_set_step_form(dsm_lattice *h, int form, int zrun) {
 
 dsm_status dsm_step_info(dsm_lattice *h, int *single_pass, int *zrun) {
   if (!h) return DSM_E_INVAL;
-  const bool single = m_active(h) ? z_form(h) : z_active(h);
+  const bool single = z_active(h);
   if (single_pass) *single_pass = single ? 1 : 0;
   if (zrun) *zrun = single ? (h->zrun > 0 ? h->zrun : m_active(h) ? m_zrun(h) : z_auto_run(h)) : 0;
   return DSM_OK;

@@ -1,7 +1,6 @@
 """dsm_step_info and Lattice.single_pass say which form dsm_step runs, and a
-given number of planes per block is taken: FP32 arithmetic with a density
-contrast on both sides of the 180000 nodes from which the automatic form runs
-two passes.  Which form ran shows in the end of the workspace: the padded copy of
+given number of planes per block is taken, also by large lattices with a density
+contrast.  Which form ran shows in the end of the workspace: the padded copy of
 C1, which only the one-pass step over populations writes.
 """
 import pytest
@@ -28,13 +27,15 @@ def _lattice(shape, prec, form="auto", zrun=0):
     return lat
 
 
-@pytest.mark.parametrize("prec,shape,auto", [("f32", (56, 56, 57), True), ("f32", (64, 64, 45), False),
-                                             ("f16", (64, 64, 45), False), ("f64", (64, 64, 45), True)])
-def test_step_info_is_the_form_that_runs(prec, shape, auto):
+@pytest.mark.parametrize("prec,shape,zauto", [
+    ("f32", (64, 64, 45), 2), ("f16", (64, 64, 45), 2), ("f64", (64, 64, 45), None),
+    ("f32", (160, 160, 100), 12), ("f32", (160, 130, 101), 7)])
+def test_step_info_is_the_form_that_runs(prec, shape, zauto):
+    # (zauto: on 152 SMs; runs of more than 12 planes become runs of 7)
     lat = _lattice(shape, prec)
     single, zrun = _lib.dsm_step_info(lat.h)
-    assert lat.single_pass == bool(single) == auto
-    assert (zrun > 0) == auto
+    assert lat.single_pass and single == 1 and zrun > 0
+    assert zauto is None or zrun == zauto
     given, two = _lattice(shape, prec, "auto", 7), _lattice(shape, prec, "two_pass")
     assert _lib.dsm_step_info(given.h) == (1, 7) and _lib.dsm_step_info(two.h) == (0, 0)
     ran = []
@@ -42,9 +43,9 @@ def test_step_info_is_the_form_that_runs(prec, shape, auto):
         x.workspace[-4 * x.n:].zero_()
         x.step(12)
         ran.append(bool(x.workspace[-4 * x.n:].any()))
-    assert ran == [auto, True, False]
+    assert ran == [True, True, False]
     fa, fg, ft = (x.populations()[0] for x in (lat, given, two))
-    assert torch.equal(fa, fg if auto else ft)
+    assert torch.equal(fa, fg)
     assert rel_err(fg.cpu().numpy(), ft.cpu().numpy()) < {"f64": 1e-13, "f32": 2e-6, "f16": 1e-3}[prec]
 
 
