@@ -1263,7 +1263,10 @@ dsm_status dsm_ml_create(const dsm_params *p, int nfluid, const double *kappa, c
     h->Pz[b] = w + L.Pz[b];
   }
   h->C1z = h->zok ? w + L.C1z : nullptr;
-  h->mok = h->zok;
+  // (four fluids in FP64 with at most one plane of a tile per SM: 32^3 144 us per step
+  // over populations, 160 on moments; 64 x 32 x 32 196 and 200, 33^3 290 and 236)
+  h->mok = h->zok && !(nfluid == 4 && rb == 8 &&
+                       (long long)z_tiles_x(p->nx) * z_tiles_y(p->ny) * p->nz <= 2 * 152);
   for (int f = 0; f < nfluid; f++) h->mok = h->mok && tau[f] == 1.0 && rho[f] == rho[0];
   for (int b = 0; b < 2; b++) h->mq2[b] = w + L.mq2[b];
   h->msol = w + L.msol;

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
+import paper_2504_19941_gb300 as P  # noqa: E402
 from paper_2504_19941_gb300 import _lib  # noqa: E402
 
 
@@ -84,3 +85,20 @@ def test_fp64_in_2d_steps_from_quads_where_that_is_faster(shape, contrast, form)
     kw = dict(tau3=0.6, **(dict(rho3=0.5) if contrast else {}))
     assert _form(_plain(shape, "f64", **kw)) == form
     assert _form(_plain(shape, "f32", **kw)) == 3
+
+
+@pytest.mark.parametrize("shape,nfluid,prec,moments", [
+    ((32, 32, 32), 4, "f64", False), ((40, 32, 40), 4, "f64", True), ((32, 32, 32), 3, "f64", True),
+    ((32, 32, 32), 4, "f32", True)])
+def test_four_fluids_in_fp64_step_on_moments_where_that_is_faster(shape, nfluid, prec, moments):
+    # the workspace starts with f_0 of the rest state, 1/3, where populations are kept
+    real = torch.float64 if prec == "f64" else torch.float32
+    n = shape[0] * shape[1] * shape[2]
+    p = P.make_params("D3Q19", shape, prec, theta_deg=90.0, alpha_s=1.0)
+    ml = P.MultiLattice(p, nfluid, (0.02,) * (nfluid + 1), (1.0,) * nfluid, (1.0,) * nfluid)
+    ml.set_solid_c1(torch.zeros(n, dtype=real, device="cuda"))
+    ml.set_fluids(torch.full((nfluid - 1, n), 0.2, dtype=real, device="cuda"))
+    f0 = ml.workspace[:n * (8 if prec == "f64" else 4)].view(real)
+    assert bool((f0 == torch.tensor(1 / 3, dtype=real)).all()) == (not moments)
+    ml.step(2)
+    assert float((ml.populations()[0].reshape(19, n)[0] - 1 / 3).abs().max()) < 1e-6
