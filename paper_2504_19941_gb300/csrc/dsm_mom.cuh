@@ -97,7 +97,8 @@ __device__ __forceinline__ T mom_bn(T v) {  // b(-v)
 //     their symmetries.
 //   - A leaves a node as 1 - w_0 and arrives as the weights, which in FP32 do not add
 //     up to it.  All of them are 2^k times the last one in any precision, so A leaves
-//     as mom_out (24 in 3D, 20 in 2D) times that weight.
+//     as mom_out (24 in 3D, 20 in 2D) times that weight (in FP64, where the difference
+//     is 1e-16 and a product more costs 1 %, as 1 - w_0 in the 3D step).
 // 256 x 256 x 192: 275 -> 284 us per step for both.
 template <class L>
 __host__ __device__ constexpr int mom_out() {
@@ -525,7 +526,9 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
             const T uu = fm(uz, uz, fm(p.uy, p.uy, ml(p.ux, p.ux)));
 #pragma unroll
             for (int f = 0; f < NF; f++) {
-              out[j][f] = fm(ml(T(1.5), p.C[f]), uu, ml(T(mom_out<Lat<1>>()), ml(w2, p.A[f])));
+              const T away = sizeof(T) == 8 ? ml(T(1) - w0, p.A[f])
+                                            : ml(T(mom_out<Lat<1>>()), ml(w2, p.A[f]));
+              out[j][f] = fm(ml(T(1.5), p.C[f]), uu, away);
               gP[j][f] = ml(w1, fm(p.C[f], h, p.A[f]));
               gR[j][f] = ml(w1, ml(p.C[f], z3));
               cn[j][f] = p.C[f];
@@ -1810,20 +1813,24 @@ struct Mom3 {
 // Planes per block of the 3D step: runs of zr planes give tiles * ceil(nz / zr)
 // blocks in waves of the resident ones; a run costs about three planes more
 // than it advances (two of halo on each side, partly summed, and the first
-// copies).  101^3: 36.7 us with the 9 planes this gives, 42.4 / 37.5 / 43.2
-// with 6 / 13 / 17; 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96
-// (without the wall pass).  FP64 blocks share their SM's FP64 pipe: two on an SM take
-// 1.85 times as long as one, which one block on each SM then beats with longer runs
-// (33 x 32 x 33 160 -> 115 us per step, 40^3 201 -> 136, 64^3 284 -> 245).
+// copies).  The blocks of an SM share its issue slots, in FP64 its FP64 pipe: a last
+// wave of k blocks per SM takes a + (1 - a) k / per_sm of a full one (FP64 0.54 and 1;
+// FP32, with the copies' latency, 0.55, 0.7, 0.85 and 1), so that a small lattice is
+// faster in few longer runs than in many short ones: 48^3 17.7 -> 15.3 us per step,
+// 64^3 20.5 -> 19.1; FP64 33 x 32 x 33 160 -> 115, 40^3 201 -> 136, 64^3 284 -> 245.
+// 101^3: 41.1 us with the 10 planes this gives, 45.2 / 44.7 / 45.9 with 6 / 12 / 16;
+// 256 x 256 x 192: 241 with 28, 251 with 20 or 32, 266 with 96 (without the wall pass).
 inline int mom_zrun(int nx, int ny, int nz, int sms, int per_sm, bool f64) {
-  const long long resident = (long long)sms * (per_sm < 1 ? 1 : per_sm);
+  if (per_sm < 1) per_sm = 1;
+  const long long resident = (long long)sms * per_sm;
   const long long tiles = (long long)((nx + M3_X - 1) / M3_X) * ((ny + 7) / 8);
+  const double a = f64 ? 0.08 : 0.4;
   double best = 1e300;
   int run = 1;
   for (int zr = 1; zr <= nz; zr++) {
-    const long long blocks = tiles * ((nz + zr - 1) / zr);
-    const double cost = (double)((blocks + resident - 1) / resident) * (zr + 3.0) *
-                        (f64 && per_sm == 2 && blocks > sms ? 1.85 : 1.0);
+    const long long blocks = tiles * ((nz + zr - 1) / zr), full = (blocks - 1) / resident;
+    const long long k = (blocks - full * resident + sms - 1) / sms;
+    const double cost = (full + a + (1.0 - a) * k / per_sm) * (zr + 3.0);
     if (cost < best - 1e-9) {
       best = cost;
       run = zr;

@@ -66,6 +66,13 @@ def _plain(shape, prec, **kw):
     return lat
 
 
+@pytest.mark.parametrize("shape,zrun", [((32, 32, 32), 1), ((48, 48, 48), 2), ((64, 64, 64), 4),
+                                        ((101, 101, 101), 10)])
+def test_fp32_runs_of_planes_on_moments(shape, zrun):
+    # on 152 SMs: one wave of blocks, fewer on each SM where that is faster
+    assert _lib.dsm_step_info(_plain(shape, "f32").h) == (1, zrun)
+
+
 @pytest.mark.parametrize("shape,form,zrun", [
     ((32, 32, 31), 1, None), ((32, 32, 32), 2, 1), ((33, 32, 33), 2, 2), ((40, 40, 40), 2, 3),
     ((64, 64, 64), 2, 8), ((24, 48, 48), 1, 0), ((31, 64, 64), 2, 0), ((128, 4, 100), 1, 0),
