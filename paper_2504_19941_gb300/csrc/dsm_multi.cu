@@ -692,8 +692,7 @@ struct dsm_mlattice {
 namespace {
 
 struct MLLayout {
-  size_t f[2], g[2], C[2], C1, M, err, Qz[2], Uz[2], Pz[2], C1z, mq2[2], msol, mlk, mnear, mlist,
-      mwall, total;
+  size_t f[2], g[2], C[2], C1, M, err, Qz[2], Uz[2], Pz[2], C1z, total;
 };
 
 // g held as g_eq: tau_g = 1 and every face periodic
@@ -730,15 +729,6 @@ MLLayout ml_layout(int q, int nf, int real_bytes, long long pitch, bool eq,
     L.Pz[b] = take(2 * (size_t)(nf - 1) * P * real_bytes);
   }
   L.C1z = take(P * real_bytes);
-  // and of the step on moments, per node: quads (dP, G) twice, the solid's
-  // pairs, link bits, a byte, a list entry, and the wall sums
-  const size_t n = z ? (size_t)pitch : 0;
-  for (int b = 0; b < 2; b++) L.mq2[b] = take(4 * n * real_bytes);
-  L.msol = take(2 * n * real_bytes);
-  L.mlk = take(4 * n);
-  L.mnear = take(n);
-  L.mlist = take(4 * n + 256);
-  L.mwall = take(4 * n * real_bytes);
   L.total = o;
   return L;
 }
@@ -1268,13 +1258,16 @@ dsm_status dsm_ml_create(const dsm_params *p, int nfluid, const double *kappa, c
   h->mok = h->zok && !(nfluid == 4 && rb == 8 &&
                        (long long)z_tiles_x(p->nx) * z_tiles_y(p->ny) * p->nz <= 2 * 152);
   for (int f = 0; f < nfluid; f++) h->mok = h->mok && tau[f] == 1.0 && rho[f] == rho[0];
-  for (int b = 0; b < 2; b++) h->mq2[b] = w + L.mq2[b];
-  h->msol = w + L.msol;
-  h->mlk = w + L.mlk;
-  h->mnear = w + L.mnear;
-  h->mcount = (int *)(w + L.mlist);
-  h->mlist = w + L.mlist + 256;
-  h->mwall = w + L.mwall;
+  // A lattice on moments keeps no populations: f[0] has the link fractions, and
+  // f[1] (19 planes of reals) the rest, 14 planes and 9 bytes per node.
+  const size_t plane = (size_t)pitch * rb;
+  for (int b = 0; b < 2; b++) h->mq2[b] = h->f[1] + 4 * b * plane;
+  h->msol = h->f[1] + 8 * plane;
+  h->mwall = h->f[1] + 10 * plane;
+  h->mlk = h->f[1] + 14 * plane;
+  h->mcount = (int *)(h->mlk + 4 * (size_t)pitch);
+  h->mlist = (char *)h->mcount + 256;
+  h->mnear = h->mlist + 4 * (size_t)pitch;
   // no solid until one is set: C1 = 0; no error latched
   if (cudaMemsetAsync(h->C1, 0, (size_t)pitch * rb, h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) != cudaSuccess) {
