@@ -336,6 +336,9 @@ __global__ void __launch_bounds__(256) lb_dir_kernel(long long n, int nv, const 
 // three squares, two sums, the solve) take 105; 193 MB of vectors, 28 us of copying.
 constexpr int LB_NV = 20, LB_NK = LB_NV + 3, LB_NT = 256;
 constexpr int LB_G = 4, LB_GV = LB_NV / LB_G;  // groups of threads, their vectors
+inline int lb_pair_grid(long long n) {  // dot_kernel's
+  return (int)std::min<long long>((n + LB_NT - 1) / LB_NT, VEC_BLOCKS);
+}
 struct LbPair {
   long long n;
   int m, hi, v0, cnt, nxt, last;
@@ -597,7 +600,7 @@ struct Minimiser {
     a.dots = dots;
     a.s = state;
     a.hi = hi = std::max(hi, nxt + 1);
-    const int grid = (int)std::min<long long>((n + LB_NT - 1) / LB_NT, VEC_BLOCKS);
+    const int grid = lb_pair_grid(n);
     for (int v = 0; v < 2 * hi; v += LB_NV) {
       a.v0 = v;
       a.cnt = std::min(LB_NV, 2 * hi - v);
@@ -842,7 +845,7 @@ static size_t lbfgs_layout_n(long long n, int m, size_t fe_bytes, size_t off[11]
   off[7] = take(sizeof(LbState));                 // the pair bookkeeping on the device
   off[8] = take(fe_bytes);
   off[9] = take(vec_scratch_bytes(n));
-  off[10] = take(256 + (size_t)VEC_BLOCKS * LB_NK * sizeof(double));
+  off[10] = take(256 + (size_t)lb_pair_grid(n) * LB_NK * sizeof(double));
   return o;
 }
 

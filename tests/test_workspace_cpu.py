@@ -14,3 +14,11 @@ from paper_2504_19941_gb300 import _lib
 def test_lattices_of_several_fluids(prec, shape, nfluid, nbytes):
     p = P.make_params("D3Q19", shape, prec, theta_deg=90.0)
     assert _lib.dsm_ml_workspace_bytes(p, nfluid) <= nbytes
+
+
+@pytest.mark.parametrize("shape,m,nbytes", [((16, 16, 16), 10, 423424), ((64, 64, 64), 10, 25408512),
+                                            ((128, 128, 128), 10, 201569280),
+                                            ((64, 64, 64), 20, 46574848)])
+def test_the_minimiser(shape, m, nbytes):
+    p = P.make_params("D3Q19", shape, "f32", theta_deg=90.0)
+    assert _lib.dsm_lbfgs_workspace_bytes(p, m) <= nbytes
