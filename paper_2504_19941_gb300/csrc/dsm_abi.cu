@@ -469,6 +469,15 @@ MomRaw m_raw(const dsm_lattice *h, int src) {
   return r;
 }
 
+// For kernels that collide only for a read: what they find non-finite is the next
+// step's, which may never come (another body force, another state), and goes to
+// the error words' second one, of which only bounds faults count.
+MomRaw m_read(const dsm_lattice *h, int src) {
+  MomRaw r = m_raw(h, src);
+  r.err = h->err + 1;
+  return r;
+}
+
 // canonical planes of buffer b
 MomPlanes m_planes(const dsm_lattice *h, int b) {
   const size_t plane = (size_t)h->pitch * h->tab.real_bytes;
@@ -589,18 +598,18 @@ bool m_peeks(const dsm_lattice *h) {
 cudaError_t m_peek(dsm_lattice *h) {
   if (h->mpk) return cudaSuccess;
   cudaError_t e = m_statics(h);
-  if (e == cudaSuccess) e = h->tab.mom_step(m_raw(h, h->mc), m_zrun(h), h->stream);
+  if (e == cudaSuccess) e = h->tab.mom_step(m_read(h, h->mc), m_zrun(h), h->stream);
   if (e == cudaSuccess) h->mpk = true;
   return e;
 }
 
 // Read and clear nothing: report the latched device error word.
 dsm_status read_err(dsm_lattice *h, int *word) {
-  int w = 0;
-  cudaError_t e = cudaMemcpyAsync(&w, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  int w[2] = {0, 0};
+  cudaError_t e = cudaMemcpyAsync(w, h->err, sizeof(w), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return DSM_E_CUDA;
-  *word = w;
+  *word = w[0] | (w[1] & ERR_BOUNDS);
   return DSM_OK;
 }
 
@@ -652,7 +661,7 @@ cudaError_t obs_launch(dsm_lattice *h) {
     e = m_statics(h);
     if (e == cudaSuccess) e = m_c(h);
     if (e == cudaSuccess)
-      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], 0, MODE_OBS, 0, 0, nullptr, h->partials,
+      e = h->tab.mom_node(m_read(h, h->mc), h->Cb[0], 0, MODE_OBS, 0, 0, nullptr, h->partials,
                           h->stream);
     if (e != cudaSuccess) return e;
     obs_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, h->obs_blocks, h->obs);
@@ -1124,7 +1133,7 @@ dsm_status dsm_get_field(dsm_lattice *h, int field, void *d_dst) {
     e = m_statics(h);
     if (e == cudaSuccess) e = m_c(h);
     if (e == cudaSuccess)
-      e = h->tab.mom_node(m_raw(h, h->mc), h->Cb[0], 0, MODE_FIELDS, field, 0, d_dst, nullptr,
+      e = h->tab.mom_node(m_read(h, h->mc), h->Cb[0], 0, MODE_FIELDS, field, 0, d_dst, nullptr,
                           h->stream);
     return cuda_status(e);
   }

@@ -668,7 +668,7 @@ struct dsm_mlattice {
   long long N, pitch;
   cudaStream_t stream;
   char *f[2], *g[2], *C[2], *C1, *M;  // C[cur]: C of the last collision; M: A_f and u
-  int *err;                            // latched error word in the workspace
+  int *err;  // latched error word in the workspace, and one for reads on moments
   int cur;
   bool eq;  // g held as g_eq (tau_g = 1, periodic faces)
   bool has_solid, has_fluid;
@@ -718,7 +718,7 @@ MLLayout ml_layout(int q, int nf, int real_bytes, long long pitch, bool eq,
   for (int b = 0; b < 2; b++) L.C[b] = take((size_t)nf * pitch * real_bytes);
   L.C1 = take((size_t)pitch * real_bytes);
   L.M = take(eq ? (size_t)(nf + 3) * pitch * real_bytes : 0);
-  L.err = take(sizeof(int));
+  L.err = take(2 * sizeof(int));
   // padded buffers of the single-pass step: per padded node a quad, u_z and
   // nf - 1 pairs (two buffers), and C1
   const bool z = p && ml_z_eligible(p);
@@ -1171,9 +1171,10 @@ cudaError_t ml_fields(dsm_mlattice *h, int field, int index, void *dst) {
   if (h->mok) {
     const cudaError_t e = mlm_c<T>(h);
     if (e != cudaSuccess) return e;
+    MomRaw r = mlm_raw(h, h->mc);
+    r.err = h->err + 1;  // (what a read finds non-finite is the next step's)
     return mlm_dispatch<T>(h, [&](auto k) {
-      return k.node(mlm_raw(h, h->mc), h->C[0], h->pitch, MODE_FIELDS, field, index, dst, nullptr,
-                    h->stream);
+      return k.node(r, h->C[0], h->pitch, MODE_FIELDS, field, index, dst, nullptr, h->stream);
     });
   }
   const cudaError_t eu = mlz_unpack<T>(h);
@@ -1270,7 +1271,7 @@ dsm_status dsm_ml_create(const dsm_params *p, int nfluid, const double *kappa, c
   h->mnear = h->mlist + 4 * (size_t)pitch;
   // no solid until one is set: C1 = 0; no error latched
   if (cudaMemsetAsync(h->C1, 0, (size_t)pitch * rb, h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) != cudaSuccess) {
+      cudaMemsetAsync(h->err, 0, 2 * sizeof(int), h->stream) != cudaSuccess) {
     delete h;
     return DSM_E_CUDA;
   }
@@ -1317,7 +1318,7 @@ dsm_status dsm_ml_set_fluids(dsm_mlattice *h, const void *d_c) {
   }
   h->cur = 0;
   h->zpacked = false;
-  if (cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) != cudaSuccess) return DSM_E_CUDA;
+  if (cudaMemsetAsync(h->err, 0, 2 * sizeof(int), h->stream) != cudaSuccess) return DSM_E_CUDA;
   cudaError_t e;
   if (h->mok) e = h->real_bytes == 8 ? mlm_init<double>(h) : mlm_init<float>(h);
   else if (h->real_bytes == 8) e = ml_dispatch<double, InitL>(h, ml_args<double>(h, 1));
@@ -1380,11 +1381,12 @@ dsm_status dsm_ml_get_populations(dsm_mlattice *h, void *d_f, void *d_g) {
 
 dsm_status dsm_ml_check(dsm_mlattice *h) {
   if (!h) return DSM_E_INVAL;
-  int word = 0;
-  if (cudaMemcpyAsync(&word, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream) !=
+  int w[2] = {0, 0};
+  if (cudaMemcpyAsync(w, h->err, sizeof(w), cudaMemcpyDeviceToHost, h->stream) !=
           cudaSuccess ||
       cudaStreamSynchronize(h->stream) != cudaSuccess)
     return DSM_E_CUDA;
+  const int word = w[0] | (w[1] & ERR_BOUNDS);
   if (word & ERR_TIMEOUT) return DSM_E_TIMEOUT;
   if (word & ERR_BOUNDS) return DSM_E_BOUNDS;
   return (word & ERR_NONFINITE) ? DSM_E_NONFINITE : DSM_OK;

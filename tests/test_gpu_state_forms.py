@@ -98,3 +98,21 @@ def test_a_state_at_rest_keeps_its_storage_form(shape):
     lat.step(2)
     other.step(2)
     assert other.g_implicit and _equal(lat, other)
+
+
+@pytest.mark.parametrize("shape,prec", [((33, 9, 5), "f32"), ((45, 13), "f32"), ((45, 13), "f64"),
+                                        ((40, 16, 8), "f16")])
+def test_a_read_does_not_latch_what_the_next_step_would_meet(shape, prec):
+    # a body force whose step overflows, read and taken back: the state is sound
+    lat, twin = gpu_lattice(_case(shape), prec), gpu_lattice(_case(shape), prec)
+    lat.step(3)
+    twin.step(3)
+    lat.set_body_force((1e200 if prec == "f64" else 1e30, 0.0, 0.0))
+    lat.field("pt")
+    assert float(lat.field("ux").abs().max()) > 1e20  # (its square overflows)
+    for x in (lat, twin):
+        x.set_body_force((1e-6, 0.0, 0.0))
+    assert lat.observables()["nonfinite"] == 0
+    lat.step(2)
+    twin.step(2)
+    assert lat.observables() == twin.observables() and _equal(lat, twin)
