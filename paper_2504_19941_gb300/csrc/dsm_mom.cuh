@@ -25,6 +25,7 @@
 // and the launch form (single or batched) cannot change it by a contraction.
 #pragma once
 
+#include <atomic>
 #include <type_traits>
 
 namespace dsm {
@@ -1771,6 +1772,19 @@ inline int mom_sms() {
   }();
   return sms;
 }
+// Opts a kernel in to its dynamic shared memory, once on each device (the attribute is
+// the device's; done: bit d for device d, devices beyond 63 every time).
+template <class... P>
+bool mom_opt_in(void (*kernel)(P...), int bytes, std::atomic<unsigned long long> &done) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_relaxed) & bit) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+    return false;
+  done.fetch_or(bit, std::memory_order_relaxed);
+  return true;
+}
 // Dynamic shared memory of a launch of FP64 blocks no more than the SMs: so much that
 // no two share an SM (and its FP64 pipe) while others idle (48^3: 283 -> 157 us).
 template <class T>
@@ -1783,11 +1797,9 @@ template <class T, int NF, int TY, int RY, int BPS>
 struct Mom3 {
   static constexpr auto kernel() { return mom_step3_kernel<T, NF, TY, RY, BPS>; }
   static constexpr unsigned smem = M3Smem<T, NF, TY>::total;
-  static bool prepare() {  // opt in to its dynamic shared memory, once
-    static const bool ok =
-        cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)mom_spread<T>(smem, 0, 1)) == cudaSuccess;
-    return ok;
+  static bool prepare() {
+    static std::atomic<unsigned long long> done{0};
+    return mom_opt_in(kernel(), (int)mom_spread<T>(smem, 0, 1), done);
   }
   static int resident() {
     int b = 0;
@@ -1970,9 +1982,8 @@ struct MomOps {
   static cudaError_t batch(const MomBatchRaw *items, int n, void *scratch, size_t bytes,
                            unsigned long long spins, cudaStream_t st) {
     if (bytes < batch_bytes(n)) return cudaErrorInvalidValue;
-    static const bool ok = cudaFuncSetAttribute(mom_batch_kernel<K, T>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)mom_spread<T>(batch_smem(), 0, 1)) == cudaSuccess;
+    static std::atomic<unsigned long long> done{0};
+    const bool ok = mom_opt_in(mom_batch_kernel<K, T>, (int)mom_spread<T>(batch_smem(), 0, 1), done);
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
