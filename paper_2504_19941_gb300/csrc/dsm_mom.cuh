@@ -373,21 +373,6 @@ struct M3Smem {
   static constexpr unsigned total = cring + 2 * NF * cplane;
 };
 
-// the links of the in-plane cross point on the -e (SG > 0) or +e side: values
-// for c_z = 0, +1, -1 (v, gv: u and G along e)
-template <int SG, class T, int NF>
-__device__ __forceinline__ void mom_cross_b(T v, T uz, T &b0, T &bp, T &bm) {
-  if (SG > 0) {
-    b0 = mom_b(v);
-    bp = mom_b(ad(v, uz));
-    bm = mom_b(sb(v, uz));
-  } else {
-    b0 = mom_bn(v);
-    bp = mom_b(sb(uz, v));
-    bm = mom_bn(ad(v, uz));
-  }
-}
-
 template <class T, int NF, int TY, int RY>
 __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, int z0, int z1,
                                          unsigned seed, unsigned char *sm) {
