@@ -422,9 +422,10 @@ def run_gpu(args, rank, world):
     step_achieved = (k2_b + k1_b) * n / (t_max / args.steps) / 1e9
     # the two secondary fractions of the measurement definitions: DRAM bytes
     # that ncu measured per lattice update, and B_min, one read and one write
-    # of f and g per node plus a read of C1 (a form that moves less, as the
-    # g_eq form does, is credited for the bytes it avoids)
-    b_min = lu_bytes(lattice, store, False)[0]  # the population form's fused-pass bytes
+    # of what fixes the state: the moments where every relaxation time is 1 and
+    # the densities are equal, else f and g per node and a read of C1 (a form that
+    # moves less, as the g_eq form does, is credited for the bytes it avoids)
+    b_min = lu_bytes_moments(store) if moments else lu_bytes(lattice, store, False)[0]
     lups_gpu = n * args.steps / t_max  # one GPU's lattice updates per second
 
     if rank == 0:
