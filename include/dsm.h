@@ -446,7 +446,10 @@ dsm_status dsm_vec_lincomb(long long n, int nv, const float *d_V, long long stri
  * returns when done.  The pair bookkeeping and the compact-form solve run on
  * the device; the host drives the line search and reads six doubles per trial
  * point (one read per iteration when the first trial is accepted).  At most 32
- * pairs (2m <= 64).  DSM_E_NONFINITE if the energy
+ * pairs (2m <= 64).  Every sum is taken in one fixed order, so that a run gives
+ * the same bits each time; iterates (not the converged point) depend on that
+ * order and differ from those of an L-BFGS that sums otherwise.
+ * DSM_E_NONFINITE if the energy
  * or gradient turns non-finite.  dsm_lbfgs_compact is the host-only
  * compact-form solve, exposed for tests: for k pairs (oldest first),
  * SY[i*k+j] = s_i.y_j, YY[i*k+j] = y_i.y_j, a = S^T g, b = Y^T g, it returns the
