@@ -404,7 +404,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
 #pragma unroll
     for (int r = 0; r < PER; r++) {
       if ((r + 1) * NT <= SM::NS || tid + r * NT < SM::NS) {
-        const int n = pzo + off[r];
+        const int n = chk(a.err, pzo + off[r], a.N);
         const unsigned d = sbase + slot + r * NT * (4 * sizeof(T));
         cp_async_bytes<4 * sizeof(T)>(d, reinterpret_cast<const Quad<T> *>(a.in.q1) + n);
         cp_async_bytes<4 * sizeof(T)>(d + SM::o2, reinterpret_cast<const Quad<T> *>(a.in.q2) + n);
@@ -717,7 +717,7 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
 #pragma unroll
         for (int j = 0; j < RY; j++) {
           if (x < nx && y + j < ny) {
-            const int n = nc + j * nx;
+            const int n = chk(a.err, nc + j * nx, a.N);
             T Sv = d2[j].S, M[3] = {d2[j].X, d2[j].Y, d2[j].Z};
             if (near[j]) {
               const Quad<T> w = reinterpret_cast<const Quad<T> *>(a.wall)[n];
@@ -733,20 +733,19 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
             r.v[1] = Cz[j][0];
             r.v[2] = o.u[0];
             r.v[3] = o.u[1];
-            const int m = chk(a.err, n, a.N);
-            reinterpret_cast<Quad<T> *>(a.out.q1)[m] = r;
+            reinterpret_cast<Quad<T> *>(a.out.q1)[n] = r;
             r.v[0] = o.dP;
             r.v[1] = o.G[0];
             r.v[2] = o.G[1];
             r.v[3] = o.G[2];
-            reinterpret_cast<Quad<T> *>(a.out.q2)[m] = r;
-            a.out.w[m] = o.u[2];
+            reinterpret_cast<Quad<T> *>(a.out.q2)[n] = r;
+            a.out.w[n] = o.u[2];
 #pragma unroll
             for (int e = 1; e < NF; e++) {
               Duo<T> p;
               p.v[0] = o.A[e];
               p.v[1] = Cz[j][e];
-              reinterpret_cast<Duo<T> *>(a.out.pe)[(e - 1) * a.N + m] = p;
+              reinterpret_cast<Duo<T> *>(a.out.pe)[(e - 1) * a.N + n] = p;
             }
           }
         }
@@ -757,8 +756,9 @@ __device__ __forceinline__ void mom_run3(const MomArgs<T> &a, int x0, int y0, in
         d2[j] = d1[j];
         // the solid's data of the node that collides next
         if (x < nx && y + j < ny && (S || (q >= z0 + 2 && q < z1 + 2))) {
-          solv[j] = reinterpret_cast<const Duo<T> *>(a.sol)[nc + j * nx];
-          near[j] = a.near[nc + j * nx];
+          const int n = chk(a.err, nc + j * nx, a.N);
+          solv[j] = reinterpret_cast<const Duo<T> *>(a.sol)[n];
+          near[j] = a.near[n];
         }
       }
     }
@@ -1141,7 +1141,7 @@ __global__ void __launch_bounds__(256) mom_solid_kernel(const __grid_constant__ 
   if (!lk) return;
   int k = n;
   if (K == 1) {
-    k = atomicAdd(a.count, 1);
+    k = chk(a.err, atomicAdd(a.count, 1), a.N);
     a.list[k] = n;
     const_cast<unsigned *>(a.lk)[k] = lk;
   }
