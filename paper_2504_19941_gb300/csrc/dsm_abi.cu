@@ -310,7 +310,8 @@ cudaError_t z_unpack(dsm_lattice *h) {
 // two passes over populations: the FP64 pipe is the bound there, and the halo of a
 // tile costs it more sums of C.  One launch against two passes, us per step:
 // 128 x 64 11.1 and 24.7, 160 x 121 22.1 and 26.7, 256 x 96 33.7 and 28.8 (34.9 with
-// tiles of 256), 256 x 128 42.3 and 32.9 (40.0), 512 x 512 87 and 140.
+// tiles of 256), 256 x 128 42.3 and 32.9 (40.0), 304 x 256 50 and 68, 400 x 320 53 and
+// 86, 512 x 512 87 and 140; ragged tiles, 19 x 1000, 28 and 37, 5 x 2000 28 and 49.
 bool f64_tiles(const dsm_params *p) {
   if (p->precision != DSM_F64 || p->lattice != DSM_D2Q9) return true;
   const long long n = (long long)p->nx * p->ny;
@@ -399,7 +400,9 @@ cudaError_t t_step(dsm_lattice *h) {
 // the solid's data goes.  dsm_set_step_form chooses one pass or two.  With
 // 16-bit populations the moments are FP32 reals all the same: 36 B per node are
 // fewer than the 38 B of the populations and the 20 B of (A, C, u) that they
-// replace, and nothing is rounded to 16 bits any more.
+// replace, and nothing is rounded to 16 bits any more.  FP32 lattices narrower than a
+// tile gain most, two launches for four (8^3 16.5 -> 9.6 us per step, 24^3 20.6 -> 10.8,
+// 31 x 100 x 100 28.9 -> 19.2, 1 x 1000 x 40 113 -> 54, 300 x 5 x 30 22.8 -> 15.2).
 // FP64 lattices in 3D, which the FP64 pipe bounds, keep their populations where a
 // run of planes has too much to sum beside its own nodes: small ones (16^3: 53 us per
 // step in two passes, 87 on moments; 32^3: 104 and 92; 64^3: 360 and 245), and those
