@@ -1798,6 +1798,7 @@ struct Mom3 {
   }
   static cudaError_t step(const MomRaw &r, int zrun, cudaStream_t st) {
     if (!prepare() || zrun < 1) return cudaErrorInvalidValue;
+    if (zrun > r.nz) zrun = r.nz;
     const MomArgs<T> a = mom_typed<T>(r);
     // Each lets the next launch in when its blocks are done (pdl_next at their end):
     // 101^3 46.3 -> 42.1 us per step, 256 x 256 x 192 279 -> 275.  Let in at their

@@ -109,3 +109,12 @@ def test_four_fluids_in_fp64_step_on_moments_where_that_is_faster(shape, nfluid,
     assert bool((f0 == torch.tensor(1 / 3, dtype=real)).all()) == (not moments)
     ml.step(2)
     assert float((ml.populations()[0].reshape(19, n)[0] - 1 / 3).abs().max()) < 1e-6
+
+
+@pytest.mark.parametrize("shape", [(20, 17, 13), (40, 16, 8)])
+def test_more_planes_per_block_than_the_lattice_has(shape):
+    lat, ref = _plain(shape, "f32"), _plain(shape, "f32")
+    lat.set_step_form("auto", 2**31 - 1)
+    lat.step(2)
+    ref.step(2)
+    assert all(torch.equal(a, b) for a, b in zip(lat.populations(), ref.populations()))
